@@ -263,7 +263,7 @@ def call_work_routed(wl, B):
     return {n: (b, o, b) for n, (b, o) in work.items()}
 
 
-def call_work(wl, B, fuse_dy1=False, through=False, bytes1=False, bits1=False):
+def call_work(wl, B, fuse_dy1=False, through=False, bytes1=False, bits1=False, codes1=False):
     """Algorithmic work of each library call of one step on a batch of B:
     (algorithmic bytes, algorithmic ops, bytes the call moves).
 
@@ -284,7 +284,13 @@ def call_work(wl, B, fuse_dy1=False, through=False, bytes1=False, bits1=False):
     table read) and the table gradient one add per (node, sample); both
     calls are then bounded by their bytes.  With wire bit rows (``bits1``)
     each wire takes one bit per sample (32-bit words, 32 per 1024-sample
-    block), written by the encoder and read by both layer-1 calls."""
+    block), written by the encoder and read by both layer-1 calls.
+
+    With corner codes (``codes1``) layer 1's output moves as one byte per
+    (node, sample) and a table per node instead of fp32 rows, and the layer-2
+    backward passes on 2^k corner sums per edge, which layer 1's table
+    gradient adds up; the bytes moved say so.  The algorithmic bytes and
+    operations stay those of the step's definition above."""
     K, k = wl.K, wl.k
     w1, w2 = wl.widths
     win, d, C = wl.w_in, wl.d, wl.classes
@@ -340,6 +346,13 @@ def call_work(wl, B, fuse_dy1=False, through=False, bytes1=False, bits1=False):
         work["backward1"] = (xin + f * (w1 * B + 2 * w1 * K + w1 * k) + csr2, dth1_ops,
                              xin + f * (2 * w1 * K + w1 * k) + csr2 + terms)
         del work["csr2"]
+    if codes1:
+        coded = w1 * (128 * ((B + 127) // 128)) + f * w1 * K      # codes and tables of layer 1
+        corners = f * w2 * k * K                                  # corner sums per edge
+        move = {"forward1": xw1 + coded + f * (w1 * K + w1 * k), "forward2": coded + f * (w2 * B + w2 * K + w2 * k),
+                "backward2": coded + f * (C * B + 2 * w2 * K + w2 * k) + corners,
+                "backward1": corners + f * (2 * w1 * K + w1 + 1)}
+        work.update({n: (work[n][0], work[n][1], m) for n, m in move.items()})
     return {n: (b, o, b if m is None else m) for n, (b, o, m) in work.items()}
 
 
@@ -400,6 +413,10 @@ TRAFFIC = {
 }
 
 
+# kernels of the corner-code route (lut_codes.cu)
+CODED_KERNELS = ("codes_forward", "coded_forward", "coded_backward", "corner_reduce")
+
+
 def code_digest(path: str) -> str:
     """SHA-256 of a C++/CUDA source with its comments and blank space
     removed, so that edits of the comments keep a capture valid."""
@@ -411,11 +428,14 @@ def code_digest(path: str) -> str:
     return hashlib.sha256(src.encode()).hexdigest()
 
 
-def kernel_traffic(workload: str, call: str):
-    """(bytes per launch, note) when the capture matches the current source, else (None, why)."""
+def kernel_traffic(workload: str, call: str, kernel: str = ""):
+    """(bytes per launch, note) when the capture matches the current source
+    and, where ``kernel`` names the step's kernel, that kernel; else (None, why)."""
     t = TRAFFIC.get((workload, call))
     if t is None:
         return None, "no capture for this workload"
+    if (kernel.startswith(CODED_KERNELS)) != (t["source"] == "lut_codes.cu"):
+        return None, "the capture is of another route's kernel"
     path = os.path.join(ROOT, "paper_2602_07400_gb300", "csrc", t["source"])
     try:
         digest = code_digest(path)
@@ -449,10 +469,14 @@ def route_of_step(st) -> dict:
         grad = "layer 2's per-edge terms summed in the layer-1 kernel"
     else:
         grad = "CSR reduction of layer 2's per-edge terms"
+    if getattr(st, "codes1", False):
+        grad = "corner sums per edge from the layer-2 backward, added up in the layer-1 kernel"
     wires = ("bytes: lookup forward, one-hot table gradient" if getattr(st, "bytes1", False)
              else "fp32: lerp-tree forward, multilinear table gradient")
     if getattr(st, "bits1", False):
         wires = "bits (one per sample): lookup forward, one-hot table gradient"
+    if getattr(st, "codes1", False):
+        wires = "bits (one per sample); layer 1's output as corner codes (a byte per sample) and tables"
     return {"layer1_wires": wires, "layer1_output_gradient": grad}
 
 
@@ -477,6 +501,9 @@ def kernels_of_step(st) -> dict:
                               else f"lut_theta_bytes_kernel<k, dY rows, {src}> (one-hot)")
     elif fused:
         names["backward1"] = "lut_backward_node_kernel<k, 0, terms>"
+    if getattr(st, "codes1", False):
+        names.update(forward1="codes_forward_kernel<k>", forward2="coded_forward_kernel<k>",
+                     backward2="coded_backward_kernel<k>", backward1="corner_reduce_kernel")
     return names
 
 
@@ -499,7 +526,7 @@ def roofline_of(call, work, per_call_ms, sms, clocks, workload, hbm, sm_max, pea
     else:
         roof = {"bound": "hbm", "achieved": byts / t_s / 1e9, "peak": hbm, "unit": "GB/s"}
     roof["frac"] = roof["achieved"] / roof["peak"]
-    traffic, traffic_note = kernel_traffic(workload, call)
+    traffic, traffic_note = kernel_traffic(workload, call, (kernels or KERNEL_OF_CALL)[call])
     roof.update({"traffic": traffic, "traffic_source": traffic_note,
                  "traffic_over_algorithmic": (traffic / byts) if traffic else None,
                  "kernel": (kernels or KERNEL_OF_CALL)[call], "call": call,
@@ -519,7 +546,7 @@ def calls_table(work, per_call_ms, hbm, workload=None, kernels=None):
              "Tops/s": round(o_ / (t * 1e-3) / 1e12, 2) if o_ else None}
         if m_ != b_:
             e["moved_GB/s"] = round(m_ / (t * 1e-3) / 1e9, 1)
-        traffic, _ = kernel_traffic(workload, n) if workload else (None, None)
+        traffic, _ = kernel_traffic(workload, n, (kernels or KERNEL_OF_CALL).get(n, "")) if workload else (None, None)
         if traffic:
             # DRAM bytes per launch from ncu against the algorithmic bytes,
             # and the DRAM rate they imply at the event-timed duration
@@ -699,7 +726,8 @@ def measure_train(wl, st, args, timer, hbm, sm_max, peak_kind, sms, world, detai
     work = call_work_routed(wl, B) if wl.Kc else call_work(wl, B, fuse_dy1=st.fuse_dy1,
                                                               through=getattr(st, "through", False),
                                                               bytes1=getattr(st, "bytes1", False),
-                                                              bits1=getattr(st, "bits1", False))
+                                                              bits1=getattr(st, "bits1", False),
+                                                              codes1=getattr(st, "codes1", False))
     single = {n: t for n, t in per_call.items() if n not in MULTI_KERNEL_CALLS}
     dom = max(single, key=single.get)
     res = {

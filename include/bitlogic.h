@@ -374,6 +374,61 @@ int bitlogic_lut_backward_bitrows(const uint32_t* X, int32_t w_in, int64_t B, co
                                   const int32_t* order, float* dtheta, float* dY_out,
                                   cudaStream_t stream);
 
+/* Layer 2 on corner codes of layer 1.  A layer on binary wires returns, per
+ * node and sample, the table entry its wires select (bitlogic_lut_forward_u8),
+ * so its output is given by the entry's index a (one byte) and the node's
+ * table.  These calls pass that form between the two layers instead of fp32
+ * rows, and the input gradient in the form the first layer's table gradient
+ * needs: per edge, the sum of the edge's terms over the samples on each
+ * corner of the input node.
+ *
+ *   codes  device uint8 [w1][S], S = 128 * ceil(B / 128): byte s of row i is
+ *          4 a_i(s), the byte offset of the selected entry; 0 for s >= B.
+ *          4-byte aligned.  Readers take a code modulo 4 * 2^k1 and rounded
+ *          down to a multiple of 4.
+ *   table  device fp32 [w1][2^k1]: t_i[a] = sigmoid(theta) or [theta > 0]
+ *          (the node form), 16-byte aligned for the layer-2 calls.
+ *
+ * bitlogic_lut_forward_codes: layer 1 on wire bit rows (as
+ *   bitlogic_lut_forward_bitrows), writing codes and table.  Any B.
+ * bitlogic_codes_decode: Y[i][s] = t_i[a_i(s)], device fp32 [w][B]: the rows
+ *   bitlogic_lut_forward_bitrows writes, bit for bit.
+ * bitlogic_lut_forward_coded: layer 2's forward (as bitlogic_lut_forward_node
+ *   on the decoded rows, up to rounding), 4 <= k <= 6, 1 <= k_in <= 6 the
+ *   fan-in of layer 1, w_in its width.  Any B and alignment of Y.
+ * bitlogic_lut_backward_coded: dtheta as bitlogic_lut_backward_node on the
+ *   decoded rows, dY rows shared by dy_group nodes, and for edge e = j*k + i
+ *   with input node c = conn[j][i]
+ *     corner_sums[row][a] = sum over the samples s with a_c(s) = a of
+ *                           dY[j][s] * dy_j/dx_i(s),
+ *   row = edge_pos[e] or e (edge_pos NULL); device fp32 [w*k][2^k_in].  Every
+ *   sum is in a fixed order.
+ * bitlogic_corner_reduce: layer 1's table gradient
+ *     dtheta[j][a] = s_a (1 - s_a) * sum over p in [csr_off[j], csr_off[j+1])
+ *                    of corner_sums[csr_edge[p]][a], s = sigmoid(theta),
+ *   in increasing p (csr_edge NULL: rows in CSR order), k the fan-in of
+ *   layer 1, n_edges the number of rows.
+ * Out-of-range indices raise the device flag and read row 0 (an out-of-range
+ * edge_pos stores at the edge's own row; an out-of-range CSR entry adds
+ * nothing).  B == 0: the forwards are no-ops, the backward zeroes its
+ * outputs.  Return BITLOGIC_ERR_NULL, BITLOGIC_ERR_SHAPE, BITLOGIC_ERR_FANIN,
+ * BITLOGIC_ERR_NODE, BITLOGIC_ERR_ALIGN, BITLOGIC_ERR_CUDA. */
+int bitlogic_lut_forward_codes(const uint32_t* X, int32_t w_in, int64_t B, const int32_t* conn,
+                               const float* theta, int32_t w, int32_t k, int32_t node, uint8_t* codes,
+                               float* table, cudaStream_t stream);
+int bitlogic_codes_decode(const uint8_t* codes, const float* table, int32_t w, int32_t k, int64_t B, float* Y,
+                          cudaStream_t stream);
+int bitlogic_lut_forward_coded(const uint8_t* codes, const float* table, int32_t w_in, int32_t k_in, int64_t B,
+                               const int32_t* conn, const float* theta, int32_t w, int32_t k, int32_t node,
+                               float* Y, cudaStream_t stream);
+int bitlogic_lut_backward_coded(const uint8_t* codes, const float* table, int32_t w_in, int32_t k_in, int64_t B,
+                                const int32_t* conn, const float* theta, int32_t w, int32_t k, int32_t node,
+                                const float* dY, int32_t dy_group, float* dtheta, float* corner_sums,
+                                const int32_t* edge_pos, cudaStream_t stream);
+int bitlogic_corner_reduce(const float* corner_sums, const int32_t* csr_off, const int32_t* csr_edge,
+                           int32_t n_edges, const float* theta, int32_t w, int32_t k, float* dtheta,
+                           cudaStream_t stream);
+
 /* Learnable routing (§3, the paragraph on connectivity: a per-slot
  * candidate pool whose selection is differentiable in training and snapped
  * to a sparse mapping at discretization; App. A "Initialization": pools

@@ -30,6 +30,8 @@ __all__ = [
     "bitlogic_head_loss_workspace", "bitlogic_head_loss_noalloc", "bitlogic_lut_backward_through", "bitlogic_lut_backward_through_u8",
     "bitlogic_lut_backward_u8", "bitlogic_lut_forward_u8", "bitlogic_encode_thermometer_bitrows",
     "bitlogic_lut_forward_bitrows", "bitlogic_lut_backward_bitrows", "bitrow_words",
+    "bitlogic_lut_forward_codes", "bitlogic_codes_decode", "bitlogic_lut_forward_coded",
+    "bitlogic_lut_backward_coded", "bitlogic_corner_reduce", "code_bytes",
     "bitlogic_head_loss", "bitlogic_binarize_tables", "bitlogic_pack_bits",
     "bitlogic_hard_forward", "bitlogic_build_csr", "bitlogic_csr_positions", "bitlogic_degree_order",
     "bitlogic_device_error",
@@ -87,6 +89,12 @@ _SIGS = {
     "bitlogic_lut_backward_bitrows": ([_P, _I32, _I64, _P, _P, _I32, _I32, _I32, _P, _I32, _P, _P, _P, _I32, _P,
                                        _P, _P, _P], ctypes.c_int),
     "bitlogic_degree_order": ([_P, _I32, _P], ctypes.c_int),
+    "bitlogic_lut_forward_codes": ([_P, _I32, _I64, _P, _P, _I32, _I32, _I32, _P, _P, _P], ctypes.c_int),
+    "bitlogic_codes_decode": ([_P, _P, _I32, _I32, _I64, _P, _P], ctypes.c_int),
+    "bitlogic_lut_forward_coded": ([_P, _P, _I32, _I32, _I64, _P, _P, _I32, _I32, _I32, _P, _P], ctypes.c_int),
+    "bitlogic_lut_backward_coded": ([_P, _P, _I32, _I32, _I64, _P, _P, _I32, _I32, _I32, _P, _I32, _P, _P, _P, _P],
+                                    ctypes.c_int),
+    "bitlogic_corner_reduce": ([_P, _P, _P, _I32, _P, _I32, _I32, _P, _P], ctypes.c_int),
     "bitlogic_lut_backward_workspace": ([_I32, _I64, _I32, _I32, _I32], _SZ),
     "bitlogic_lut_backward": ([_P, _I32, _I64, _P, _P, _I32, _I32, _P, _P, _P, _P, _P,
                                _P, _SZ, _P], ctypes.c_int),
@@ -645,6 +653,97 @@ def bitlogic_lut_backward_bitrows(X: torch.Tensor, B: int, conn: torch.Tensor, t
     _check("bitlogic_lut_backward_bitrows", load().bitlogic_lut_backward_bitrows(
         _ptr(X), w_in, B, _ptr(conn), _ptr(theta), w, k, _node_code(node), _ptr(dY), int(dy_group),
         _ptr(up_terms), _ptr(up_off), _ptr(up_edge), n_up, _ptr(order), _ptr(dtheta), _ptr(dY_out),
+        _stream(stream)))
+
+
+def code_bytes(B: int) -> int:
+    """Bytes per corner-code row of a batch of B (whole 128-sample blocks)."""
+    return 128 * ((int(B) + 127) // 128)
+
+
+def bitlogic_lut_forward_codes(X: torch.Tensor, B: int, conn: torch.Tensor, theta: torch.Tensor,
+                               codes: torch.Tensor, table: torch.Tensor, node="soft", stream=None):
+    """Layer 1 on wire bit rows X [w_in, bitrow_words(B)] int32: corner codes
+    uint8 [w, code_bytes(B)] and node tables fp32 [w, 2^k]."""
+    w_in = X.shape[0]
+    w, k = conn.shape
+    _need(X, "X", torch.int32, (w_in, bitrow_words(B)))
+    _need(conn, "conn", torch.int32, (w, k))
+    _need(theta, "theta", torch.float32, (w, 1 << k))
+    _need(codes, "codes", torch.uint8, (w, code_bytes(B)))
+    _need(table, "table", torch.float32, (w, 1 << k))
+    _check("bitlogic_lut_forward_codes", load().bitlogic_lut_forward_codes(
+        _ptr(X), w_in, B, _ptr(conn), _ptr(theta), w, k, _node_code(node), _ptr(codes), _ptr(table), _stream(stream)))
+
+
+def _need_codes(codes: torch.Tensor, table: torch.Tensor, B: int) -> Tuple[int, int]:
+    w1, K1 = table.shape
+    _need(table, "table", torch.float32, (w1, K1))
+    _need(codes, "codes", torch.uint8, (w1, code_bytes(B)))
+    if K1 & (K1 - 1):
+        raise ValueError("table: 2^k entries per node expected")
+    return w1, K1.bit_length() - 1
+
+
+def bitlogic_codes_decode(codes: torch.Tensor, table: torch.Tensor, Y: torch.Tensor, stream=None):
+    """The fp32 rows Y [w, B] that codes and table stand for."""
+    B = Y.shape[1]
+    w, k = _need_codes(codes, table, B)
+    _need(Y, "Y", torch.float32, (w, B))
+    _check("bitlogic_codes_decode", load().bitlogic_codes_decode(
+        _ptr(codes), _ptr(table), w, k, B, _ptr(Y), _stream(stream)))
+
+
+def bitlogic_lut_forward_coded(codes: torch.Tensor, table: torch.Tensor, conn: torch.Tensor, theta: torch.Tensor,
+                               Y: torch.Tensor, node="soft", stream=None):
+    """Layer forward (fan-in 4..6) on corner codes and tables of the layer below."""
+    w, k = conn.shape
+    B = Y.shape[1]
+    w_in, k_in = _need_codes(codes, table, B)
+    _need(conn, "conn", torch.int32, (w, k))
+    _need(theta, "theta", torch.float32, (w, 1 << k))
+    _need(Y, "Y", torch.float32, (w, B))
+    _check("bitlogic_lut_forward_coded", load().bitlogic_lut_forward_coded(
+        _ptr(codes), _ptr(table), w_in, k_in, B, _ptr(conn), _ptr(theta), w, k, _node_code(node), _ptr(Y),
+        _stream(stream)))
+
+
+def bitlogic_lut_backward_coded(codes: torch.Tensor, table: torch.Tensor, B: int, conn: torch.Tensor,
+                                theta: torch.Tensor, dtheta: torch.Tensor, corner_sums: torch.Tensor,
+                                dY: torch.Tensor, dy_group: int = 1, node="soft",
+                                edge_pos: Optional[torch.Tensor] = None, stream=None):
+    """Layer backward (fan-in 4..6) on corner codes: dtheta, and per edge the
+    corner sums [w*k, 2^k_in] of its input-gradient terms."""
+    w, k = conn.shape
+    w_in, k_in = _need_codes(codes, table, B)
+    _need(conn, "conn", torch.int32, (w, k))
+    _need(theta, "theta", torch.float32, (w, 1 << k))
+    _need(dtheta, "dtheta", torch.float32, (w, 1 << k))
+    _need(corner_sums, "corner_sums", torch.float32, (w * k, 1 << k_in))
+    if w % dy_group != 0:
+        raise ValueError("dy_group must divide w")
+    _need(dY, "dY", torch.float32, (w // dy_group, B))
+    if edge_pos is not None:
+        _need(edge_pos, "edge_pos", torch.int32, (w * k,))
+    _check("bitlogic_lut_backward_coded", load().bitlogic_lut_backward_coded(
+        _ptr(codes), _ptr(table), w_in, k_in, B, _ptr(conn), _ptr(theta), w, k, _node_code(node), _ptr(dY),
+        int(dy_group), _ptr(dtheta), _ptr(corner_sums), _ptr(edge_pos), _stream(stream)))
+
+
+def bitlogic_corner_reduce(corner_sums: torch.Tensor, csr_off: torch.Tensor, csr_edge: Optional[torch.Tensor],
+                           theta: torch.Tensor, dtheta: torch.Tensor, stream=None):
+    """Table gradient of the layer below from the corner sums of its consumer
+    edges; csr_edge None: the rows are stored in CSR order."""
+    w, K = theta.shape
+    n = corner_sums.shape[0]
+    _need(corner_sums, "corner_sums", torch.float32, (n, K))
+    _need(csr_off, "csr_off", torch.int32, (w + 1,))
+    if csr_edge is not None:
+        _need(csr_edge, "csr_edge", torch.int32, (n,))
+    _need(theta, "theta", torch.float32, (w, K))
+    _need(dtheta, "dtheta", torch.float32, (w, K))
+    _check("bitlogic_corner_reduce", load().bitlogic_corner_reduce(
+        _ptr(corner_sums), _ptr(csr_off), _ptr(csr_edge), n, _ptr(theta), w, K.bit_length() - 1, _ptr(dtheta),
         _stream(stream)))
 
 

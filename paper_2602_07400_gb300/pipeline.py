@@ -25,7 +25,9 @@ from . import (NODE_FORMS, bitlogic_adamw_update, bitlogic_binarize_tables, bitl
                bitlogic_pack_bits, bitlogic_route_backward, bitlogic_route_backward_u8, bitlogic_route_forward,
                bitlogic_route_forward_u8, bitlogic_route_snap, bitlogic_encode_thermometer_u8,
                bitlogic_lut_forward_u8, bitlogic_encode_thermometer_bitrows, bitlogic_lut_forward_bitrows,
-               bitlogic_lut_backward_bitrows, bitrow_words, bitlogic_degree_order)
+               bitlogic_lut_backward_bitrows, bitrow_words, bitlogic_degree_order,
+               bitlogic_lut_forward_codes, bitlogic_lut_forward_coded, bitlogic_lut_backward_coded,
+               bitlogic_corner_reduce, bitlogic_codes_decode, code_bytes)
 
 
 def _nomark(name: str) -> None:
@@ -202,7 +204,16 @@ class TrainStep:
     bitlogic_encode_thermometer_bitrows writes them and the layer-1 kernels
     read those words (bitlogic_lut_forward_bitrows / _backward_bitrows) with
     the same results bit for bit; ``bits`` is then the int32 tensor of words
-    and ``wires()`` writes the wires out as bytes on demand.  Set
+    and ``wires()`` writes the wires out as bytes on demand.
+
+    With ``codes1`` (the default on wire bit rows when ``fuse_dy1`` is left to
+    the step and layer 2's fan-in is at least 4) layer 1's output is kept as
+    corner codes, a byte per node and sample, and node tables
+    (bitlogic_lut_forward_codes) in place of fp32 rows; layer 2 reads its
+    inputs from those, and its backward reduces each edge's terms to the
+    2^k1 corner sums that layer 1's table gradient adds up
+    (bitlogic_lut_backward_coded, bitlogic_corner_reduce), so no per-edge rows
+    are stored.  ``y1`` is then written out on demand.  Set
     ``keep_dy1`` to also write dY1 (e.g. to check it).  ``node`` picks the
     LightLUT form of both layers: "soft", or "st" (hard table samples in the
     forward, straight-through gradient to the logits)."""
@@ -211,7 +222,7 @@ class TrainStep:
                  tau: float, want_dx1: bool = False, keep_dy1: bool = False,
                  fuse_dy1: Optional[bool] = None, csr_order: bool = True, node: str = "soft",
                  through: Optional[bool] = None, bytes1: Optional[bool] = None,
-                 bits1: Optional[bool] = None, device="cuda"):
+                 bits1: Optional[bool] = None, device="cuda", codes1: Optional[bool] = None):
         dev = torch.device(device)
         if node not in NODE_FORMS:
             raise ValueError(f"node must be one of {sorted(NODE_FORMS)}")
@@ -227,6 +238,7 @@ class TrainStep:
         self.through = bool(through)
         if bytes1 is None:
             bytes1 = B % 4 == 0 and not want_dx1
+        terms_asked = fuse_dy1 is not None
         if fuse_dy1 is None:
             # on byte wires the layer-1 backward streams the terms itself
             # (faster than the CSR reduction at every measured shape); on fp32
@@ -235,7 +247,6 @@ class TrainStep:
         f32 = dict(dtype=torch.float32, device=dev)
         self.x = torch.zeros(B, d, dtype=torch.uint8, device=dev)
         self.labels = torch.zeros(B, dtype=torch.int32, device=dev)
-        self.y1 = torch.empty(net.w1, B, **f32)
         self.y2 = torch.empty(net.w2, B, **f32)
         self.logits = torch.empty(B, C, **f32)
         self.loss = torch.zeros(1, **f32)
@@ -249,6 +260,21 @@ class TrainStep:
         if bits1 and not (self.bytes1 and not self.through):
             raise ValueError("wire bit rows need byte wires for layer 1 and a route other than through")
         self.bits1 = bool(bits1)
+        may_code = self.bits1 and self.fuse_dy1 and csr_order and net.k2 >= 4
+        if codes1 is None:
+            codes1 = may_code and not terms_asked
+        if codes1 and not may_code:
+            raise ValueError("corner codes need wire bit rows, the fused route in CSR order and layer-2 fan-in >= 4")
+        self.codes1 = bool(codes1)
+        # layer 1's output: corner codes and node tables, or fp32 rows
+        if self.codes1:
+            self.codes = torch.empty(net.w1, code_bytes(B), dtype=torch.uint8, device=dev)
+            self.table1 = torch.empty_like(net.theta1)
+            self.corners2 = torch.empty(net.w2 * net.k2, 1 << net.k1, **f32)
+        if not self.codes1 or keep_dy1:
+            self._y1 = torch.empty(net.w1, B, **f32)
+        if self.codes1 and keep_dy1:
+            self._dth2_terms = torch.empty_like(net.theta2)
         # the encoder's output: wire bit rows (bits1), byte rows (bytes1) or
         # fp32 rows
         if self.bits1:
@@ -259,14 +285,27 @@ class TrainStep:
         # read without the edge map) instead of edge order
         self.csr_order = bool(csr_order)
         self.dy1 = torch.empty(net.w1, B, **f32) if (keep_dy1 or not (self.fuse_dy1 or self.through)) else None
+        # under codes1 nothing but dY1 itself needs the per-edge terms
+        need_terms = not self.through and not (self.codes1 and self.dy1 is None)
         self.dth1 = torch.empty_like(net.theta1)
         self.dth2 = torch.empty_like(net.theta2)
         self.dbits = torch.empty(net.w_in, B, **f32) if want_dx1 else None
         # per-edge input-gradient terms of layer 2 (and of layer 1 when its
         # input gradient is wanted)
-        self.edges2 = None if self.through else torch.empty(net.w2 * net.k2, B, **f32)
+        self.edges2 = torch.empty(net.w2 * net.k2, B, **f32) if need_terms else None
         self.edges1 = torch.empty(net.w1 * net.k1, B, **f32) if want_dx1 else None
         self.ws_head = torch.empty(bitlogic_head_loss_workspace(B, C), dtype=torch.uint8, device=dev)
+
+    @property
+    def y1(self) -> torch.Tensor:
+        """Layer 1's output [w1, B]: the buffer of the last forward, or under
+        ``codes1`` the last forward's codes and tables written out as fp32 rows
+        into a new tensor."""
+        if not self.codes1:
+            return self._y1
+        out = torch.empty(self.net.w1, self.B, dtype=torch.float32, device=self.codes.device)
+        bitlogic_codes_decode(self.codes, self.table1, out)
+        return out
 
     def load(self, x: torch.Tensor, labels: torch.Tensor, non_blocking: bool = False):
         self.x.copy_(x, non_blocking=non_blocking)
@@ -274,7 +313,11 @@ class TrainStep:
 
     def forward(self, stream=None, mark=_nomark):
         n = self.net
-        if self.bits1:
+        if self.codes1:
+            bitlogic_encode_thermometer_bitrows(self.x, self.thr, self.bits, stream)
+            mark("encode")
+            bitlogic_lut_forward_codes(self.bits, self.B, n.conn1, n.theta1, self.codes, self.table1, self.node, stream)
+        elif self.bits1:
             bitlogic_encode_thermometer_bitrows(self.x, self.thr, self.bits, stream)
             mark("encode")
             bitlogic_lut_forward_bitrows(self.bits, self.B, n.conn1, n.theta1, self.y1, self.node, stream)
@@ -287,7 +330,10 @@ class TrainStep:
             mark("encode")
             bitlogic_lut_forward_node(self.bits, n.conn1, n.theta1, self.y1, self.node, stream)
         mark("forward1")
-        bitlogic_lut_forward_node(self.y1, n.conn2, n.theta2, self.y2, self.node, stream)
+        if self.codes1:
+            bitlogic_lut_forward_coded(self.codes, self.table1, n.conn2, n.theta2, self.y2, self.node, stream)
+        else:
+            bitlogic_lut_forward_node(self.y1, n.conn2, n.theta2, self.y2, self.node, stream)
         mark("forward2")
         bitlogic_head_loss_ex(self.y2, self.labels, self.C, self.tau, self.loss, self.ws_head,
                               logits=self.logits, dY_grouped=self.dyg, stream=stream)
@@ -298,6 +344,19 @@ class TrainStep:
         co = self.csr_order
         nd = self.node
         g = n.w2 // self.C
+        if self.codes1:
+            bitlogic_lut_backward_coded(self.codes, self.table1, self.B, n.conn2, n.theta2, self.dth2, self.corners2,
+                                        self.dyg, g, nd, edge_pos=n.pos2, stream=stream)
+            mark("backward2")
+            bitlogic_corner_reduce(self.corners2, n.off2, None, n.theta1, self.dth1, stream)
+            mark("backward1")
+            if self.dy1 is not None:   # dY1 is kept: from the terms, as the other routes form it
+                bitlogic_codes_decode(self.codes, self.table1, self._y1, stream)
+                bitlogic_lut_backward_node(self._y1, n.conn2, n.theta2, self._dth2_terms, nd, dY=self.dyg, dy_group=g,
+                                           edge_terms=self.edges2, edge_pos=n.pos2, stream=stream)
+                bitlogic_csr_reduce(self.edges2, n.off2, None, self.dy1, stream)
+                mark("dy1")
+            return
         if self.through:
             # layer 2: table gradient only; layer 1: its output gradient
             # recomputed through layer 2 inside its table-gradient kernel
@@ -387,9 +446,12 @@ class TrainStep:
 
     # kernels one run() launches: encode 1, forwards 2, head 2, backwards 2
     # (+ the CSR reduction of layer 2's terms unless fused or recomputed, +
-    # the layer-1 CSR reduction when the input gradient is wanted)
+    # the layer-1 CSR reduction when the input gradient is wanted; on corner
+    # codes + decode, terms and CSR reduction when dY1 is kept)
     @property
     def kernels_per_run(self) -> int:
+        if self.codes1:
+            return 7 + (3 if self.dy1 is not None else 0)
         return 7 + (0 if (self.fuse_dy1 or self.through) else 1) + (1 if self.dbits is not None else 0)
 
 

@@ -1,0 +1,135 @@
+"""GPU parity of layer 2 on corner codes of layer 1: the codes and tables
+against the bit-row forward (bit for bit), the layer-2 forward and backward
+and the corner reduction against the oracle on the decoded rows, at the edges
+of the kernels' stages (64 and 128 samples), fan-ins and table sizes."""
+import os
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2602_07400_gb300 as bl
+from paper_2602_07400_gb300 import synth
+from parity_util import check_exact, check_fwd, check_grad
+from test_gpu_bitrows import dev, pack_rows
+
+pytestmark = pytest.mark.gpu
+
+oracle.set_threads(os.cpu_count() or 1)
+
+
+def _layer1(w_in, w1, k1, B, node, seed=0):
+    """Codes and table of a layer on random binary wires, and its fp32 rows."""
+    bits = synth.binary_activations(w_in, B, seed=seed + B)
+    conn = synth.connectivity(w1, k1, w_in, seed=seed + 1)
+    theta = synth.table_logits(w1, 1 << k1, seed=seed + 2)
+    X = dev(pack_rows(bits))
+    codes = torch.full((w1, bl.code_bytes(B)), 255, dtype=torch.uint8, device="cuda")
+    table = torch.empty(w1, 1 << k1, device="cuda")
+    bl.bitlogic_lut_forward_codes(X, B, dev(conn), dev(theta), codes, table, node)
+    Y = torch.empty(w1, B, device="cuda")
+    bl.bitlogic_lut_forward_bitrows(X, B, dev(conn), dev(theta), Y, node)
+    corner = (bits[conn].astype(np.int64) << np.arange(k1)[None, :, None]).sum(axis=1)
+    return codes, table, Y, corner, theta
+
+
+@pytest.mark.parametrize("k1,B,node", [(1, 5, "soft"), (2, 128, "st"), (3, 1024, "soft"), (4, 1027, "st"),
+                                       (5, 2049, "soft"), (6, 907, "soft"), (6, 1024, "st")])
+def test_codes_and_decode(k1, B, node):
+    codes, table, Y, corner, theta = _layer1(50, 37, k1, B, node)
+    got = codes.cpu().numpy()
+    check_exact(got[:, :B], (4 * corner).astype(np.uint8), "codes")
+    assert not got[:, B:].any()                       # padding
+    out = torch.full_like(Y, np.nan)
+    bl.bitlogic_codes_decode(codes, table, out)
+    check_exact(out.cpu().numpy(), Y.cpu().numpy(), "decoded rows vs bit-row forward")
+    assert bl.bitlogic_device_error() == 0
+
+
+# B: below a stage, at its edges, ragged and unaligned rows, several stages;
+# w: fewer and more nodes than one wave of the persistent warps
+SHAPES = [(6, 6, 40, 30, 1), (6, 6, 90, 60, 64), (6, 6, 120, 3000, 132), (6, 4, 300, 200, 1027), (6, 1, 60, 40, 907),
+          (5, 5, 80, 50, 63), (5, 6, 200, 4000, 200), (5, 2, 70, 36, 128), (4, 4, 100, 3000, 65), (4, 6, 64, 40, 1000),
+          (4, 3, 50, 24, 37), (6, 5, 100, 80, 2048)]
+
+
+@pytest.mark.parametrize("k,k1,w1,w,B", SHAPES)
+@pytest.mark.parametrize("node", ["soft", "st"])
+def test_layer2_on_codes(k, k1, w1, w, B, node):
+    codes, table, Y1, corner, theta1 = _layer1(64, w1, k1, B, node)
+    conn = synth.connectivity(w, k, w1, seed=11)
+    theta = synth.table_logits(w, 1 << k, seed=12)
+    X = Y1.cpu().numpy().astype(np.float64)
+    Y = torch.full((w, B), np.nan, device="cuda")
+    bl.bitlogic_lut_forward_coded(codes, table, dev(conn), dev(theta), Y, node)
+    want = oracle.lut_forward(X, conn, theta, node)
+    if node == "st":
+        check_exact(Y.cpu().numpy().astype(np.float64), want, "y (binary inputs)")
+    else:
+        check_fwd(Y, want, "y")
+    # the fp32-row forward evaluates the same expressions
+    Yr = torch.empty_like(Y)
+    if B % 4 == 0:
+        bl.bitlogic_lut_forward_node(Y1, dev(conn), dev(theta), Yr, node)
+        check_exact(Y.cpu().numpy(), Yr.cpu().numpy(), "y vs fp32 rows")
+    group = 2
+    dYg = synth.uniform_gradients(w // group, B, seed=13, scale=1e-2)
+    off, edge = bl.bitlogic_build_csr(conn, w1)
+    pos = bl.bitlogic_csr_positions(edge)
+    dth = torch.full((w, 1 << k), np.nan, device="cuda")
+    H = torch.full((w * k, 1 << k1), np.nan, device="cuda")
+    bl.bitlogic_lut_backward_coded(codes, table, B, dev(conn), dev(theta), dth, H, dev(dYg), group, node)
+    Hp = torch.full_like(H, np.nan)
+    dth_p = torch.empty_like(dth)
+    bl.bitlogic_lut_backward_coded(codes, table, B, dev(conn), dev(theta), dth_p, Hp, dev(dYg), group, node,
+                                   edge_pos=dev(pos))
+    check_exact(dth_p.cpu().numpy(), dth.cpu().numpy(), "dtheta with positions (and run to run)")
+    check_exact(Hp.cpu().numpy(), H.cpu().numpy()[edge], "corner sums at CSR positions")
+    dY = np.repeat(dYg.astype(np.float64), group, axis=0)
+    wth, wdx = oracle.lut_backward(X, conn, theta, dY, want_dx=True, node=node)
+    check_grad(dth, wth, "dtheta")
+    # corner sums of an edge add up to the edge's terms: their totals per input
+    # node and corner are those of the input gradient
+    tot = np.zeros((w1, 1 << k1))
+    np.add.at(tot, conn.reshape(-1), H.cpu().numpy().astype(np.float64))
+    want_tot = np.zeros((w1, 1 << k1))
+    for a in range(1 << k1):
+        want_tot[:, a] = np.where(corner == a, wdx, 0.0).sum(axis=1)
+    check_grad(tot, want_tot, "corner sums")
+    d1 = torch.full((w1, 1 << k1), np.nan, device="cuda")
+    bl.bitlogic_corner_reduce(Hp, dev(off), None, dev(theta1), d1)
+    d1e = torch.empty_like(d1)
+    bl.bitlogic_corner_reduce(H, dev(off), dev(edge), dev(theta1), d1e)
+    check_exact(d1e.cpu().numpy(), d1.cpu().numpy(), "corner reduction with an edge map")
+    s = 1.0 / (1.0 + np.exp(-theta1.astype(np.float64)))
+    check_grad(d1, s * (1 - s) * want_tot, "layer-1 dtheta")
+    assert bl.bitlogic_device_error() == 0
+
+
+def test_out_of_range_indices_are_flagged():
+    codes, table, Y1, corner, theta1 = _layer1(64, 40, 4, 100, "soft")
+    conn = synth.connectivity(20, 4, 40, seed=3)
+    theta = dev(synth.table_logits(20, 16, seed=4))
+    bad = conn.copy()
+    bad[3, 1] = 40
+    bad[7, 0] = -1
+    zero = conn.copy()
+    zero[3, 1] = zero[7, 0] = 0
+    outs = []
+    for c in (bad, zero):
+        Y, dth = torch.empty(20, 100, device="cuda"), torch.empty(20, 16, device="cuda")
+        H = torch.empty(80, 16, device="cuda")
+        bl.bitlogic_lut_forward_coded(codes, table, dev(c), theta, Y)
+        bl.bitlogic_lut_backward_coded(codes, table, 100, dev(c), theta, dth, H, Y)
+        outs.append((Y.cpu().numpy(), dth.cpu().numpy(), H.cpu().numpy()))
+        assert bl.bitlogic_device_error() == (-8 if c is bad else 0)
+    for a, b in zip(*outs):
+        check_exact(a, b, "row 0 in place of an index out of range")
+    # codes beyond the table are taken modulo its size
+    wild = codes.clone()
+    wild |= 0xC3
+    Y, Yw = torch.empty(20, 100, device="cuda"), torch.empty(20, 100, device="cuda")
+    bl.bitlogic_lut_forward_coded(codes, table, dev(conn), theta, Y)
+    bl.bitlogic_lut_forward_coded(wild, table, dev(conn), theta, Yw)
+    check_exact(Yw.cpu().numpy(), Y.cpu().numpy(), "code bits outside the table")
