@@ -189,51 +189,76 @@ hard_layer_kernel(const uint32_t* __restrict__ xp, int w_in, long long W,
     }
 }
 
-// ------------------------------------------- staged layer (vector path) --
+// ---------------------------------------------------------- staged layer --
 //
-// The vector paths (W % 4 == 0, 16-byte aligned rows) stream the gathered
-// input words through a per-warp ring of shared-memory stages filled by
-// 16-byte cp.async copies; a stage holds the k input rows of one node over
-// 128 words.  Lane l copies, and later reads, only words 4l .. 4l + 3 of each
-// row, so the ring is lane-private: a lane waits for its own copies
-// (cp.async.wait_group) and no warp synchronisation guards the ring.  The
-// ring runs across node boundaries, so the copies of the next node are in
-// flight while the current node is evaluated, and the connectivity row and
-// table of the next node are loaded one node ahead.
+// The staged kernels stream the gathered input words through a per-warp ring
+// of shared-memory stages filled by cp.async copies; a stage holds the k input
+// rows of one node over 128 words, four per lane.  With VEC (W % 4 == 0,
+// 16-byte aligned rows) lane l takes words 4l .. 4l + 3 of the stage with
+// 16-byte copies, loads and stores; otherwise, for any W and alignment, words
+// l, l + 32, l + 64 and l + 96 with 4-byte ones (coalesced, no bank
+// conflicts; 36 more instructions on about 340 per stage).  A lane copies,
+// and later reads, only its own words, so the ring is lane-private: a lane
+// waits for its own copies (cp.async.wait_group) and no warp synchronisation
+// guards the ring.  The ring runs across node boundaries, so the copies of
+// the next node are in flight while the current node is evaluated, and the
+// connectivity row and table of the next node are loaded one node ahead.
 
 constexpr int kStageWords = 128;  // words per stage (4 per lane)
 
-template <int k>
-__device__ __forceinline__ void read_stage(const uint4* slot, uint32_t (&x)[4][k]) {
+// The lane's words of a stage at its position in a ring slot.
+template <int k, bool VEC>
+__device__ __forceinline__ void read_stage(const uint32_t* slot, uint32_t (&x)[4][k]) {
 #pragma unroll
     for (int i = 0; i < k; ++i) {
-        const uint4 v = slot[i * 32];
-        x[0][i] = v.x; x[1][i] = v.y; x[2][i] = v.z; x[3][i] = v.w;
+        if constexpr (VEC) {
+            const uint4 v = *reinterpret_cast<const uint4*>(slot + i * kStageWords);
+            x[0][i] = v.x; x[1][i] = v.y; x[2][i] = v.z; x[3][i] = v.w;
+        } else {
+#pragma unroll
+            for (int r = 0; r < 4; ++r) x[r][i] = slot[i * kStageWords + 32 * r];
+        }
     }
 }
 
 template <int k>
-__host__ __device__ constexpr int ring_bytes_per_warp(int stages) { return stages * k * 32 * 16; }
+__host__ __device__ constexpr int ring_bytes_per_warp(int stages) { return stages * k * kStageWords * 4; }
 
-// A node's k input rows as 32-bit offsets, in 16-byte units from the start
-// of the packed input, of the lane's first words: (row * W + wl) / 4.  The
-// launchers use the staged kernels only when w_in * W / 4 < 2^32.
-template <int k>
+// A node's k input rows as 32-bit word offsets from the start of the packed
+// input to the lane's first word: row * W + wl, in 16-byte units with VEC.
+// The launchers use the staged kernels only when these fit 32 bits.
+template <int k, bool VEC>
 __device__ __forceinline__ void node_offsets(const int* __restrict__ conn, int j, int w_in, int lane,
-                                             uint32_t W4, uint32_t wl4, uint32_t (&off)[k]) {
+                                             long long W, long long wl, uint32_t (&off)[k]) {
     int rows[k];
     node_rows<k>(conn, j, w_in, lane, rows);
+    const uint32_t Wu = (uint32_t)(VEC ? W >> 2 : W), wu = (uint32_t)(VEC ? wl >> 2 : wl);
 #pragma unroll
-    for (int i = 0; i < k; ++i) off[i] = (uint32_t)rows[i] * W4 + wl4;
+    for (int i = 0; i < k; ++i) off[i] = (uint32_t)rows[i] * Wu + wu;
 }
 
-// Copies of one stage (the lane's 16 bytes of each of the k rows, `s16`
-// 16-byte units past the node's offsets) into a ring slot.
-template <int k>
-__device__ __forceinline__ void issue_stage(uint4* slot, const uint4* __restrict__ xp4,
-                                            const uint32_t (&off)[k], uint32_t s16) {
+__device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
+    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem) : "memory");
+}
+
+// Copies of one stage (the lane's words of each of the k rows, `st` words past
+// the node's offsets) into a ring slot; without VEC and FULL only the words r
+// with left > 32 r (left: words of the row from the lane's first one).
+template <int k, bool VEC, bool FULL>
+__device__ __forceinline__ void issue_stage(uint32_t* slot, const uint32_t* __restrict__ xp,
+                                            const uint32_t (&off)[k], uint32_t st, long long left) {
 #pragma unroll
-    for (int i = 0; i < k; ++i) cp_async16(slot + i * 32, xp4 + (off[i] + s16));
+    for (int i = 0; i < k; ++i) {
+        if constexpr (VEC) {
+            cp_async16(slot + i * kStageWords, reinterpret_cast<const uint4*>(xp) + (off[i] + st / 4));
+        } else {
+            const uint32_t* src = xp + (off[i] + st);
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+                if (FULL || left > 32 * r) cp_async4(slot + i * kStageWords + 32 * r, src + 32 * r);
+        }
+    }
 }
 
 // Three stages per node and warp ring, three blocks per SM: the level-0
@@ -256,33 +281,32 @@ constexpr int kLayerMinBlocks = BITLOGIC_HARD_MINB;
 // s + NS - 1 (the last stage of node j, or stage s - 1 of the warp's next
 // node) are in flight.  FULL: the chunk lies inside the words and holds no
 // partial tail word, so no lane checks.
-template <int k, int NS, bool FULL>
-__device__ __forceinline__ void layer_staged_body(const uint4* __restrict__ xp4, int w_in, long long W,
+template <int k, int NS, bool VEC, bool FULL>
+__device__ __forceinline__ void layer_staged_body(const uint32_t* __restrict__ xp, int w_in, long long W,
                                                   const int* __restrict__ conn,
                                                   const uint64_t* __restrict__ table, int w,
                                                   uint32_t* __restrict__ yp, uint32_t tail_mask,
-                                                  uint4* ring_smem, int2* sPQ) {
-    constexpr int H = 1 << (k - 1);
-    constexpr int kSlot = k * 32;   // uint4 per stage
+                                                  uint32_t* ring_smem, int2* sPQ) {
+    constexpr int kSlot = k * kStageWords;   // words per stage
     static_assert(NS >= 2, "at least one stage in flight");
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    uint4* ring = ring_smem + (size_t)warp * (NS * kSlot) + lane;
-    const long long wl = (long long)blockIdx.y * (NS * kStageWords) + 4 * lane;   // stage 0 words
-    const uint32_t W4 = (uint32_t)(W >> 2), wl4 = (uint32_t)(wl >> 2);
+    const int l0 = VEC ? 4 * lane : lane;    // the lane's first word of a stage
+    uint32_t* ring = ring_smem + (size_t)warp * (NS * kSlot) + l0;
+    const long long wl = (long long)blockIdx.y * (NS * kStageWords) + l0;   // stage 0 words
     const int jstride = gridDim.x * kHardWarps;
     int j = blockIdx.x * kHardWarps + warp;
 
     uint32_t oc[k], on[k];   // row offsets of node j and of node j + jstride
 #pragma unroll
     for (int i = 0; i < k; ++i) oc[i] = on[i] = 0;
-    if (j < w) node_offsets<k>(conn, j, w_in, lane, W4, wl4, oc);
-    if (j + jstride < w) node_offsets<k>(conn, j + jstride, w_in, lane, W4, wl4, on);
-    // stage s of a node into slot s (W % 4 == 0: a lane's four words are all
-    // in range or all out); one commit group per stage
+    if (j < w) node_offsets<k, VEC>(conn, j, w_in, lane, W, wl, oc);
+    if (j + jstride < w) node_offsets<k, VEC>(conn, j + jstride, w_in, lane, W, wl, on);
+    // stage s of a node into slot s (with VEC a lane's four words are all in
+    // range or all out); one commit group per stage
     auto issue = [&](const uint32_t (&off)[k], int node, int s) {
         bool ok = node < w;
         if constexpr (!FULL) ok = ok && wl + s * kStageWords < W;
-        if (ok) issue_stage<k>(ring + s * kSlot, xp4, off, (uint32_t)(s * kStageWords / 4));
+        if (ok) issue_stage<k, VEC, FULL>(ring + s * kSlot, xp, off, (uint32_t)(s * kStageWords), W - wl - s * kStageWords);
         cp_async_commit();
     };
 #pragma unroll
@@ -298,7 +322,7 @@ __device__ __forceinline__ void layer_staged_body(const uint4* __restrict__ xp4,
         for (int s = 0; s < NS; ++s) {
             if (s == 0) {
                 issue(oc, j, NS - 1);
-                if (jn + jstride < w) node_offsets<k>(conn, jn + jstride, w_in, lane, W4, wl4, oc);
+                if (jn + jstride < w) node_offsets<k, VEC>(conn, jn + jstride, w_in, lane, W, wl, oc);
             } else {
                 issue(on, jn, s - 1);
             }
@@ -307,13 +331,25 @@ __device__ __forceinline__ void layer_staged_body(const uint4* __restrict__ xp4,
             if constexpr (!FULL) ok = wl + s * kStageWords < W;
             if (ok) {
                 uint32_t x[4][k];
-                read_stage<k>(ring + s * kSlot, x);
+                read_stage<k, VEC>(ring + s * kSlot, x);
                 uint32_t y[4];
                 mux_tree4_smem<k - 1, 0, k>(sPQ, x, y);
                 if constexpr (!FULL) {
-                    if (wl + s * kStageWords + 4 == W) y[3] &= tail_mask;   // word W - 1 is y[3]
+                    if constexpr (VEC) {
+                        if (wl + s * kStageWords + 4 == W) y[3] &= tail_mask;   // word W - 1 is y[3]
+                    } else {
+#pragma unroll
+                        for (int r = 0; r < 4; ++r)
+                            if (wl + s * kStageWords + 32 * r == W - 1) y[r] &= tail_mask;
+                    }
                 }
-                store_words<4>(out + s * kStageWords, y);
+                if constexpr (VEC) {
+                    store_words<4>(out + s * kStageWords, y);
+                } else {
+#pragma unroll
+                    for (int r = 0; r < 4; ++r)
+                        if (FULL || wl + s * kStageWords + 32 * r < W) out[s * kStageWords + 32 * r] = y[r];
+                }
             }
         }
         __syncwarp();   // the pairs are read before the next node rewrites them
@@ -327,23 +363,21 @@ __device__ __forceinline__ void layer_staged_body(const uint4* __restrict__ xp4,
     cp_async_wait<0>();
 }
 
-template <int k>
+template <int k, bool VEC>
 __global__ void __launch_bounds__(kHardWarps * 32, kLayerMinBlocks)
-hard_layer_staged_kernel(const uint4* __restrict__ xp4, int w_in, long long W,
+hard_layer_staged_kernel(const uint32_t* __restrict__ xp, int w_in, long long W,
                          const int* __restrict__ conn, const uint64_t* __restrict__ table, int w,
                          uint32_t* __restrict__ yp, uint32_t tail_mask) {
     constexpr int H = 1 << (k - 1);
-    extern __shared__ uint4 ring_smem[];
+    extern __shared__ __align__(16) uint32_t ring_smem[];
     __shared__ __align__(16) int2 sPQ[kHardWarps][H < 2 ? 2 : H];
     const long long end = (long long)(blockIdx.y + 1) * (kLayerNS * kStageWords);
     const bool full = end < W || (end == W && tail_mask == 0xffffffffu);
     int2* mine = sPQ[threadIdx.x >> 5];
     if (full)
-        layer_staged_body<k, kLayerNS, true>(xp4, w_in, W, conn, table, w, yp, tail_mask,
-                                              ring_smem, mine);
+        layer_staged_body<k, kLayerNS, VEC, true>(xp, w_in, W, conn, table, w, yp, tail_mask, ring_smem, mine);
     else
-        layer_staged_body<k, kLayerNS, false>(xp4, w_in, W, conn, table, w, yp, tail_mask,
-                                                         ring_smem, mine);
+        layer_staged_body<k, kLayerNS, VEC, false>(xp, w_in, W, conn, table, w, yp, tail_mask, ring_smem, mine);
 }
 
 // ------------------------------------------------- layer + popcount head --
@@ -359,7 +393,7 @@ __device__ __forceinline__ void csa(uint32_t& carry, uint32_t& sum, uint32_t a, 
 constexpr int kHeadWarps = 8;
 constexpr int kBigPlanes = 10;   // weight-8 planes: up to 8 * 1023 + 7 nodes per warp
 
-// Scalar path (any W and alignment).  grid.x: groups of 32 * R words,
+// One-word-per-lane path (any W and alignment; short rows).  grid.x: groups of 32 * R words,
 // grid.y: class c x split.  Lane l covers words R * l .. R * l + R - 1 of
 // the group.  Warp r of
 // a block takes nodes n0 + r, n0 + r + 8, ... of its slice and feeds their
@@ -463,7 +497,7 @@ hard_head_kernel(const uint32_t* __restrict__ xp, int w_in, long long W, long lo
     }
 }
 
-// ------------------------------------------- staged head (vector path) --
+// ----------------------------------------------------------- staged head --
 //
 // grid.x: class c x split (fast), grid.y: groups of 128 words, so that the
 // blocks in flight share a few word groups and the gathered slice of the
@@ -511,24 +545,25 @@ __host__ __device__ constexpr int head_smem_bytes() {
     return head_ring_bytes<k>() + kHeadSliceNodes * (k * 4 + 8);
 }
 
-template <int k, bool FULL>
-__device__ __forceinline__ void head_staged_body(const uint4* __restrict__ xp4, int w_in, long long W,
+template <int k, bool VEC, bool FULL>
+__device__ __forceinline__ void head_staged_body(const uint32_t* __restrict__ xp, int w_in, long long W,
                                                  long long N, const int* __restrict__ conn,
                                                  const uint64_t* __restrict__ table, int C, int g,
                                                  int splits, int per_split, uint32_t* __restrict__ yp,
                                                  int* __restrict__ counts, uint32_t tail_mask,
-                                                 uint4* ring_smem, int2* sPQ, const int* sConn,
+                                                 uint32_t* ring_smem, int2* sPQ, const int* sConn,
                                                  const uint64_t* sTab) {
-    constexpr int kSlot = k * 32;   // uint4 per stage
+    constexpr int kSlot = k * kStageWords;   // words per stage
     static_assert(kHeadRing == 4, "a loop iteration is kHeadRing node steps");
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int c = blockIdx.x / splits, sp = blockIdx.x - c * splits;
     const int n0 = c * g + sp * per_split;
     const int n1 = min(c * g + g, n0 + per_split);
-    const long long wq = (long long)blockIdx.y * kStageWords + 4 * lane;   // this lane's 4 words
-    const bool active = FULL || wq < W;   // W % 4 == 0: all four words are in range
-    const uint32_t W4 = (uint32_t)(W >> 2), wq4 = (uint32_t)(wq >> 2);
-    uint4* ring = ring_smem + (size_t)warp * (kHeadRing * kSlot) + lane;
+    const int l0 = VEC ? 4 * lane : lane;    // the lane's first word of the group
+    const long long wq = (long long)blockIdx.y * kStageWords + l0;
+    const bool active = FULL || wq < W;      // with VEC all four words are in range, or none
+    const uint32_t Wu = (uint32_t)(VEC ? W >> 2 : W), wu = (uint32_t)(VEC ? wq >> 2 : wq);
+    uint32_t* ring = ring_smem + (size_t)warp * (kHeadRing * kSlot) + l0;
     const int jfirst = n0 + warp;
 
     // issue stream: node ji, kHeadRing - 1 nodes ahead of the compute stream;
@@ -540,8 +575,8 @@ __device__ __forceinline__ void head_staged_body(const uint4* __restrict__ xp4, 
                 const int* rr = sConn + (ji - n0) * k;
                 uint32_t off[k];
 #pragma unroll
-                for (int i = 0; i < k; ++i) off[i] = (uint32_t)rr[i] * W4 + wq4;
-                issue_stage<k>(ring + slot * kSlot, xp4, off, 0u);
+                for (int i = 0; i < k; ++i) off[i] = (uint32_t)rr[i] * Wu + wu;
+                issue_stage<k, VEC, FULL>(ring + slot * kSlot, xp, off, 0u, W - wq);
             }
             ji += kHSWarps;
         }
@@ -569,12 +604,29 @@ __device__ __forceinline__ void head_staged_body(const uint4* __restrict__ xp4, 
         for (int r = 0; r < 4; ++r) y[r] = 0;
         if (jj < n1 && active) {
             uint32_t x[4][k];
-            read_stage<k>(ring + u * kSlot, x);
+            read_stage<k, VEC>(ring + u * kSlot, x);
             mux_tree4_smem<k - 1, 0, k>(sPQ, x, y);
             if constexpr (!FULL) {
-                if (wq + 4 == W) y[3] &= tail_mask;
+                if constexpr (VEC) {
+                    if (wq + 4 == W) y[3] &= tail_mask;
+                } else {
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        if (wq + 32 * r >= W) y[r] = 0;
+                        else if (wq + 32 * r == W - 1) y[r] &= tail_mask;
+                    }
+                }
             }
-            if (yp) store_words<4>(yp + (long long)jj * W + wq, y);
+            if (yp) {
+                uint32_t* out = yp + (long long)jj * W + wq;
+                if constexpr (VEC) {
+                    store_words<4>(out, y);
+                } else {
+#pragma unroll
+                    for (int r = 0; r < 4; ++r)
+                        if (FULL || wq + 32 * r < W) out[32 * r] = y[r];
+                }
+            }
         }
     };
 #pragma unroll 1
@@ -603,15 +655,23 @@ __device__ __forceinline__ void head_staged_body(const uint4* __restrict__ xp4, 
     __syncthreads();   // every warp is done with its ring: reuse it for the flush
 
     // planes [warp][plane][word], then the block sum [plane][word]
-    uint32_t* pl = reinterpret_cast<uint32_t*>(ring_smem);
+    uint32_t* pl = ring_smem;
     uint32_t* sum = pl + kHSWarps * kHeadPlanes * kStageWords;
     {
-        uint4* mine = reinterpret_cast<uint4*>(pl + warp * kHeadPlanes * kStageWords) + lane;
-        mine[0] = make_uint4(ones[0], ones[1], ones[2], ones[3]);
-        mine[kStageWords / 4] = make_uint4(twos[0], twos[1], twos[2], twos[3]);
+        uint32_t* mine = pl + warp * kHeadPlanes * kStageWords + l0;
+        auto put = [&](int plane, const uint32_t (&v)[4]) {
+            uint32_t* o = mine + plane * kStageWords;
+            if constexpr (VEC) {
+                *reinterpret_cast<uint4*>(o) = make_uint4(v[0], v[1], v[2], v[3]);
+            } else {
 #pragma unroll
-        for (int b = 0; b < kHeadNB; ++b)
-            mine[(2 + b) * (kStageWords / 4)] = make_uint4(big[b][0], big[b][1], big[b][2], big[b][3]);
+                for (int r = 0; r < 4; ++r) o[32 * r] = v[r];
+            }
+        };
+        put(0, ones);
+        put(1, twos);
+#pragma unroll
+        for (int b = 0; b < kHeadNB; ++b) put(2 + b, big[b]);
     }
     __syncthreads();
     if (threadIdx.x < kStageWords) {
@@ -644,14 +704,14 @@ __device__ __forceinline__ void head_staged_body(const uint4* __restrict__ xp4, 
 }
 
 
-template <int k>
+template <int k, bool VEC>
 __global__ void __launch_bounds__(kHSWarps * 32, kHeadMinBlocks)
-hard_head_staged_kernel(const uint4* __restrict__ xp4, int w_in, long long W, long long N,
+hard_head_staged_kernel(const uint32_t* __restrict__ xp, int w_in, long long W, long long N,
                         const int* __restrict__ conn, const uint64_t* __restrict__ table,
                         int C, int g, int splits, int per_split, uint32_t* __restrict__ yp,
                         int* __restrict__ counts, uint32_t tail_mask) {
     constexpr int H = 1 << (k - 1);
-    extern __shared__ uint4 ring_smem[];
+    extern __shared__ __align__(16) uint32_t ring_smem[];
     __shared__ __align__(16) int2 sPQ[kHSWarps][H < 2 ? 2 : H];
     int* sConn = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(ring_smem) + head_ring_bytes<k>());
     uint64_t* sTab = reinterpret_cast<uint64_t*>(sConn + kHeadSliceNodes * k);
@@ -676,10 +736,10 @@ hard_head_staged_kernel(const uint4* __restrict__ xp4, int w_in, long long W, lo
     const bool full = end < W || (end == W && tail_mask == 0xffffffffu);
     int2* mine = sPQ[threadIdx.x >> 5];
     if (full)
-        head_staged_body<k, true>(xp4, w_in, W, N, conn, table, C, g, splits, per_split, yp, counts,
+        head_staged_body<k, VEC, true>(xp, w_in, W, N, conn, table, C, g, splits, per_split, yp, counts,
                                   tail_mask, ring_smem, mine, sConn, sTab);
     else
-        head_staged_body<k, false>(xp4, w_in, W, N, conn, table, C, g, splits, per_split, yp, counts,
+        head_staged_body<k, VEC, false>(xp, w_in, W, N, conn, table, C, g, splits, per_split, yp, counts,
                                    tail_mask, ring_smem, mine, sConn, sTab);
 }
 
@@ -707,6 +767,17 @@ long long hard_word_chunk(int w_in, long long W) {
     return c < W ? c : W;
 }
 
+// Rows that the 16-byte form cannot take go to the staged kernels from this
+// many words on; up to 32 words three quarters of a stage would be idle, and
+// the one-word-per-lane kernels take those.  Measured against those kernels
+// for 313 words (10000 samples, 64000 x 64000 nodes, fan-in 6): pass 424 ->
+// 273 us; 2759 words (88278 samples, 26337 x 1900, 100 classes) 811 -> 444 us;
+// 226 words (7222 samples, 9534 x 17760, fan-in 4) 94 -> 58 us.
+#ifndef BITLOGIC_HARD_STAGED_MIN
+#define BITLOGIC_HARD_STAGED_MIN 33
+#endif
+constexpr long long kStagedMinWords = BITLOGIC_HARD_STAGED_MIN;
+
 // Opt in to more than the default 48 KB of shared memory per block when the
 // dynamic part plus the kernel's static part (a few KB) may exceed it.
 template <typename F>
@@ -721,11 +792,13 @@ int launch_hard(const uint32_t* xp, int w_in, long long N, const int* conn, cons
                 int w, uint32_t* yp, int C, int* counts, int* pred, cudaStream_t st) {
     const long long W = (N + 31) / 32;
     const uint32_t tail_mask = (N % 32) ? ((1u << (N % 32)) - 1u) : 0xffffffffu;
-    // staged kernels: 16-byte rows and 32-bit row offsets in 16-byte units
+    // staged kernels: 16-byte rows with 32-bit row offsets in 16-byte units, or
+    // any rows with 32-bit offsets in words
     const bool vec4 = (W % 4 == 0) && aligned16(xp) && (!yp || aligned16(yp)) &&
                       (unsigned long long)w_in * (unsigned long long)(W / 4) < (1ull << 32);
+    const bool staged = vec4 || (W >= kStagedMinWords && (unsigned long long)w_in * (unsigned long long)W < (1ull << 32));
     if (C == 0) {
-        if (vec4) {
+        if (staged) {
             // chunks of kLayerNS stages; nodes per warp: enough blocks for
             // about four waves of two per SM
             const long long gy = (W + kLayerNS * kStageWords - 1) / (kLayerNS * kStageWords);
@@ -735,9 +808,10 @@ int launch_hard(const uint32_t* xp, int w_in, long long N, const int* conn, cons
             npw = npw < 1 ? 1 : (npw > 8 ? 8 : npw);
             const long long gx = (w + kHardWarps * npw - 1) / (kHardWarps * npw);
             const int smem = kHardWarps * ring_bytes_per_warp<k>(kLayerNS);
-            if (set_dynamic_smem(hard_layer_staged_kernel<k>, smem)) return BITLOGIC_ERR_CUDA;
-            hard_layer_staged_kernel<k><<<dim3((unsigned)gx, (unsigned)gy), kHardWarps * 32, smem, st>>>(
-                reinterpret_cast<const uint4*>(xp), w_in, W, conn, table, w, yp, tail_mask);
+            auto kern = vec4 ? hard_layer_staged_kernel<k, true> : hard_layer_staged_kernel<k, false>;
+            if (set_dynamic_smem(kern, smem)) return BITLOGIC_ERR_CUDA;
+            kern<<<dim3((unsigned)gx, (unsigned)gy), kHardWarps * 32, smem, st>>>(xp, w_in, W, conn, table, w, yp,
+                                                                                 tail_mask);
         } else {
             const long long chunk = hard_word_chunk(w_in, W);
             const long long ny = (W + chunk - 1) / chunk;
@@ -751,7 +825,7 @@ int launch_hard(const uint32_t* xp, int w_in, long long N, const int* conn, cons
     const int g = w / C;
     if (cudaMemsetAsync(counts, 0, sizeof(int) * (size_t)N * (size_t)C, st) != cudaSuccess)
         return BITLOGIC_ERR_CUDA;
-    if (vec4) {
+    if (staged) {
         const long long wg = W / kStageWords + (W % kStageWords ? 1 : 0);
         // split a class over several blocks until a word group has about one
         // block per SM (the blocks in flight then share one or two word
@@ -766,10 +840,10 @@ int launch_hard(const uint32_t* xp, int w_in, long long N, const int* conn, cons
         }
         if ((long long)C * splits > 0x7fffffffll || wg > 65535) return BITLOGIC_ERR_SHAPE;
         const int smem = head_smem_bytes<k>();
-        if (set_dynamic_smem(hard_head_staged_kernel<k>, smem)) return BITLOGIC_ERR_CUDA;
-        hard_head_staged_kernel<k><<<dim3((unsigned)(C * splits), (unsigned)wg), kHSWarps * 32, smem, st>>>(
-            reinterpret_cast<const uint4*>(xp), w_in, W, N, conn, table, C, g, splits, per_split, yp, counts,
-            tail_mask);
+        auto kern = vec4 ? hard_head_staged_kernel<k, true> : hard_head_staged_kernel<k, false>;
+        if (set_dynamic_smem(kern, smem)) return BITLOGIC_ERR_CUDA;
+        kern<<<dim3((unsigned)(C * splits), (unsigned)wg), kHSWarps * 32, smem, st>>>(
+            xp, w_in, W, N, conn, table, C, g, splits, per_split, yp, counts, tail_mask);
     } else {
         const long long wg = (W + 31) / 32;
         int splits = 1;
