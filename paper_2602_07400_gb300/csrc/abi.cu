@@ -34,6 +34,7 @@ extern "C" int bitlogic_internal_index_error_route(cudaStream_t);
 extern "C" int bitlogic_internal_index_error_lut_through(cudaStream_t);
 extern "C" int bitlogic_internal_index_error_lut_bytes(cudaStream_t);
 extern "C" int bitlogic_internal_index_error_lut_codes(cudaStream_t);
+extern "C" int bitlogic_internal_index_error_lut_packed(cudaStream_t);
 
 extern "C" const char* bitlogic_status_string(int code) {
     switch (code) {
@@ -103,7 +104,7 @@ extern "C" int bitlogic_degree_order(const int32_t* off_host, int32_t n, int32_t
 
 extern "C" int bitlogic_device_error(cudaStream_t stream) {
     int worst = BITLOGIC_OK;
-    const int r[9] = {bitlogic_internal_index_error_lut_soft(stream),
+    const int r[10] = {bitlogic_internal_index_error_lut_soft(stream),
                       bitlogic_internal_index_error_head(stream),
                       bitlogic_internal_index_error_encode(stream),
                       bitlogic_internal_index_error_hard(stream),
@@ -111,7 +112,8 @@ extern "C" int bitlogic_device_error(cudaStream_t stream) {
                       bitlogic_internal_index_error_route(stream),
                       bitlogic_internal_index_error_lut_through(stream),
                       bitlogic_internal_index_error_lut_bytes(stream),
-                      bitlogic_internal_index_error_lut_codes(stream)};
+                      bitlogic_internal_index_error_lut_codes(stream),
+                       bitlogic_internal_index_error_lut_packed(stream)};
     for (int v : r) {
         if (v == BITLOGIC_ERR_CUDA) return v;
         if (v != BITLOGIC_OK) worst = v;

@@ -71,15 +71,45 @@ inline int make_thresholds(const uint8_t* thr_host, int32_t b, Thresholds* out) 
 // IEEE-rounded division (no fast-math).
 __device__ __forceinline__ float sigmoidf(float z) { return 1.0f / (1.0f + expf(-z)); }
 
-// Asynchronous 16-byte global -> shared copies (cp.async, bypassing L1),
-// grouped per pipeline stage.
+// Asynchronous global -> shared copies (cp.async), 16 bytes (bypassing L1) or
+// 4, grouped per pipeline stage.
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
     const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
 }
+__device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {   // 4 bytes, through L1
+    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem) : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
+
+// Reduce-scatter of N values per lane over the lane offsets O, O/2, ..., 1:
+// at each step a lane keeps half of its values (the upper half when lane bit
+// O is set), adds its partner's copy of that half and hands over the other
+// half; once one value is left the remaining steps add it across lanes.
+// Afterwards, for N0 = 2^k >= 32 values, lane l holds the sums of entries
+// l N0/32 .. l N0/32 + N0/32 - 1; for N0 < 32, of entry l >> (5 - k).  The
+// order of every addition is fixed.
+template <int N, int O, int M>
+__device__ __forceinline__ void warp_reduce_scatter(float (&v)[M], int lane) {
+    if constexpr (O > 0) {
+        if constexpr (N > 1) {
+            const bool up = (lane & O) != 0;
+#pragma unroll
+            for (int i = 0; i < N / 2; ++i) {
+                const float send = up ? v[i] : v[i + N / 2];
+                const float keep = up ? v[i + N / 2] : v[i];
+                v[i] = keep + __shfl_xor_sync(0xffffffffu, send, O);
+            }
+            warp_reduce_scatter<N / 2, O / 2>(v, lane);
+        } else {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], O);
+            warp_reduce_scatter<1, O / 2>(v, lane);
+        }
+    }
+}
 
 // Programmatic dependent launch (sm_90 and later).  A kernel launched with
 // launch_dependent() may start while the kernel before it on the stream is

@@ -237,11 +237,6 @@ __device__ __forceinline__ void node_offsets(const int* __restrict__ conn, int j
     for (int i = 0; i < k; ++i) off[i] = (uint32_t)rows[i] * Wu + wu;
 }
 
-__device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
-    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem) : "memory");
-}
-
 // Copies of one stage (the lane's words of each of the k rows, `st` words past
 // the node's offsets) into a ring slot; without VEC and FULL only the words r
 // with left > 32 r (left: words of the row from the lane's first one).

@@ -22,7 +22,7 @@
 // spending registers.
 #include <type_traits>
 
-#include "common.cuh"
+#include "lut_packed.cuh"
 
 namespace bitlogic {
 namespace {
@@ -44,6 +44,13 @@ namespace {
 #endif
 #ifndef BITLOGIC_FWD_WAVES
 #define BITLOGIC_FWD_WAVES 2
+#endif
+// rows that the 16-byte form cannot take (B % 4 != 0) are staged from this
+// fan-in on; below it the scalar kernel's occupancy is as good (16000 nodes,
+// 907 samples, forward and backward with input gradient: fan-in 4 167 us
+// scalar, 176 us staged; fan-in 6 600 us with the scalar kernels, 325 us staged)
+#ifndef BITLOGIC_FWD_STAGED_MIN_K
+#define BITLOGIC_FWD_STAGED_MIN_K 5
 #endif
 constexpr int kFwdWarps = BITLOGIC_FWD_WARPS;
 static_assert(kFwdWarps >= 1 && kFwdWarps <= 16, "forward warps per block");
@@ -286,10 +293,11 @@ lut_forward_kernel(const float* __restrict__ X, int w_in, long long B,
 }
 
 // Staged forward: one warp per (node, batch slice).  Each lane copies, reads
-// back and evaluates its own 4 consecutive samples of a stage (16-byte
-// chunks), so the ring needs no warp synchronisation.  Needs B % 4 == 0,
-// chunk % 4 == 0 and 16-byte aligned X and Y.
-template <int k>
+// back and evaluates its own 4 samples of a stage, so the ring needs no warp
+// synchronisation: with VEC (B % 4 == 0, chunk % 4 == 0, 16-byte aligned X and
+// Y) 4 consecutive ones in 16-byte pieces, otherwise samples lane + 32 c, 4
+// bytes each.
+template <int k, bool VEC>
 __global__ void __launch_bounds__(kFwdWarps * 32)
 lut_forward_staged_kernel(const float* __restrict__ X, int w_in, long long B,
                           const int* __restrict__ conn, const float* __restrict__ theta, int w,
@@ -325,22 +333,31 @@ lut_forward_staged_kernel(const float* __restrict__ X, int w_in, long long B,
         const float4 v = *reinterpret_cast<const float4*>(&sCoef[warp][a]);
         cf[a] = v.x; cf[a + 1] = v.y; cf[a + 2] = v.z; cf[a + 3] = v.w;
     }
-    float* ring = sRing[warp] + 4 * lane;       // this lane's column of every stage row
+    float* ring = sRing[warp] + (VEC ? 4 : 1) * lane;   // this lane's column of every stage row
     const long long s0 = (long long)blockIdx.y * chunk;
     const long long s1 = min(B, s0 + chunk);
     const float* src[k];
 #pragma unroll
-    for (int i = 0; i < k; ++i) src[i] = X + (long long)rows[i] * B + s0 + 4 * lane;
-    float* yr = Y + (long long)j * B + s0 + 4 * lane;
+    for (int i = 0; i < k; ++i) src[i] = X + (long long)rows[i] * B + s0 + (VEC ? 4 : 1) * lane;
+    float* yr = Y + (long long)j * B + s0 + (VEC ? 4 : 1) * lane;
     const int nst = (int)((s1 - s0 + CH - 1) / CH);
-    const long long lim = s1 - s0 - 4 * lane;   // this lane's chunks start below lim
+    const long long lim = s1 - s0 - (VEC ? 4 : 1) * lane;   // this lane's samples, from its first one, below lim
 
     int ib = 0;   // ring slot of the next stage to issue
     auto issue = [&](int st) {
         if (st < nst && (long long)st * CH < lim) {
             float* buf = ring + ib * (k * CH);
 #pragma unroll
-            for (int r = 0; r < k; ++r) cp_async16(buf + r * CH, src[r] + (long long)st * CH);
+            for (int r = 0; r < k; ++r) {
+                const float* row = src[r] + (long long)st * CH;
+                if constexpr (VEC) {
+                    cp_async16(buf + r * CH, row);
+                } else {
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+                        if ((long long)st * CH + 32 * c < lim) cp_async4(buf + r * CH + 32 * c, row + 32 * c);
+                }
+            }
         }
         cp_async_commit();
         ib = (ib + 1 == kStages) ? 0 : ib + 1;
@@ -355,7 +372,10 @@ lut_forward_staged_kernel(const float* __restrict__ X, int w_in, long long B,
             const float* buf = ring + rb * (k * CH);
             float4 xv[k];
 #pragma unroll
-            for (int i = 0; i < k; ++i) xv[i] = *reinterpret_cast<const float4*>(buf + i * CH);
+            for (int i = 0; i < k; ++i) {
+                if constexpr (VEC) xv[i] = *reinterpret_cast<const float4*>(buf + i * CH);
+                else xv[i] = make_float4(buf[i * CH], buf[i * CH + 32], buf[i * CH + 64], buf[i * CH + 96]);
+            }
             float o[4];
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
@@ -364,7 +384,14 @@ lut_forward_staged_kernel(const float* __restrict__ X, int w_in, long long B,
                 for (int i = 0; i < k; ++i) x[i] = comp(xv[i], c);
                 o[c] = fwd_tree_poly<k - 1, 0, L>(cf, x);
             }
-            *reinterpret_cast<float4*>(yr + (long long)st * CH) = make_float4(o[0], o[1], o[2], o[3]);
+            float* out = yr + (long long)st * CH;
+            if constexpr (VEC) {
+                *reinterpret_cast<float4*>(out) = make_float4(o[0], o[1], o[2], o[3]);
+            } else {
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    if ((long long)st * CH + 32 * c < lim) out[32 * c] = o[c];
+            }
         }
         rb = (rb + 1 == kStages) ? 0 : rb + 1;
     }
@@ -372,22 +399,6 @@ lut_forward_staged_kernel(const float* __restrict__ X, int w_in, long long B,
 }
 
 // ------------------------------------------------------------ backward --
-
-// Where a node's output gradient dY[j][.] comes from.
-//   rows:  dY + (j / group) * B   (group = 1: one row per node; group = g:
-//          the head's per-class gradient, shared by the g nodes of a class)
-//   terms: sum over e in [off[j], off[j+1]) of terms[edge[e]][.] in
-//          increasing e -- the next layer's input gradient, reduced on the
-//          fly from its per-edge terms instead of being materialised.  With
-//          edge == nullptr the term rows are stored in CSR order (row e).
-struct GradSource {
-    const float* dY;
-    int group;
-    const float* terms;
-    const int* off;
-    const int* edge;
-    int n_edges;
-};
 
 // Term row of CSR position e (edge == nullptr: rows in CSR order).
 __device__ __forceinline__ int term_row(const GradSource& gs, int e) {
@@ -415,8 +426,9 @@ __device__ __forceinline__ void term_range(const GradSource& gs, int j, int lane
     }
 }
 
-// Scalar backward (any B, any alignment, any k): one warp per node, one
-// sample per lane, next sample's gathers issued before this sample's tree.
+// Scalar backward (any B and alignment; fan-in 1 and 2 with the input
+// gradient, any fan-in without it): one warp per node, one sample per lane,
+// next sample's gathers issued before this sample's tree.
 template <int k, bool WANT_DX, bool TERMS>
 __global__ void __launch_bounds__(kFwdWarps * 32)
 lut_backward_kernel(const float* __restrict__ X, int w_in, long long B,
@@ -527,7 +539,10 @@ constexpr size_t node_smem_bytes() {
            (size_t)kNodesPerBlock * (1 << k) * sizeof(float);
 }
 
-// Staged backward.  A block holds kNodesPerBlock nodes with kWarpsPerNode
+// Staged backward for fan-in 2 with the input gradient, and for every fan-in
+// from 2 on without it when the gradient comes from upstream terms (fan-in 3
+// and more with the input gradient: lut_packed.cu).  A block holds
+// kNodesPerBlock nodes with kWarpsPerNode
 // warps each (by default one warp per node and per block, over the whole
 // batch); each warp of a node takes a contiguous range of its 128-sample
 // stages.
@@ -826,32 +841,6 @@ __host__ __device__ constexpr int theta_floats_per_warp() {
     return kStages * (k + 1) * kStageSamples;
 }
 
-// Reduce-scatter of N values per lane over the lane offsets O, O/2, ..., 1:
-// at each step a lane keeps half of its values (the upper half when lane bit
-// O is set), adds its partner's copy of that half and hands over the other
-// half; once one value is left the remaining steps add it across lanes.
-// Afterwards, for N0 = 2^k >= 32 values, lane l holds the sums of entries
-// l N0/32 .. l N0/32 + N0/32 - 1; for N0 < 32, of entry l >> (5 - k).  The
-// order of every addition is fixed.
-template <int N, int O, int M>
-__device__ __forceinline__ void warp_reduce_scatter(float (&v)[M], int lane) {
-    if constexpr (O > 0) {
-        if constexpr (N > 1) {
-            const bool up = (lane & O) != 0;
-#pragma unroll
-            for (int i = 0; i < N / 2; ++i) {
-                const float send = up ? v[i] : v[i + N / 2];
-                const float keep = up ? v[i + N / 2] : v[i];
-                v[i] = keep + __shfl_xor_sync(0xffffffffu, send, O);
-            }
-            warp_reduce_scatter<N / 2, O / 2>(v, lane);
-        } else {
-            v[0] += __shfl_xor_sync(0xffffffffu, v[0], O);
-            warp_reduce_scatter<1, O / 2>(v, lane);
-        }
-    }
-}
-
 template <int k>
 __host__ __device__ constexpr int theta_min_blocks() {
     return k <= 3 ? BITLOGIC_BWD_MIN_BLOCKS_SMALL : BITLOGIC_BWD_MIN_BLOCKS;
@@ -975,16 +964,16 @@ lut_backward_theta_kernel(const float* __restrict__ X, int w_in, long long B,
 
 // dX[i][s] = sum over the CSR positions p of input i (increasing p) of
 // P[edge[p]][s].  One block per input row i (and batch slice); warp r of the
-// block owns 128 samples (vector path: 4 per lane) or 32 (scalar path) and
-// issues the loads of all of the row's terms back to back, so each warp has
-// deg x 512 bytes in flight.  The row's ids are read once, one per lane.
+// block owns 128 samples, four per lane (VEC: consecutive ones in 16-byte
+// accesses; otherwise, for any B and alignment, 32 apart), and issues the
+// loads of all of the row's terms back to back, so each warp has deg x 512
+// bytes in flight.  The row's ids are read once, one per lane.
 constexpr int kCsrWarps = 8;
 
 template <bool VEC>
 __global__ void __launch_bounds__(kCsrWarps * 32)
 csr_reduce_kernel(const float* __restrict__ P, long long B, const int* __restrict__ off,
                   const int* __restrict__ edge, int w_in, int nE, float* __restrict__ dX) {
-    constexpr int SPW = VEC ? 128 : 32;   // samples per warp
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int i = blockIdx.x;
     int e0 = __ldg(off + i), e1 = __ldg(off + i + 1);
@@ -1010,40 +999,44 @@ csr_reduce_kernel(const float* __restrict__ P, long long B, const int* __restric
         }
         return id;
     };
-    const long long s = ((long long)blockIdx.y * kCsrWarps + warp) * SPW + (VEC ? 4 : 1) * lane;
-    const bool in = s < B;   // vector path: B % 4 == 0, all four samples in range
+    const long long s = ((long long)blockIdx.y * kCsrWarps + warp) * 128 + (VEC ? 4 : 1) * lane;
+    bool in[4];   // VEC: B % 4 == 0, all four samples in range or none
+#pragma unroll
+    for (int c = 0; c < 4; ++c) in[c] = s + (VEC ? 0 : 32 * c) < B;
     float* out = dX + (long long)i * B + s;
     // loads of up to kCsrBatch rows are issued before the first add; the
     // adds keep increasing position order
-    constexpr int kCsrBatch = 8;
+    constexpr int kCsrBatch = VEC ? 8 : 4;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int q0 = 0; q0 < deg; q0 += kCsrBatch) {
+        float4 v[kCsrBatch];
+#pragma unroll
+        for (int u = 0; u < kCsrBatch; ++u) {
+            const int id = q0 + u < deg ? edge_id(q0 + u) : -1;   // warp-uniform condition
+            v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (id >= 0) {
+                const float* row = P + (long long)id * B + s;
+                if constexpr (VEC) {
+                    if (in[0]) v[u] = ldg4(row);
+                } else {
+                    if (in[0]) v[u].x = __ldg(row);
+                    if (in[1]) v[u].y = __ldg(row + 32);
+                    if (in[2]) v[u].z = __ldg(row + 64);
+                    if (in[3]) v[u].w = __ldg(row + 96);
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < kCsrBatch; ++u)
+            if (q0 + u < deg) acc = add4(acc, v[u]);
+    }
     if constexpr (VEC) {
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int q0 = 0; q0 < deg; q0 += kCsrBatch) {
-            float4 v[kCsrBatch];
-#pragma unroll
-            for (int u = 0; u < kCsrBatch; ++u) {
-                const int id = q0 + u < deg ? edge_id(q0 + u) : -1;   // warp-uniform condition
-                v[u] = (in && id >= 0) ? ldg4(P + (long long)id * B + s) : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-#pragma unroll
-            for (int u = 0; u < kCsrBatch; ++u)
-                if (q0 + u < deg) acc = add4(acc, v[u]);
-        }
-        if (in) *reinterpret_cast<float4*>(out) = acc;
+        if (in[0]) *reinterpret_cast<float4*>(out) = acc;
     } else {
-        float acc = 0.f;
-        for (int q0 = 0; q0 < deg; q0 += kCsrBatch) {
-            float v[kCsrBatch];
-#pragma unroll
-            for (int u = 0; u < kCsrBatch; ++u) {
-                const int id = q0 + u < deg ? edge_id(q0 + u) : -1;
-                v[u] = (in && id >= 0) ? __ldg(P + (long long)id * B + s) : 0.f;
-            }
-#pragma unroll
-            for (int u = 0; u < kCsrBatch; ++u)
-                if (q0 + u < deg) acc += v[u];
-        }
-        if (in) *out = acc;
+        if (in[0]) out[0] = acc.x;
+        if (in[1]) out[32] = acc.y;
+        if (in[2]) out[64] = acc.z;
+        if (in[3]) out[96] = acc.w;
     }
 }
 
@@ -1072,7 +1065,9 @@ int launch_forward(const float* X, int w_in, long long B, const int* conn, const
     if (ny > 65535) return BITLOGIC_ERR_SHAPE;
     dim3 grid((unsigned)((w + kFwdWarps - 1) / kFwdWarps), (unsigned)ny);
     if (vec)
-        lut_forward_staged_kernel<k><<<grid, kFwdWarps * 32, 0, st>>>(X, w_in, B, conn, theta, w, node, Y, chunk);
+        lut_forward_staged_kernel<k, true><<<grid, kFwdWarps * 32, 0, st>>>(X, w_in, B, conn, theta, w, node, Y, chunk);
+    else if (k >= BITLOGIC_FWD_STAGED_MIN_K)
+        lut_forward_staged_kernel<k, false><<<grid, kFwdWarps * 32, 0, st>>>(X, w_in, B, conn, theta, w, node, Y, chunk);
     else
         lut_forward_kernel<k><<<grid, kFwdWarps * 32, 0, st>>>(X, w_in, B, conn, theta, w, node, Y, chunk);
     return launch_status();
@@ -1126,7 +1121,10 @@ int launch_backward(const float* X, int w_in, long long B, const int* conn, cons
             X, w_in, B, conn, theta, w, gs.dY, gs.group, dtheta, dY_out);
         return launch_status();
     }
-    if (P) {
+    // with the input gradient: fan-in 3 and more on packed pairs
+    if constexpr (k >= 3) {
+        if (P) return launch_backward_packed(k, X, w_in, B, conn, theta, w, node, gs, dtheta, P, epos, dY_out, st);
+    } else if (P) {
         return terms ? launch_backward_impl<k, true, true>(X, w_in, B, conn, theta, w, node, gs, dtheta, P, epos, dY_out,
                                                            staged, st)
                      : launch_backward_impl<k, true, false>(X, w_in, B, conn, theta, w, node, gs, dtheta, P, epos, dY_out,
@@ -1255,7 +1253,7 @@ extern "C" int bitlogic_csr_reduce(const float* edge_terms, int64_t B, const int
     if (B == 0) return BITLOGIC_OK;
     if (!edge_terms || !csr_off || !dX) return BITLOGIC_ERR_NULL;   // csr_edge NULL: terms in CSR order
     const bool vec = (B % 4 == 0) && aligned16(edge_terms) && aligned16(dX);
-    const long long per_block = (long long)kCsrWarps * (vec ? 128 : 32);
+    const long long per_block = (long long)kCsrWarps * 128;
     const long long gy = (B + per_block - 1) / per_block;
     if (gy > 65535) return BITLOGIC_ERR_SHAPE;
     dim3 grid((unsigned)w_in, (unsigned)gy);

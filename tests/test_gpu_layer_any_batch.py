@@ -1,0 +1,67 @@
+"""GPU parity of the fp32 layer kernels on batches that are no multiple of
+four and on rows off a 16-byte boundary: forward, backward with per-edge
+terms (from rows and from upstream terms, at given positions) and the CSR
+reduction, around the 32- and 128-sample edges of their stages."""
+import os
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2602_07400_gb300 as bl
+from paper_2602_07400_gb300 import synth
+from parity_util import check_exact, check_fwd, check_grad
+
+pytestmark = pytest.mark.gpu
+
+oracle.set_threads(os.cpu_count() or 1)
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def off_boundary(a, offset):
+    """The rows of a on the device, starting `offset` floats past an aligned address."""
+    buf = torch.empty(a.size + 8, device="cuda")
+    t = buf[offset:offset + a.size].view(a.shape)
+    t.copy_(dev(a))
+    return t
+
+
+@pytest.mark.parametrize("k", [3, 4, 5, 6])
+@pytest.mark.parametrize("B,offset", [(1, 0), (31, 0), (33, 0), (127, 0), (129, 0), (258, 0), (515, 0), (128, 1), (260, 3)])
+@pytest.mark.parametrize("node", ["soft", "st"])
+def test_layer_on_any_batch(k, B, offset, node):
+    w_in, w = 40, 70
+    X = synth.uniform_activations(w_in, B, seed=B)
+    conn = synth.connectivity(w, k, w_in, seed=1)
+    theta = synth.table_logits(w, 1 << k, seed=2)
+    dY = synth.uniform_gradients(w // 2, B, seed=3, scale=1e-2)
+    Xd, dYd = off_boundary(X, offset), off_boundary(dY, offset)
+    off, edge = bl.bitlogic_build_csr(conn, w_in)
+    pos = bl.bitlogic_csr_positions(edge)
+    Y = torch.full((w, B), np.nan, device="cuda")
+    bl.bitlogic_lut_forward_node(Xd, dev(conn), dev(theta), Y, node)
+    X64 = X.astype(np.float64)
+    check_fwd(Y, oracle.lut_forward(X64, conn, theta, node), "y", atol=1e-6 if node == "st" else 0.0)
+    dth = torch.full((w, 1 << k), np.nan, device="cuda")
+    P = torch.full((w * k, B), np.nan, device="cuda")
+    out = torch.full((w, B), np.nan, device="cuda")
+    bl.bitlogic_lut_backward_node(Xd, dev(conn), dev(theta), dth, node, dY=dYd, dy_group=2, edge_terms=P,
+                                  edge_pos=dev(pos), dY_out=out)
+    dX = torch.full((w_in, B), np.nan, device="cuda")
+    bl.bitlogic_csr_reduce(P, dev(off), None, dX)
+    full = np.repeat(dY, 2, axis=0)
+    check_exact(out.cpu().numpy(), full, "gradient used")
+    wth, wdx = oracle.lut_backward(X64, conn, theta, full.astype(np.float64), want_dx=True, node=node)
+    check_grad(dth, wth, "dtheta")
+    check_grad(dX, wdx, "dX")
+    # the gradient as one upstream term row per node: the same sums
+    dth_t, P_t = torch.empty_like(dth), torch.full_like(P, np.nan)
+    bl.bitlogic_lut_backward_node(Xd, dev(conn), dev(theta), dth_t, node, up_terms=dev(full),
+                                  up_off=dev(np.arange(w + 1, dtype=np.int32)), edge_terms=P_t, edge_pos=dev(pos))
+    check_exact(dth_t.cpu().numpy(), dth.cpu().numpy(), "dtheta from terms")
+    check_exact(P_t.cpu().numpy(), P.cpu().numpy(), "edge terms from terms")
+    assert bl.bitlogic_device_error() == 0
