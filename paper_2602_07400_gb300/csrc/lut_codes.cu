@@ -165,6 +165,28 @@ __device__ __forceinline__ uint32_t entry_addr(uint32_t v, int c, uint32_t base)
 // Bits of four codes that lie inside a table of 2^k1 entries.
 __device__ __forceinline__ uint32_t code_mask(int k1) { return (((1u << k1) - 1u) << 2) * 0x01010101u; }
 
+// A lane's samples in a 128-sample stage: nc consecutive ones from sample `at`
+// of the stage, the bytes of code word `word` from bit `shift` on.  A full
+// stage has one word and four samples per lane.  In the TAIL form of the
+// layer-2 kernels a last stage with at most 64 (32) samples left puts two
+// (four) lanes on a word, so that a half (a quarter) of the steps do for it.
+// The form is taken for small batches (short_tail): its second sample loop
+// costs the compiler's schedule of the first one more (4.05 -> 4.60 ms for the
+// step at 128000 nodes x 2048 samples, which has no tail) than it saves when
+// there are several full stages.  30000 x 30000 nodes, fan-in 6, per step:
+// 32 samples 187 (per-edge terms) -> 165 us, 64 samples 188 -> 172 us; without
+// it 64 samples took about as long as 128 (190 us).
+struct LaneSamples {
+    int word, shift, at, nc;
+};
+__device__ __forceinline__ LaneSamples lane_samples(long long left, int lane) {
+    const int lg = left > 64 ? 0 : left > 32 ? 1 : 2;   // lanes per word, as a power of two
+    const int word = lane & ((32 >> lg) - 1), part = lane >> (5 - lg), nc = 4 >> lg;
+    return {word, 8 * nc * part, 4 * word + nc * part, nc};
+}
+
+inline bool short_tail(long long B) { return B <= 192 && B % 128 != 0 && B % 128 <= 64; }
+
 // ------------------------------------------------------------ layer 2 value --
 
 // Horner value of the 8-entry Moebius subtable at O of both table halves.
@@ -196,7 +218,7 @@ __device__ __forceinline__ f32x2 fwd_tree2(const f32x2 (&cf)[N], const f32x2 (&x
 // samples 0.93 ms against 0.985 ms on fp32 rows, which waits for DRAM (6.9 GB
 // at 7 TB/s); here 2.6 GB move and the FP32 pipe and its operand reads bound
 // it (55% pipe-active).  12 or 20 blocks per SM: 1 and 9% slower steps.
-template <int k>
+template <int k, bool TAIL>
 __global__ void __launch_bounds__(32, BITLOGIC_CODED_FWD_BLOCKS)
 coded_forward_kernel(const uint8_t* __restrict__ codes, long long stride, const float* __restrict__ table1, int w_in,
                      int k1, long long B, const int* __restrict__ conn, const float* __restrict__ theta, int w,
@@ -218,14 +240,21 @@ coded_forward_kernel(const uint8_t* __restrict__ codes, long long stride, const 
 #pragma unroll
         for (int i = 0; i < NF; ++i) th[i] = (j < w && e0 + i < K) ? __ldg(theta + (long long)j * K + e0 + i) : 0.f;
     };
-    // code words of the first stage of the node whose inputs are in cin, into
-    // c; then cin moves on to node j
+    const LaneSamples tail = lane_samples(B - 128ll * (nst - 1), lane);   // of the last stage
+    // code words of stage st of the current row pointers
+    auto words = [&](uint32_t (&c)[k], int st) {
+        const int at = 32 * st + (!TAIL ? 0 : st + 1 == nst ? tail.word : lane);
+#pragma unroll
+        for (int i = 0; i < k; ++i) c[i] = __ldg(src[i] + at);
+    };
+    // the same of the first stage of the node whose inputs are in cin; then
+    // cin moves on to node j
     auto first_words = [&](uint32_t (&c)[k], int j) {
 #pragma unroll
-        for (int i = 0; i < k; ++i) {
-            src[i] = reinterpret_cast<const uint32_t*>(codes + (long long)__shfl_sync(0xffffffffu, cin, i) * stride) + lane;
-            c[i] = __ldg(src[i]);
-        }
+        for (int i = 0; i < k; ++i)
+            src[i] = reinterpret_cast<const uint32_t*>(codes + (long long)__shfl_sync(0xffffffffu, cin, i) * stride) +
+                     (TAIL ? 0 : lane);
+        words(c, 0);
         cin = load_inputs<k>(conn, j, w, lane);
     };
     ahead(blockIdx.x);
@@ -279,13 +308,12 @@ coded_forward_kernel(const uint8_t* __restrict__ codes, long long stride, const 
             uint32_t cn[k];   // the next stage's words, or the next node's first
             if (st + 1 < nst) {
 #pragma unroll
-                for (int i = 0; i < k; ++i) cn[i] = __ldg(src[i] + 32 * (st + 1));
+                for (int i = 0; i < k; ++i) cn[i] = 0u;
+                words(cn, st + 1);
             } else {
                 first_words(cn, j + 2 * G);   // past the last node: row 0, unused
             }
-            float o[4];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
+            auto value = [&](int c) {   // the node's value at sample c of the lane's words
                 f32x2 x[k - 1];
 #pragma unroll
                 for (int i = 0; i < k - 1; ++i) {
@@ -295,15 +323,29 @@ coded_forward_kernel(const uint8_t* __restrict__ codes, long long stride, const 
                 const float xt = lds(entry_addr(cw[k - 1], c, sTab) + (k - 1) * 256u);
                 float lo, hi;
                 unpack2(fwd_tree2<k - 2, 0>(cf, x), lo, hi);
-                o[c] = fmaf(xt, hi - lo, lo);
-            }
-            const long long s4 = 128ll * st + 4 * lane;
-            if (vec) {
-                if (s4 < B) *reinterpret_cast<float4*>(yr + s4) = make_float4(o[0], o[1], o[2], o[3]);
+                return fmaf(xt, hi - lo, lo);
+            };
+            if (!TAIL || st + 1 < nst) {
+                float o[4];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) o[c] = value(c);
+                const long long s4 = 128ll * st + 4 * lane;
+                if (vec) {
+                    if (s4 < B) *reinterpret_cast<float4*>(yr + s4) = make_float4(o[0], o[1], o[2], o[3]);
+                } else {
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+                        if (s4 + c < B) yr[s4 + c] = o[c];
+                }
             } else {
 #pragma unroll
-                for (int c = 0; c < 4; ++c)
-                    if (s4 + c < B) yr[s4 + c] = o[c];
+                for (int i = 0; i < k; ++i) cw[i] >>= tail.shift;
+                const long long s = 128ll * st + tail.at;
+#pragma unroll 1
+                for (int c = 0; c < tail.nc; ++c) {
+                    const float v = value(c);
+                    if (s + c < B) yr[s + c] = v;
+                }
             }
 #pragma unroll
             for (int i = 0; i < k; ++i) cw[i] = cn[i] & cmask;   // masked only now: nothing waits for the loads before
@@ -420,7 +462,7 @@ constexpr int coded_bwd_smem() {
     return (Order<k>::kArrays * 64 * 32 + k * 64) * (int)sizeof(float);
 }
 
-template <int k>
+template <int k, bool TAIL>
 __global__ void __launch_bounds__(32, coded_bwd_blocks<k>())
 coded_backward_kernel(const uint8_t* __restrict__ codes, long long stride, const float* __restrict__ table1, int w_in,
                       int k1, long long B, const int* __restrict__ conn, const float* __restrict__ theta, int w,
@@ -463,10 +505,14 @@ coded_backward_kernel(const uint8_t* __restrict__ codes, long long stride, const
 #pragma unroll
         for (int i = 0; i < NF; ++i) th[i] = (j < w && e0 + i < K) ? __ldg(theta + (long long)j * K + e0 + i) : 0.f;
     };
+    const LaneSamples tail = lane_samples(B - 128ll * (nst - 1), lane);   // of the last stage
+    // output gradient of the lane's samples of stage st (with TAIL those past
+    // nc are not evaluated), and with TAIL their code words
     auto load_g = [&](int st) {
-        const long long s = 128ll * st + 4 * lane;
+        const bool last = TAIL && st + 1 == nst;
+        const long long s = 128ll * st + (last ? tail.at : 4 * lane);
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (vec) {
+        if (vec && !last) {
             if (s < B) v = __ldg(reinterpret_cast<const float4*>(gsrc + s));
         } else {
             if (s < B) v.x = __ldg(gsrc + s);
@@ -476,6 +522,7 @@ coded_backward_kernel(const uint8_t* __restrict__ codes, long long stride, const
         }
         return v;
     };
+    auto word_of = [&](int st) { return st + 1 == nst ? tail.word : lane; };   // TAIL
     auto start = [&](int j) {   // tables, row pointers and first loads of node j
         cin = checked_input(cin, w_in);
         copy_tables<k>(sTab, table1, k1, cin, lane);
@@ -483,8 +530,8 @@ coded_backward_kernel(const uint8_t* __restrict__ codes, long long stride, const
 #pragma unroll
         for (int m = 0; m < k; ++m) {
             const int c = __shfl_sync(0xffffffffu, cin, O::slot_of(h, m));
-            src[m] = reinterpret_cast<const uint32_t*>(codes + (long long)c * stride) + lane;
-            cw[m] = __ldg(src[m]);
+            src[m] = reinterpret_cast<const uint32_t*>(codes + (long long)c * stride) + (TAIL ? 0 : lane);
+            cw[m] = __ldg(src[m] + (TAIL ? word_of(0) : 0));
         }
         g4 = load_g(0);
         cin = load_inputs<k>(conn, j + G, w, lane);
@@ -532,7 +579,7 @@ coded_backward_kernel(const uint8_t* __restrict__ codes, long long stride, const
         cp_async_wait<0>();
         __syncwarp();
 #pragma unroll
-        for (int m = 0; m < k; ++m) cw[m] &= cmask;
+        for (int m = 0; m < k; ++m) cw[m] = (cw[m] & cmask) >> (TAIL && nst == 1 ? tail.shift : 0);
         look(0);
 #pragma unroll 1
         for (int st = 0; st < nst; ++st) {
@@ -543,22 +590,23 @@ coded_backward_kernel(const uint8_t* __restrict__ codes, long long stride, const
             gn = make_float4(0.f, 0.f, 0.f, 0.f);
             if (st + 1 < nst) {
 #pragma unroll
-                for (int m = 0; m < k; ++m) cn[m] = __ldg(src[m] + 32 * (st + 1));
+                for (int m = 0; m < k; ++m) cn[m] = __ldg(src[m] + 32 * (st + 1) + (TAIL ? word_of(st + 1) : 0));
                 gn = load_g(st + 1);
             }
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const float g = c == 0 ? g4.x : c == 1 ? g4.y : c == 2 ? g4.z : g4.w;
+            // one sample: its tree, the inputs of sample `next` of the words in cw
+            // (after moving on to the next stage's words when `step`), its terms
+            // into the columns
+            auto sample = [&](float g, bool step, int next) {
                 float dx[k];
                 node_sample2<k>(cp, x, g, dx, acc);
                 uint32_t at[k];   // this sample's columns
 #pragma unroll
                 for (int m = 0; m < k; ++m) at[m] = 32u * ea[m] + cb[base(m)];
-                if (c == 3) {   // the inputs of the next sample
+                if (step) {   // on to the next stage
 #pragma unroll
-                    for (int m = 0; m < k; ++m) cw[m] = cn[m] & cmask;
+                    for (int m = 0; m < k; ++m) cw[m] = (cn[m] & cmask) >> (TAIL && st + 2 == nst ? tail.shift : 0);
                 }
-                look((c + 1) & 3);
+                look(next);
 #pragma unroll
                 for (int m0 = 0; m0 < k; m0 += C) {   // a step: slots m0 .. m0 + C - 1 of this lane's order
                     float old[C];
@@ -570,6 +618,15 @@ coded_backward_kernel(const uint8_t* __restrict__ codes, long long stride, const
                         if (m0 + i < k) sts(at[m0 + i] + column_off(m0 + i), old[i] + dx[m0 + i]);
                     __syncwarp();   // the other lane of these columns comes to them in another step
                 }
+            };
+            if (!TAIL || st + 1 < nst) {
+                sample(g4.x, false, 1);
+                sample(g4.y, false, 2);
+                sample(g4.z, false, 3);
+                sample(g4.w, true, 0);
+            } else {
+#pragma unroll 1
+                for (int c = 0; c < tail.nc; ++c) sample(c ? g4.y : g4.x, false, c + 1);   // nc <= 2
             }
             g4 = gn;
         }
@@ -701,7 +758,8 @@ int launch_coded_forward(const uint8_t* codes, long long stride, const float* ta
                          const int* conn, const float* theta, int w, int node, float* Y, cudaStream_t st) {
     const size_t smem = ((1 << k) + 2 * k * 64) * sizeof(float);
     const long long resident = (long long)sm_count() * BITLOGIC_CODED_FWD_BLOCKS;
-    coded_forward_kernel<k><<<(unsigned)(w < resident ? w : resident), 32, smem, st>>>(
+    auto kern = short_tail(B) ? coded_forward_kernel<k, true> : coded_forward_kernel<k, false>;
+    kern<<<(unsigned)(w < resident ? w : resident), 32, smem, st>>>(
         codes, stride, table, w_in, k1, B, conn, theta, w, node, Y, B % 4 == 0 && aligned16(Y));
     return launch_status();
 }
@@ -715,7 +773,8 @@ int launch_coded_backward(const uint8_t* codes, long long stride, const float* t
     // 1 KB of it per block) hold
     constexpr int fit = (228 * 1024) / (smem + 1024);
     const long long resident = (long long)sm_count() * (fit < coded_bwd_blocks<k>() ? fit : coded_bwd_blocks<k>());
-    coded_backward_kernel<k><<<(unsigned)(w < resident ? w : resident), 32, smem, st>>>(
+    auto kern = short_tail(B) ? coded_backward_kernel<k, true> : coded_backward_kernel<k, false>;
+    kern<<<(unsigned)(w < resident ? w : resident), 32, smem, st>>>(
         codes, stride, table, w_in, k1, B, conn, theta, w, node, dY, group, B % 4 == 0 && aligned16(dY), dtheta, corner,
         epos);
     return launch_status();

@@ -190,7 +190,8 @@ class TrainStep:
       dtheta-only layer-1 backward reads.
 
     Layer 1 reads the encoder's wires as bytes (``bytes1``, the default when
-    B % 4 == 0 and no layer-1 input gradient is wanted): its inputs are
+    B % 4 == 0, or on corner codes for any B, and no layer-1 input gradient is
+    wanted): its inputs are
     binary, so every corner weight of the relaxed table is 0 or 1 and the
     layer-1 forward is a table lookup (bitlogic_lut_forward_u8) and its table
     gradient adds each sample's gradient to the one entry the sample selects
@@ -236,8 +237,12 @@ class TrainStep:
         if through and (net.k2 > 3 or B % 4 != 0 or want_dx1):
             raise ValueError("the through route needs layer-2 fan-in <= 3, B % 4 == 0 and no layer-1 input gradient")
         self.through = bool(through)
+        # a batch that is no multiple of four takes binary wires for layer 1
+        # only on corner codes, whose kernels accept any B
+        ragged_codes = (B % 4 != 0 and not want_dx1 and csr_order and net.k2 >= 4 and fuse_dy1 is None
+                        and bytes1 is None and bits1 is None and codes1 is not False)
         if bytes1 is None:
-            bytes1 = B % 4 == 0 and not want_dx1
+            bytes1 = (B % 4 == 0 or ragged_codes) and not want_dx1
         terms_asked = fuse_dy1 is not None
         if fuse_dy1 is None:
             # on byte wires the layer-1 backward streams the terms itself
@@ -252,7 +257,7 @@ class TrainStep:
         self.loss = torch.zeros(1, **f32)
         self.dyg = torch.empty(C, B, **f32)          # gradient row shared by each class's nodes
         self.fuse_dy1 = bool(fuse_dy1) and not self.through
-        if bytes1 and (B % 4 != 0 or want_dx1):
+        if bytes1 and ((B % 4 != 0 and not ragged_codes) or want_dx1):
             raise ValueError("byte wires for layer 1 need B % 4 == 0 and no layer-1 input gradient")
         self.bytes1 = bool(bytes1)
         if bits1 is None:

@@ -11,6 +11,7 @@ import torch
 import oracle
 import paper_2602_07400_gb300 as bl
 from paper_2602_07400_gb300 import synth
+from paper_2602_07400_gb300.pipeline import Network, TrainStep
 from parity_util import check_exact, check_fwd, check_grad
 from test_gpu_bitrows import dev, pack_rows
 
@@ -133,3 +134,42 @@ def test_out_of_range_indices_are_flagged():
     bl.bitlogic_lut_forward_coded(codes, table, dev(conn), theta, Y)
     bl.bitlogic_lut_forward_coded(wild, table, dev(conn), theta, Yw)
     check_exact(Yw.cpu().numpy(), Y.cpu().numpy(), "code bits outside the table")
+
+
+@pytest.mark.parametrize("B,k,node", [(256, 6, "soft"), (127, 6, "soft"), (255, 4, "st"), (130, 5, "soft"), (37, 4, "soft")])
+def test_training_step_on_codes(B, k, node):
+    # the whole step, ragged batches included, against the oracle, and with
+    # dY1 kept (formed from the terms) the same outputs
+    wl = synth.Workload("codes", B, 60, 5, 40.0, (64, 128, 192), (300, 200), k, 5.0)
+    conn1, th1, conn2, th2 = synth.network(wl, seed=3)
+    x, labels = synth.blob_batch(B, wl.d, wl.classes, wl.sigma, seed=4)
+    net = Network(conn1, th1, conn2, th2, wl.w_in)
+    steps = []
+    for keep in (False, True):
+        st = TrainStep(net, B, wl.d, wl.thresholds, wl.classes, wl.tau, node=node, keep_dy1=keep)
+        assert st.codes1 and st.bits1 and st.fuse_dy1 and (st.dy1 is not None) == keep
+        st.load(x.cuda(), labels.cuda())
+        st.run()
+        steps.append(st)
+    torch.cuda.synchronize()
+    r = oracle.train_step(x.numpy(), labels.numpy(), wl.thresholds, conn1, th1, conn2, th2, wl.classes, wl.tau,
+                          want_dx1=False, node=node)
+    a, b = steps
+    check_fwd(a.y1, r["y1"], "y1")
+    check_fwd(a.y2, r["y2"], "y2", atol=1e-6 if node == "st" else 0.0)
+    check_fwd(a.logits, r["logits"], "logits", atol=1e-6)
+    for name in ("dth1", "dth2"):
+        check_grad(getattr(a, name), r[name], name)
+        check_exact(getattr(a, name).cpu().numpy(), getattr(b, name).cpu().numpy(), name)
+    check_grad(b.dy1, r["dy1"], "dy1")
+    assert bl.bitlogic_device_error() == 0
+
+
+def test_ragged_batch_refuses_other_binary_wires():
+    wl = synth.Workload("codes", 37, 60, 5, 40.0, (64, 128, 192), (300, 200), 4, 5.0)
+    net = Network(*synth.network(wl, seed=3), wl.w_in)
+    for kw in (dict(bytes1=True), dict(bits1=True), dict(bytes1=True, bits1=True)):
+        with pytest.raises(ValueError):
+            TrainStep(net, 37, wl.d, wl.thresholds, wl.classes, wl.tau, **kw)
+    st = TrainStep(net, 37, wl.d, wl.thresholds, wl.classes, wl.tau, codes1=False)
+    assert not st.codes1 and not st.bytes1 and st.bits.dtype == torch.float32
