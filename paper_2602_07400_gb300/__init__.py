@@ -15,6 +15,7 @@ bits int32 [rows, ceil(N/32)] holding uint32 words.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 from typing import Optional, Tuple
 
@@ -157,16 +158,33 @@ def _check(fn: str, code: int):
 
 
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
-def _stream(stream) -> ctypes.c_void_p:
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+def _current_stream() -> int:
+    return torch.cuda.current_stream().cuda_stream
+
+
+# The handle of the current stream without building a Stream object (this and
+# the checks below are most of a call's host time: the smallest training step
+# issues six calls).
+if hasattr(torch._C, "_cuda_getCurrentRawStream") and hasattr(torch._C, "_cuda_getDevice"):
+    def _current_stream() -> int:   # noqa: F811
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+
+
+def _stream(stream) -> int:
+    return _current_stream() if stream is None else stream.cuda_stream
 
 
 def _need(t: torch.Tensor, name: str, dtype: torch.dtype, shape: Tuple[int, ...]):
+    # one pass when everything fits; what does not is named by _refuse
+    if not ((t.__class__ is torch.Tensor or isinstance(t, torch.Tensor)) and t.dtype is dtype and t.is_cuda
+            and t.shape == shape and t.is_contiguous()):
+        _refuse(t, name, dtype, shape)
+
+
+def _refuse(t, name, dtype, shape):
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{name} must be a torch.Tensor")
     if t.dtype != dtype:
@@ -179,11 +197,21 @@ def _need(t: torch.Tensor, name: str, dtype: torch.dtype, shape: Tuple[int, ...]
         raise ValueError(f"{name}: expected shape {tuple(shape)}, got {tuple(t.shape)}")
 
 
-def _thr_buf(thresholds) -> Tuple[ctypes.Array, int]:
-    vals = [int(v) for v in thresholds]
+def _make_thr(vals) -> Tuple[ctypes.Array, int]:
     if any(v < 0 or v > 255 for v in vals):
         raise ValueError("thresholds must be uint8 values")
     return (ctypes.c_uint8 * max(1, len(vals)))(*vals), len(vals)
+
+
+# by value, so that equal thresholds share one host array; the library only
+# reads it, during the call
+_thr_of_ints = functools.lru_cache(maxsize=64)(_make_thr)
+
+
+def _thr_buf(thresholds) -> Tuple[ctypes.Array, int]:
+    if isinstance(thresholds, (list, tuple)) and all(type(v) is int for v in thresholds):
+        return _thr_of_ints(tuple(thresholds))
+    return _make_thr([int(v) for v in thresholds])
 
 
 def bitlogic_status_string(code: int) -> str:
