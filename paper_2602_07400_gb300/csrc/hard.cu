@@ -773,6 +773,32 @@ long long hard_word_chunk(int w_in, long long W) {
 #endif
 constexpr long long kStagedMinWords = BITLOGIC_HARD_STAGED_MIN;
 
+// Splits of a class for the staged head when there are few word groups: the
+// grid is then a few waves of blocks, and what counts is their number times a
+// block's time, its nodes per warp plus the flush of its counters (about
+// kHeadFlush nodes' worth).  Any number of splits that leaves a warp at least
+// four nodes.
+#ifndef BITLOGIC_HEAD_FLUSH
+#define BITLOGIC_HEAD_FLUSH 12
+#endif
+constexpr int kHeadFlush = BITLOGIC_HEAD_FLUSH, kHeadFewGroups = 16;
+int head_splits(int g, int C, long long wg) {
+    const long long slots = (long long)kHeadMinBlocks * sm_count();
+    int best = 1;
+    long long best_cost = -1;
+    for (int s = 1; s == 1 || (g / s >= 4 * kHSWarps && (long long)C * s * wg <= 8 * slots); ++s) {
+        const int per = (g + s - 1) / s;
+        if (per > kHeadSliceNodes) continue;
+        const long long waves = ((long long)C * s * wg + slots - 1) / slots;
+        const long long cost = waves * ((per + kHSWarps - 1) / kHSWarps + kHeadFlush);
+        if (best_cost < 0 || cost < best_cost) {
+            best_cost = cost;
+            best = s;
+        }
+    }
+    return best;
+}
+
 // Opt in to more than the default 48 KB of shared memory per block when the
 // dynamic part plus the kernel's static part (a few KB) may exceed it.
 template <typename F>
@@ -824,9 +850,14 @@ int launch_hard(const uint32_t* xp, int w_in, long long N, const int* conn, cons
         const long long wg = W / kStageWords + (W % kStageWords ? 1 : 0);
         // split a class over several blocks until a word group has about one
         // block per SM (the blocks in flight then share one or two word
-        // groups), keeping at least 8 nodes per warp
+        // groups), keeping at least 8 nodes per warp; for a few word groups
+        // see head_splits
         int splits = 1;
-        while (C * splits < sm_count() && g / (splits * 2) >= 8 * kHSWarps) splits *= 2;
+        if (wg < kHeadFewGroups) {
+            splits = head_splits(g, C, wg);
+        } else {
+            while (C * splits < sm_count() && g / (splits * 2) >= 8 * kHSWarps) splits *= 2;
+        }
         int per_split = (g + splits - 1) / splits;
         // counter capacity and the staged slice
         while ((per_split + kHSWarps - 1) / kHSWarps > kMaxNodesPerWarp || per_split > kHeadSliceNodes) {
