@@ -189,28 +189,6 @@ inline bool short_tail(long long B) { return B <= 192 && B % 128 != 0 && B % 128
 
 // ------------------------------------------------------------ layer 2 value --
 
-// Value of the subtree at level LV, index M of both table halves: 8-entry
-// Moebius subtables by Horner steps (levels 0 to 2) under lerps.  A subtable's
-// steps are written level by level, which the compiler schedules better than
-// the nested form (4.05 -> 4.02 ms for the step at 128000 nodes x 2048
-// samples; two or four samples at a time, to read each coefficient pair once
-// for all, gave no more: 4.02 and 4.14 ms).
-template <int LV, int M, int N, int n>
-__device__ __forceinline__ f32x2 fwd_tree2(const f32x2 (&cf)[N], const f32x2 (&x)[n]) {
-    if constexpr (LV == 2) {
-        f32x2 t[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) t[j] = fma2(cf[8 * M + 2 * j + 1], x[0], cf[8 * M + 2 * j]);
-        t[0] = fma2(x[1], t[1], t[0]);
-        t[2] = fma2(x[1], t[3], t[2]);
-        return fma2(x[2], t[2], t[0]);
-    } else {
-        const f32x2 lo = fwd_tree2<LV - 1, 2 * M>(cf, x);
-        const f32x2 hi = fwd_tree2<LV - 1, 2 * M + 1>(cf, x);
-        return fma2(x[LV], sub2(hi, lo), lo);
-    }
-}
-
 // Persistent one-warp blocks, a node over the whole batch; lane = 4
 // consecutive samples of a 128-sample stage, the code words of the next stage
 // (or node) and the next node's tables in flight.  The table's two halves
