@@ -10,6 +10,8 @@
 // and word.  The popcount GroupSum head (§3) is fused into the last layer:
 // every lane keeps carry-save (Harley-Seal) bit-sliced counters over its
 // group's nodes, so the last layer's packed outputs never reach memory.
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace bitlogic {
@@ -51,22 +53,22 @@ __device__ __forceinline__ uint32_t mux_tree(const int (&p)[H], const int (&q)[H
     }
 }
 
-// The tree for four words at once with the level-0 pairs read from shared
+// The tree for NW words at once with the level-0 pairs read from shared
 // memory (broadcast loads) instead of registers: depth first, so at most one
 // partial result per level and word is live.
-template <int L, int M, int k>
-__device__ __forceinline__ void mux_tree4_smem(const int2* __restrict__ sPQ, const uint32_t (&x)[4][k],
-                                               uint32_t (&out)[4]) {
+template <int L, int M, int k, int NW>
+__device__ __forceinline__ void mux_tree_smem(const int2* __restrict__ sPQ, const uint32_t (&x)[NW][k],
+                                              uint32_t (&out)[NW]) {
     if constexpr (L == 0) {
         const int2 v = sPQ[M];
 #pragma unroll
-        for (int r = 0; r < 4; ++r) out[r] = x[r][0] * (uint32_t)v.x + (uint32_t)v.y;
+        for (int r = 0; r < NW; ++r) out[r] = x[r][0] * (uint32_t)v.x + (uint32_t)v.y;
     } else {
-        uint32_t lo[4], hi[4];
-        mux_tree4_smem<L - 1, 2 * M, k>(sPQ, x, lo);
-        mux_tree4_smem<L - 1, 2 * M + 1, k>(sPQ, x, hi);
+        uint32_t lo[NW], hi[NW];
+        mux_tree_smem<L - 1, 2 * M, k>(sPQ, x, lo);
+        mux_tree_smem<L - 1, 2 * M + 1, k>(sPQ, x, hi);
 #pragma unroll
-        for (int r = 0; r < 4; ++r) out[r] = (x[r][L] & hi[r]) | (~x[r][L] & lo[r]);
+        for (int r = 0; r < NW; ++r) out[r] = (x[r][L] & hi[r]) | (~x[r][L] & lo[r]);
     }
 }
 
@@ -197,7 +199,9 @@ hard_layer_kernel(const uint32_t* __restrict__ xp, int w_in, long long W,
 // 16-byte aligned rows) lane l takes words 4l .. 4l + 3 of the stage with
 // 16-byte copies, loads and stores; otherwise, for any W and alignment, words
 // l, l + 32, l + 64 and l + 96 with 4-byte ones (coalesced, no bank
-// conflicts; 36 more instructions on about 340 per stage).  A lane copies,
+// conflicts; 36 more instructions on about 340 per stage), of which a last
+// stage of at most 64 (32) words evaluates two (one): 10000 samples, 313
+// words, through 64000 x 64000 nodes 254 -> 230 us.  A lane copies,
 // and later reads, only its own words, so the ring is lane-private: a lane
 // waits for its own copies (cp.async.wait_group) and no warp synchronisation
 // guards the ring.  The ring runs across node boundaries, so the copies of
@@ -206,9 +210,10 @@ hard_layer_kernel(const uint32_t* __restrict__ xp, int w_in, long long W,
 
 constexpr int kStageWords = 128;  // words per stage (4 per lane)
 
-// The lane's words of a stage at its position in a ring slot.
-template <int k, bool VEC>
-__device__ __forceinline__ void read_stage(const uint32_t* slot, uint32_t (&x)[4][k]) {
+// The lane's first NW words of a stage at its position in a ring slot.
+template <int k, bool VEC, int NW>
+__device__ __forceinline__ void read_stage(const uint32_t* slot, uint32_t (&x)[NW][k]) {
+    static_assert(!VEC || NW == 4, "16-byte pieces hold four words");
 #pragma unroll
     for (int i = 0; i < k; ++i) {
         if constexpr (VEC) {
@@ -216,7 +221,7 @@ __device__ __forceinline__ void read_stage(const uint32_t* slot, uint32_t (&x)[4
             x[0][i] = v.x; x[1][i] = v.y; x[2][i] = v.z; x[3][i] = v.w;
         } else {
 #pragma unroll
-            for (int r = 0; r < 4; ++r) x[r][i] = slot[i * kStageWords + 32 * r];
+            for (int r = 0; r < NW; ++r) x[r][i] = slot[i * kStageWords + 32 * r];
         }
     }
 }
@@ -324,27 +329,37 @@ __device__ __forceinline__ void layer_staged_body(const uint32_t* __restrict__ x
             cp_async_wait<NS - 1>();
             bool ok = true;
             if constexpr (!FULL) ok = wl + s * kStageWords < W;
-            if (ok) {
-                uint32_t x[4][k];
+            // NW words of the lane (the rest of a short stage is not evaluated)
+            auto eval = [&](auto words) {
+                constexpr int NW = decltype(words)::value;
+                uint32_t x[NW][k];
                 read_stage<k, VEC>(ring + s * kSlot, x);
-                uint32_t y[4];
-                mux_tree4_smem<k - 1, 0, k>(sPQ, x, y);
+                uint32_t y[NW];
+                mux_tree_smem<k - 1, 0, k>(sPQ, x, y);
                 if constexpr (!FULL) {
                     if constexpr (VEC) {
-                        if (wl + s * kStageWords + 4 == W) y[3] &= tail_mask;   // word W - 1 is y[3]
+                        if (wl + s * kStageWords + 4 == W) y[NW - 1] &= tail_mask;   // word W - 1 is y[3]
                     } else {
 #pragma unroll
-                        for (int r = 0; r < 4; ++r)
+                        for (int r = 0; r < NW; ++r)
                             if (wl + s * kStageWords + 32 * r == W - 1) y[r] &= tail_mask;
                     }
                 }
                 if constexpr (VEC) {
-                    store_words<4>(out + s * kStageWords, y);
+                    store_words<NW>(out + s * kStageWords, y);
                 } else {
 #pragma unroll
-                    for (int r = 0; r < 4; ++r)
+                    for (int r = 0; r < NW; ++r)
                         if (FULL || wl + s * kStageWords + 32 * r < W) out[s * kStageWords + 32 * r] = y[r];
                 }
+            };
+            if constexpr (VEC || FULL) {
+                if (ok) eval(std::integral_constant<int, 4>{});
+            } else {
+                const long long left = W - (wl - l0) - s * kStageWords;   // words of the stage: warp-uniform
+                if (left > 64) eval(std::integral_constant<int, 4>{});
+                else if (left > 32) eval(std::integral_constant<int, 2>{});
+                else if (left > 0) eval(std::integral_constant<int, 1>{});
             }
         }
         __syncwarp();   // the pairs are read before the next node rewrites them
@@ -540,7 +555,7 @@ __host__ __device__ constexpr int head_smem_bytes() {
     return head_ring_bytes<k>() + kHeadSliceNodes * (k * 4 + 8);
 }
 
-template <int k, bool VEC, bool FULL>
+template <int k, bool VEC, bool FULL, int NW>
 __device__ __forceinline__ void head_staged_body(const uint32_t* __restrict__ xp, int w_in, long long W,
                                                  long long N, const int* __restrict__ conn,
                                                  const uint64_t* __restrict__ table, int C, int g,
@@ -580,33 +595,33 @@ __device__ __forceinline__ void head_staged_body(const uint32_t* __restrict__ xp
     issue(0);
     issue(1);
     issue(2);
-    uint32_t ones[4], twos[4], big[kHeadNB][4];
+    uint32_t ones[NW], twos[NW], big[kHeadNB][NW];
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
+    for (int r = 0; r < NW; ++r) {
         ones[r] = twos[r] = 0;
 #pragma unroll
         for (int b = 0; b < kHeadNB; ++b) big[b][r] = 0;
     }
     // node step u of a loop iteration (node jj): the loop body has kHeadRing
     // steps, so step u reads slot u and refills slot u + 3 (mod kHeadRing).
-    // Returns the node's four output words (0 past the slice or the words).
-    auto node = [&](int jj, int u, uint32_t (&y)[4]) {
+    // Returns the node's NW output words (0 past the slice or the words).
+    auto node = [&](int jj, int u, uint32_t (&y)[NW]) {
         __syncwarp();   // the previous node's pairs are read
         node_pairs_smem<k>(jj < n1 ? sTab[jj - n0] : 0ull, lane, sPQ);   // 0 past the slice: harmless
         issue((u + kHeadRing - 1) % kHeadRing);
         cp_async_wait<kHeadRing - 1>();
 #pragma unroll
-        for (int r = 0; r < 4; ++r) y[r] = 0;
+        for (int r = 0; r < NW; ++r) y[r] = 0;
         if (jj < n1 && active) {
-            uint32_t x[4][k];
+            uint32_t x[NW][k];
             read_stage<k, VEC>(ring + u * kSlot, x);
-            mux_tree4_smem<k - 1, 0, k>(sPQ, x, y);
+            mux_tree_smem<k - 1, 0, k>(sPQ, x, y);
             if constexpr (!FULL) {
                 if constexpr (VEC) {
-                    if (wq + 4 == W) y[3] &= tail_mask;
+                    if (wq + 4 == W) y[NW - 1] &= tail_mask;
                 } else {
 #pragma unroll
-                    for (int r = 0; r < 4; ++r) {
+                    for (int r = 0; r < NW; ++r) {
                         if (wq + 32 * r >= W) y[r] = 0;
                         else if (wq + 32 * r == W - 1) y[r] &= tail_mask;
                     }
@@ -615,10 +630,10 @@ __device__ __forceinline__ void head_staged_body(const uint32_t* __restrict__ xp
             if (yp) {
                 uint32_t* out = yp + (long long)jj * W + wq;
                 if constexpr (VEC) {
-                    store_words<4>(out, y);
+                    store_words<NW>(out, y);
                 } else {
 #pragma unroll
-                    for (int r = 0; r < 4; ++r)
+                    for (int r = 0; r < NW; ++r)
                         if (FULL || wq + 32 * r < W) out[32 * r] = y[r];
                 }
             }
@@ -626,15 +641,15 @@ __device__ __forceinline__ void head_staged_body(const uint32_t* __restrict__ xp
     };
 #pragma unroll 1
     for (int j = jfirst; j < n1; j += 4 * kHSWarps) {
-        uint32_t ya[4], yb[4], t1[4];
+        uint32_t ya[NW], yb[NW], t1[NW];
         node(j, 0, ya);
         node(j + kHSWarps, 1, yb);
 #pragma unroll
-        for (int r = 0; r < 4; ++r) csa(t1[r], ones[r], ones[r], ya[r], yb[r]);
+        for (int r = 0; r < NW; ++r) csa(t1[r], ones[r], ones[r], ya[r], yb[r]);
         node(j + 2 * kHSWarps, 2, ya);
         node(j + 3 * kHSWarps, 3, yb);
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
+        for (int r = 0; r < NW; ++r) {
             uint32_t t2, e;
             csa(t2, ones[r], ones[r], ya[r], yb[r]);
             csa(e, twos[r], twos[r], t1[r], t2);
@@ -654,13 +669,15 @@ __device__ __forceinline__ void head_staged_body(const uint32_t* __restrict__ xp
     uint32_t* sum = pl + kHSWarps * kHeadPlanes * kStageWords;
     {
         uint32_t* mine = pl + warp * kHeadPlanes * kStageWords + l0;
-        auto put = [&](int plane, const uint32_t (&v)[4]) {
+        // with NW < 4 the group's other words are past the row's end: their
+        // sums are formed from whatever is there and belong to no sample
+        auto put = [&](int plane, const uint32_t (&v)[NW]) {
             uint32_t* o = mine + plane * kStageWords;
             if constexpr (VEC) {
-                *reinterpret_cast<uint4*>(o) = make_uint4(v[0], v[1], v[2], v[3]);
+                store_words<NW>(o, v);
             } else {
 #pragma unroll
-                for (int r = 0; r < 4; ++r) o[32 * r] = v[r];
+                for (int r = 0; r < NW; ++r) o[32 * r] = v[r];
             }
         };
         put(0, ones);
@@ -730,12 +747,21 @@ hard_head_staged_kernel(const uint32_t* __restrict__ xp, int w_in, long long W, 
     const long long end = (long long)(blockIdx.y + 1) * kStageWords;
     const bool full = end < W || (end == W && tail_mask == 0xffffffffu);
     int2* mine = sPQ[threadIdx.x >> 5];
-    if (full)
-        head_staged_body<k, VEC, true>(xp, w_in, W, N, conn, table, C, g, splits, per_split, yp, counts,
-                                  tail_mask, ring_smem, mine, sConn, sTab);
-    else
-        head_staged_body<k, VEC, false>(xp, w_in, W, N, conn, table, C, g, splits, per_split, yp, counts,
-                                   tail_mask, ring_smem, mine, sConn, sTab);
+    auto body = [&](auto full_group, auto words) {
+        head_staged_body<k, VEC, decltype(full_group)::value, decltype(words)::value>(
+            xp, w_in, W, N, conn, table, C, g, splits, per_split, yp, counts, tail_mask, ring_smem, mine, sConn, sTab);
+    };
+    using std::integral_constant;
+    if (full) {
+        body(std::true_type{}, integral_constant<int, 4>{});
+    } else if constexpr (VEC) {
+        body(std::false_type{}, integral_constant<int, 4>{});
+    } else {
+        const long long left = W - (long long)blockIdx.y * kStageWords;   // words of the group
+        if (left > 64) body(std::false_type{}, integral_constant<int, 4>{});
+        else if (left > 32) body(std::false_type{}, integral_constant<int, 2>{});
+        else body(std::false_type{}, integral_constant<int, 1>{});
+    }
 }
 
 __global__ void __launch_bounds__(256)
@@ -766,7 +792,7 @@ long long hard_word_chunk(int w_in, long long W) {
 // many words on; up to 32 words three quarters of a stage would be idle, and
 // the one-word-per-lane kernels take those.  Measured against those kernels
 // for 313 words (10000 samples, 64000 x 64000 nodes, fan-in 6): pass 424 ->
-// 273 us; 2759 words (88278 samples, 26337 x 1900, 100 classes) 811 -> 444 us;
+// 273 us (230 with the short stages and the head's splits below); 2759 words (88278 samples, 26337 x 1900, 100 classes) 811 -> 444 us;
 // 226 words (7222 samples, 9534 x 17760, fan-in 4) 94 -> 58 us.
 #ifndef BITLOGIC_HARD_STAGED_MIN
 #define BITLOGIC_HARD_STAGED_MIN 33
