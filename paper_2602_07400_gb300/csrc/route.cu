@@ -27,6 +27,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "packed.cuh"
 
 namespace bitlogic {
 namespace {
@@ -38,12 +39,26 @@ __device__ __forceinline__ float4 ldg4r(const float* p) { return __ldg(reinterpr
 // Layer inputs come as fp32 rows or as byte rows (the encoder's 0/1 wires,
 // a quarter of the bytes to gather): one value and four consecutive values
 // of a row, as floats.
+// Bytes t and t + 1 of w as floats: each byte in the lowest mantissa bits of
+// 2^23, less 2^23 (exact), the two subtractions in one packed instruction.  The
+// byte-row kernels are bound by issue slots (81 and 71%), most of them these
+// conversions and the multiply-adds: 32000 slots x 16 candidates x 1024
+// samples, forward 73 -> 65 us with the multiply-adds packed too, logits'
+// gradient 95 -> 92 us.
+__device__ __forceinline__ f32x2 byte_pair(uint32_t w, int t) {
+    const float a = __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7440u + (unsigned)t));
+    const float b = __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7440u + (unsigned)(t + 1)));
+    return sub2(pack2(a, b), pack2(8388608.0f, 8388608.0f));
+}
 __device__ __forceinline__ float in_value(const float* p) { return __ldg(p); }
 __device__ __forceinline__ float in_value(const uint8_t* p) { return (float)__ldg(p); }
 __device__ __forceinline__ float4 in_quad(const float* p) { return ldg4r(p); }
 __device__ __forceinline__ float4 in_quad(const uint8_t* p) {
     const uint32_t w = __ldg(reinterpret_cast<const uint32_t*>(p));
-    return make_float4((float)(w & 0xffu), (float)((w >> 8) & 0xffu), (float)((w >> 16) & 0xffu), (float)(w >> 24));
+    float4 v;
+    unpack2(byte_pair(w, 0), v.x, v.y);
+    unpack2(byte_pair(w, 2), v.z, v.w);
+    return v;
 }
 
 // Softmax of the slot's logits on lanes m < Kc (other lanes 0), the lane's
@@ -147,9 +162,9 @@ route_forward_bytes16_kernel(const uint8_t* __restrict__ X, int w_in, long long 
     const long long s1 = min(B, s0 + chunk);
     float* out = Xr + e * B;
     for (long long s = s0 + 16 * lane; s < s1; s += 512) {
-        float acc[16];
+        f32x2 acc[8];   // the 16 samples in pairs: each sample's sum as in the fp32 form
 #pragma unroll
-        for (int t = 0; t < 16; ++t) acc[t] = 0.f;
+        for (int t = 0; t < 8; ++t) acc[t] = 0ull;
         constexpr int G = KC < 4 ? KC : 4;   // loads issued together
 #pragma unroll
         for (int m0 = 0; m0 < KC; m0 += G) {
@@ -158,16 +173,15 @@ route_forward_bytes16_kernel(const uint8_t* __restrict__ X, int w_in, long long 
             for (int u = 0; u < G; ++u) v[u] = __ldg(reinterpret_cast<const uint4*>(row[m0 + u] + s));
 #pragma unroll
             for (int u = 0; u < G; ++u) {
-                const float q = pm[m0 + u];
+                const f32x2 q = pack2(pm[m0 + u], pm[m0 + u]);
                 const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
 #pragma unroll
-                for (int t = 0; t < 16; ++t)
-                    acc[t] = fmaf(q, (float)((w[t >> 2] >> (8 * (t & 3))) & 0xffu), acc[t]);
+                for (int t = 0; t < 8; ++t) acc[t] = fma2(q, byte_pair(w[t >> 1], 2 * (t & 1)), acc[t]);
             }
         }
 #pragma unroll
         for (int t = 0; t < 16; t += 4)
-            *reinterpret_cast<float4*>(out + s + t) = make_float4(acc[t], acc[t + 1], acc[t + 2], acc[t + 3]);
+            *reinterpret_cast<ulonglong2*>(out + s + t) = make_ulonglong2(acc[t / 2], acc[t / 2 + 1]);
     }
 }
 
@@ -279,10 +293,15 @@ route_dr_kernel(const T* __restrict__ X, int w_in, long long B, const int* __res
 // dX[c][s] = sum over the CSR positions q of input c (increasing q) of
 // prob[id_q] G[id_q / Kc][s], id_q = csr_edge[q] (candidate edge e*Kc + m).
 // Warp w of a block owns input row 8 blockIdx.x + w and the block's batch
-// slice (128 samples on the vector path, 32 otherwise); the grid runs the
-// rows fastest, so the blocks in flight share one slice of G, which stays
-// in L2 while every G row is read by about Kc input rows.  The row's first
-// 32 edge ids and weights are held one per lane.
+// slice (256 samples on the vector path, two groups of 4 per lane, 32
+// otherwise); the grid runs the rows fastest, so the blocks in flight share
+// one slice of G, which stays in L2 while every G row is read by about Kc
+// input rows.  The row's positions are taken 32 at a time, lane u holding the
+// row and weight of position u; a batch of four rows has no checks of its own
+// unless one of the 32 is out of range.  Bound by L2 reads (2.1 GB for 32000
+// slots x 16 candidates x 1024 samples, 18 TB/s): 131 -> 116 us against one
+// group of 4 samples per lane with a check per row, which was bound by issue
+// slots (75%).
 constexpr int kRdxWarps = 8;
 
 template <bool VEC>
@@ -290,7 +309,7 @@ __global__ void __launch_bounds__(kRdxWarps * 32)
 route_dx_kernel(const float* __restrict__ G, long long B, const float* __restrict__ prob, int Kc,
                 const int* __restrict__ off, const int* __restrict__ edge, int w_in, int nE,
                 float* __restrict__ dX) {
-    constexpr int SPW = VEC ? 128 : 32;
+    constexpr int SPW = VEC ? 256 : 32;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int i = blockIdx.x * kRdxWarps + warp;
     if (i >= w_in) return;
@@ -301,67 +320,98 @@ route_dx_kernel(const float* __restrict__ G, long long B, const float* __restric
     }
     const int deg = e1 - e0;
     const long long s = (long long)blockIdx.y * SPW + (VEC ? 4 : 1) * lane;
-    const bool in = s < B;
-    // the row's positions in chunks of 32: lane u holds the G row (slot) and
-    // weight of position q0 + u (slot -1: out of range, read as zero)
-    constexpr int kBatch = 8;
-    auto accumulate = [&](auto& acc) {
+    // lane u: slot (G row) and weight of position c0 + u; slot -1 past the end
+    // or out of range (adds nothing)
+    int my_slot;
+    float my_w;
+    auto take = [&](int c0) {
+        my_slot = -1;
+        my_w = 0.f;
+        bool bad = false;
+        if (c0 + lane < deg) {
+            const int id = __ldg(edge + e0 + c0 + lane);
+            if ((unsigned)id >= (unsigned)nE) {
+                flag_index_error();
+                bad = true;
+            } else {
+                my_slot = id / Kc;
+                my_w = __ldg(prob + id);
+            }
+        }
+        return __any_sync(0xffffffffu, bad);
+    };
+    if constexpr (VEC) {
+        const bool in0 = s < B, in1 = s + 128 < B;
+        float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
+        const float* base = G + (in0 ? s : 0);
+        const int second = in1 ? 128 : 0;   // lanes out of range read, and drop, the first samples
+        auto add = [](float4& a, float w, const float4& v) {
+            a.x = fmaf(w, v.x, a.x);
+            a.y = fmaf(w, v.y, a.y);
+            a.z = fmaf(w, v.z, a.z);
+            a.w = fmaf(w, v.w, a.w);
+        };
         for (int c0 = 0; c0 < deg; c0 += 32) {
-            int my_slot = -1;
-            float my_w = 0.f;
-            if (c0 + lane < deg) {
-                const int id = __ldg(edge + e0 + c0 + lane);
-                if ((unsigned)id >= (unsigned)nE) {
-                    flag_index_error();
-                } else {
-                    my_slot = id / Kc;
-                    my_w = __ldg(prob + id);
+            const bool bad = take(c0);
+            const int n = min(32, deg - c0);
+            int q = 0;
+            constexpr int kBatch = 4;
+            if (!bad) {
+                for (; q + kBatch <= n; q += kBatch) {
+                    float4 v0[kBatch], v1[kBatch];
+                    float wt[kBatch];
+#pragma unroll
+                    for (int u = 0; u < kBatch; ++u) {
+                        const float* row = base + (long long)__shfl_sync(0xffffffffu, my_slot, q + u) * B;
+                        wt[u] = __shfl_sync(0xffffffffu, my_w, q + u);
+                        v0[u] = ldg4r(row);
+                        v1[u] = ldg4r(row + second);
+                    }
+#pragma unroll
+                    for (int u = 0; u < kBatch; ++u) {
+                        add(a0, wt[u], v0[u]);
+                        add(a1, wt[u], v1[u]);
+                    }
                 }
             }
+            for (; q < n; ++q) {
+                const int slot = __shfl_sync(0xffffffffu, my_slot, q);
+                const float w = __shfl_sync(0xffffffffu, my_w, q);
+                if (slot >= 0) {
+                    const float* row = base + (long long)slot * B;
+                    const float4 v0 = ldg4r(row), v1 = ldg4r(row + second);
+                    add(a0, w, v0);
+                    add(a1, w, v1);
+                }
+            }
+        }
+        float* out = dX + (long long)i * B + s;
+        if (in0) *reinterpret_cast<float4*>(out) = a0;
+        if (in1) *reinterpret_cast<float4*>(out + 128) = a1;
+    } else {
+        const bool in = s < B;
+        float acc = 0.f;
+        constexpr int kBatch = 8;
+        for (int c0 = 0; c0 < deg; c0 += 32) {
+            take(c0);
             const int n = min(32, deg - c0);
             for (int q0 = 0; q0 < n; q0 += kBatch) {
                 int slot[kBatch];
-                float wt[kBatch];
+                float wt[kBatch], v[kBatch];
 #pragma unroll
                 for (int u = 0; u < kBatch; ++u) {
                     slot[u] = __shfl_sync(0xffffffffu, my_slot, (q0 + u) & 31);
                     wt[u] = __shfl_sync(0xffffffffu, my_w, (q0 + u) & 31);
                     if (q0 + u >= n) slot[u] = -1;
                 }
-                if constexpr (VEC) {
-                    float4 v[kBatch];
 #pragma unroll
-                    for (int u = 0; u < kBatch; ++u)
-                        v[u] = (in && slot[u] >= 0) ? ldg4r(G + (long long)slot[u] * B + s)
-                                                    : make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int u = 0; u < kBatch; ++u)
+                    v[u] = (in && slot[u] >= 0) ? __ldg(G + (long long)slot[u] * B + s) : 0.f;
 #pragma unroll
-                    for (int u = 0; u < kBatch; ++u) {
-                        if (q0 + u < n) {
-                            acc.x = fmaf(wt[u], v[u].x, acc.x);
-                            acc.y = fmaf(wt[u], v[u].y, acc.y);
-                            acc.z = fmaf(wt[u], v[u].z, acc.z);
-                            acc.w = fmaf(wt[u], v[u].w, acc.w);
-                        }
-                    }
-                } else {
-                    float v[kBatch];
-#pragma unroll
-                    for (int u = 0; u < kBatch; ++u)
-                        v[u] = (in && slot[u] >= 0) ? __ldg(G + (long long)slot[u] * B + s) : 0.f;
-#pragma unroll
-                    for (int u = 0; u < kBatch; ++u)
-                        if (q0 + u < n) acc = fmaf(wt[u], v[u], acc);
-                }
+                for (int u = 0; u < kBatch; ++u)
+                    if (q0 + u < n) acc = fmaf(wt[u], v[u], acc);
             }
         }
-    };
-    if constexpr (VEC) {
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        accumulate(acc);
-        if (in) *reinterpret_cast<float4*>(dX + (long long)i * B + s) = acc;
-    } else {
-        float acc = 0.f;
-        accumulate(acc);
         if (in) dX[(long long)i * B + s] = acc;
     }
 }
@@ -507,7 +557,7 @@ extern "C" int bitlogic_route_backward(const float* X, int32_t w_in, int64_t B, 
     if (st || !dX) return st;
     const int nE = slots * Kc;
     const bool vx = (B % 4 == 0) && aligned16(G) && aligned16(dX);
-    const long long per_block = vx ? 128 : 32;
+    const long long per_block = vx ? 256 : 32;
     const long long gy = (B + per_block - 1) / per_block;
     if (gy > 65535) return BITLOGIC_ERR_SHAPE;
     dim3 grid((unsigned)((w_in + kRdxWarps - 1) / kRdxWarps), (unsigned)gy);
