@@ -800,23 +800,26 @@ long long hard_word_chunk(int w_in, long long W) {
 constexpr long long kStagedMinWords = BITLOGIC_HARD_STAGED_MIN;
 
 // Splits of a class for the staged head when there are few word groups: the
-// grid is then a few waves of blocks, and what counts is their number times a
-// block's time, its nodes per warp plus the flush of its counters (about
-// kHeadFlush nodes' worth).  Any number of splits that leaves a warp at least
-// four nodes.
-#ifndef BITLOGIC_HEAD_FLUSH
-#define BITLOGIC_HEAD_FLUSH 12
-#endif
-constexpr int kHeadFlush = BITLOGIC_HEAD_FLUSH, kHeadFewGroups = 16;
-int head_splits(int g, int C, long long wg) {
+// grid is then a few waves of blocks.  Least estimated time over all splits
+// that leave a warp at least four nodes, in instructions of a warp: waves x
+// (nodes per warp x a node's instructions + those of staging the slice and
+// flushing the counters), and what every further split costs in atomic adds
+// to the same counts.  10000 samples through 64000 nodes of fan-in 6, 10
+// classes: 20 splits (2 full waves) against 16, pass 273 -> 254 us; 1500
+// samples, 58080 nodes of fan-in 2 45.5 -> 39.3 us; without the last term 2807
+// samples, 17350 nodes of fan-in 2 took 30 splits, 28.0 us against 26.6 us
+// with 16.
+constexpr int kHeadFewGroups = 16;
+int head_splits(int k, int g, int C, long long wg) {
     const long long slots = (long long)kHeadMinBlocks * sm_count();
+    const long long node = 4 * ((1 << k) - 1) + 60 + 4 * k, fixed = 4000, split = 72;
     int best = 1;
     long long best_cost = -1;
     for (int s = 1; s == 1 || (g / s >= 4 * kHSWarps && (long long)C * s * wg <= 8 * slots); ++s) {
         const int per = (g + s - 1) / s;
         if (per > kHeadSliceNodes) continue;
         const long long waves = ((long long)C * s * wg + slots - 1) / slots;
-        const long long cost = waves * ((per + kHSWarps - 1) / kHSWarps + kHeadFlush);
+        const long long cost = waves * ((per + kHSWarps - 1) / kHSWarps * node + fixed) + s * split;
         if (best_cost < 0 || cost < best_cost) {
             best_cost = cost;
             best = s;
@@ -880,7 +883,7 @@ int launch_hard(const uint32_t* xp, int w_in, long long N, const int* conn, cons
         // see head_splits
         int splits = 1;
         if (wg < kHeadFewGroups) {
-            splits = head_splits(g, C, wg);
+            splits = head_splits(k, g, C, wg);
         } else {
             while (C * splits < sm_count() && g / (splits * 2) >= 8 * kHSWarps) splits *= 2;
         }
