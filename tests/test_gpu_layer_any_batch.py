@@ -1,7 +1,7 @@
 """GPU parity of the fp32 layer kernels on batches that are no multiple of
 four and on rows off a 16-byte boundary: forward, backward with per-edge
 terms (from rows and from upstream terms, at given positions) and the CSR
-reduction, around the 32- and 128-sample edges of their stages."""
+reduction, around the 32- and 128-sample edges of their stages, and the head's group sums likewise."""
 import os
 
 import numpy as np
@@ -31,7 +31,7 @@ def off_boundary(a, offset):
 
 
 @pytest.mark.parametrize("k", [3, 4, 5, 6])
-@pytest.mark.parametrize("B,offset", [(1, 0), (31, 0), (33, 0), (127, 0), (129, 0), (258, 0), (515, 0), (128, 1), (260, 3)])
+@pytest.mark.parametrize("B,offset", [(1, 0), (31, 0), (33, 0), (127, 0), (129, 0), (258, 0), (515, 0), (1030, 0), (128, 1), (260, 3)])
 @pytest.mark.parametrize("node", ["soft", "st"])
 def test_layer_on_any_batch(k, B, offset, node):
     w_in, w = 40, 70
@@ -64,4 +64,22 @@ def test_layer_on_any_batch(k, B, offset, node):
                                   up_off=dev(np.arange(w + 1, dtype=np.int32)), edge_terms=P_t, edge_pos=dev(pos))
     check_exact(dth_t.cpu().numpy(), dth.cpu().numpy(), "dtheta from terms")
     check_exact(P_t.cpu().numpy(), P.cpu().numpy(), "edge terms from terms")
+    assert bl.bitlogic_device_error() == 0
+
+
+@pytest.mark.parametrize("C,g,B,offset", [(10, 64, 1, 0), (10, 129, 127, 0), (1, 257, 131, 0), (10, 513, 158, 0),
+                                          (100, 90, 907, 0), (3, 1025, 256, 1)])
+def test_head_on_any_batch(C, g, B, offset):
+    rng = np.random.default_rng(C + B)
+    Y = rng.random((C * g, B)).astype(np.float32)
+    labels = rng.integers(0, C, size=B).astype(np.int32)
+    loss = torch.zeros(1, device="cuda")
+    logits = torch.full((B, C), np.nan, device="cuda")
+    dY = torch.full((C * g, B), np.nan, device="cuda")
+    ws = torch.empty(bl.bitlogic_head_loss_workspace(B, C), dtype=torch.uint8, device="cuda")
+    bl.bitlogic_head_loss(off_boundary(Y, offset), dev(labels), C, 20.0, loss, ws, logits=logits, dY=dY)
+    wl, wloss, wdy = oracle.head_loss(Y.astype(np.float64), labels, C, 20.0)
+    check_fwd(logits, wl, "logits")
+    check_fwd(loss, np.array([wloss]), "loss")
+    check_grad(dY, wdy, "dY")
     assert bl.bitlogic_device_error() == 0
