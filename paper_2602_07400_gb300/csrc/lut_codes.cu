@@ -668,19 +668,23 @@ coded_backward_kernel(const uint8_t* __restrict__ codes, long long stride, const
 // --------------------------------------------------- layer 1 table gradient --
 
 // dtheta[j][a] = slope(theta_j[a]) * sum of the corner sums H[edge[p]][a] over
-// the CSR positions p of node j, in increasing p.  A warp per node, lane =
-// table entry (two neighbours per lane for 64 entries).  The rows of up to
-// eight positions and the logits are in flight together: the kernel reads each
-// byte once and is bound by the latency of its two dependent loads at small
-// widths, by DRAM at large ones.
-template <bool WIDE>   // 64 entries
+// the CSR positions p of node j.  `parts` warps of a block per node, each over
+// a run of its positions in increasing p, then the runs in order; lane = table
+// entry (two neighbours per lane for 64 entries).  The rows of up to eight
+// positions and the logits are in flight together: the kernel reads each byte
+// once and is bound by the latency of its two dependent loads at small widths,
+// by DRAM at large ones.
+template <bool WIDE, bool SPLIT>   // 64 entries; several parts per node
 __global__ void __launch_bounds__(256)
 corner_reduce_kernel(const float* __restrict__ corner, const int* __restrict__ off, const int* __restrict__ edge,
-                     int n_edges, const float* __restrict__ theta, int w, int k, float* __restrict__ dtheta) {
+                     int n_edges, const float* __restrict__ theta, int w, int k, int parts,
+                     float* __restrict__ dtheta) {
     constexpr int kRows = 8;
-    const int lane = threadIdx.x & 31, K = 1 << k;
-    const int j = blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (j >= w) return;   // warp-uniform
+    __shared__ float2 run[SPLIT ? 8 : 1][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, K = 1 << k;
+    const int at = SPLIT ? blockIdx.x * (8 / parts) + warp / parts : blockIdx.x * 8 + warp;
+    if (!SPLIT && at >= w) return;   // warp-uniform
+    const int j = SPLIT ? min(at, w - 1) : at;   // past the end: the last node once more, not written
     int e0 = __ldg(off + j), e1 = __ldg(off + j + 1);
     const long long o = (long long)j * K + (WIDE ? 2 * lane : lane);
     const bool in = WIDE || lane < K;
@@ -690,6 +694,11 @@ corner_reduce_kernel(const float* __restrict__ corner, const int* __restrict__ o
     if (e0 < 0 || e1 < e0 || e1 > n_edges) {
         if (lane == 0) flag_index_error();
         e0 = e1 = 0;
+    }
+    if constexpr (SPLIT) {
+        const int len = (e1 - e0 + parts - 1) / parts;
+        e0 = min(e0 + warp % parts * len, e1);
+        e1 = min(e0 + len, e1);
     }
     float2 s = make_float2(0.f, 0.f);
     for (int q = e0; q < e1; q += kRows) {
@@ -712,6 +721,15 @@ corner_reduce_kernel(const float* __restrict__ corner, const int* __restrict__ o
         for (int r = 0; r < kRows; ++r) {
             s.x += v[r].x;
             s.y += v[r].y;
+        }
+    }
+    if constexpr (SPLIT) {
+        run[warp][lane] = s;
+        __syncthreads();
+        if (warp % parts != 0 || at >= w) return;
+        for (int r = 1; r < parts; ++r) {
+            s.x += run[warp + r][lane].x;
+            s.y += run[warp + r][lane].y;
         }
     }
     const float t0 = sigmoidf(th.x), t1 = sigmoidf(th.y);
@@ -866,7 +884,16 @@ extern "C" int bitlogic_corner_reduce(const float* corner_sums, const int32_t* c
     if (wide && ((reinterpret_cast<uintptr_t>(corner_sums) | reinterpret_cast<uintptr_t>(theta) |
                   reinterpret_cast<uintptr_t>(dtheta)) & 7u) != 0)
         return BITLOGIC_ERR_ALIGN;
-    auto kern = wide ? corner_reduce_kernel<true> : corner_reduce_kernel<false>;
-    kern<<<(unsigned)((w + 7) / 8), 256, 0, stream>>>(corner_sums, csr_off, csr_edge, n_edges, theta, w, k, dtheta);
+    // more warps per node while they all fit one wave and keep four positions
+    // each on average: few nodes with many readers are bound by the chain of
+    // their rows (training steps of fan-in 6: 1015 and 9110 nodes at 68 samples
+    // 81 -> 69 us; 1015 and 20000 at 1024 samples 386 -> 362 us; fan-in 5, 500
+    // and 50000 at 200 samples 349 -> 233 us)
+    int parts = 1;
+    while (parts < 8 && 2ll * parts * w <= 64ll * sm_count() && n_edges / (2ll * parts * w) >= 4) parts *= 2;
+    auto kern = parts > 1 ? (wide ? corner_reduce_kernel<true, true> : corner_reduce_kernel<false, true>)
+                          : (wide ? corner_reduce_kernel<true, false> : corner_reduce_kernel<false, false>);
+    kern<<<(unsigned)((w * (long long)parts + 7) / 8), 256, 0, stream>>>(corner_sums, csr_off, csr_edge, n_edges, theta,
+                                                                       w, k, parts, dtheta);
     return launch_status();
 }

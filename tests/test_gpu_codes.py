@@ -173,3 +173,35 @@ def test_ragged_batch_refuses_other_binary_wires():
             TrainStep(net, 37, wl.d, wl.thresholds, wl.classes, wl.tau, **kw)
     st = TrainStep(net, 37, wl.d, wl.thresholds, wl.classes, wl.tau, codes1=False)
     assert not st.codes1 and not st.bytes1 and st.bits.dtype == torch.float32
+
+
+@pytest.mark.parametrize("k1", [1, 4, 6])
+@pytest.mark.parametrize("w,deg", [(1, 4), (5, 8), (3, 63), (7, 32), (13, 100), (2500, 9)])
+def test_corner_reduce_with_few_nodes(k1, w, deg):
+    # several warps per node: runs of unequal length, nodes without a reader
+    rng = np.random.default_rng(w + deg)
+    n, K = w * deg, 1 << k1
+    owner = np.sort(rng.integers(0, w, size=n))
+    if w > 2:
+        owner[owner == 1] = 0
+    off = np.searchsorted(owner, np.arange(w + 1)).astype(np.int32)
+    H = rng.standard_normal((n, K), dtype=np.float32)
+    theta = synth.table_logits(w, K, seed=2)
+    total = np.zeros((w, K))
+    np.add.at(total, owner, H.astype(np.float64))
+    size = np.zeros((w, K))
+    np.add.at(size, owner, np.abs(H).astype(np.float64))
+    s = 1.0 / (1.0 + np.exp(-theta.astype(np.float64)))
+    perm = rng.permutation(n).astype(np.int32)
+    shuffled = np.empty_like(H)
+    shuffled[perm] = H
+    outs = []
+    for rows, edge in ((H, None), (shuffled, dev(perm))):
+        d = torch.full((w, K), np.nan, device="cuda")
+        bl.bitlogic_corner_reduce(dev(rows), dev(off), edge, dev(theta), d)
+        outs.append(d.cpu().numpy())
+    check_exact(outs[1], outs[0], "with an edge map")
+    # fp32 sums of m terms: error below m 2^-24 of the terms' magnitudes
+    bound = s * (1 - s) * (size * (deg * 8 + 8) * 2.0 ** -24 + 2.0 ** -20 * np.abs(total)) + 1e-30
+    assert np.all(np.abs(outs[0] - s * (1 - s) * total) <= bound)
+    assert bl.bitlogic_device_error() == 0
