@@ -1010,19 +1010,31 @@ lut_backward_theta_kernel(const float* __restrict__ X, int w_in, long long B,
 // slots of blocks and warps, and a fixed eight left up to seven of them idle
 // (8000 rows of 16000 nodes, layer backward and forward: fan-in 4, 47 samples
 // 57 -> 36 us, 245 samples 80 -> 62 us; fan-in 2, 64 samples 45 -> 33 us; one
-// sample per lane instead: 245 samples 73 us).
+// sample per lane instead: 245 samples 73 us).  SPLIT: `parts` times as many
+// warps, each group over a run of the row's positions in increasing order,
+// then the runs in order, for few rows with many terms, where the chain of a
+// row's loads bounds the kernel.
 constexpr int kCsrWarps = 8;
 
-template <bool VEC>
+template <bool VEC, bool SPLIT>
 __global__ void __launch_bounds__(kCsrWarps * 32)
 csr_reduce_kernel(const float* __restrict__ P, long long B, const int* __restrict__ off,
-                  const int* __restrict__ edge, int w_in, int nE, float* __restrict__ dX) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+                  const int* __restrict__ edge, int w_in, int nE, int parts, float* __restrict__ dX) {
+    __shared__ float4 run[SPLIT ? kCsrWarps : 1][32];
+    const int lane = threadIdx.x & 31;
+    const int warps = (blockDim.x >> 5) / (SPLIT ? parts : 1);   // over the batch
+    const int part = SPLIT ? (threadIdx.x >> 5) / warps : 0;
+    const int warp = (threadIdx.x >> 5) - part * warps;
     const int i = blockIdx.x;
     int e0 = __ldg(off + i), e1 = __ldg(off + i + 1);
     if (e0 < 0 || e1 < e0 || e1 > nE) {
         if (threadIdx.x == 0) flag_index_error();
         e0 = e1 = 0;
+    }
+    if constexpr (SPLIT) {
+        const int len = (e1 - e0 + parts - 1) / parts;
+        e0 = min(e0 + part * len, e1);
+        e1 = min(e0 + len, e1);
     }
     const int deg = e1 - e0;
     int my_id = -1;   // ids of the first 32 positions, -1 when out of range
@@ -1042,7 +1054,7 @@ csr_reduce_kernel(const float* __restrict__ P, long long B, const int* __restric
         }
         return id;
     };
-    const long long s = ((long long)blockIdx.y * (blockDim.x >> 5) + warp) * 128 + (VEC ? 4 : 1) * lane;
+    const long long s = ((long long)blockIdx.y * warps + warp) * 128 + (VEC ? 4 : 1) * lane;
     bool in[4];   // VEC: B % 4 == 0, all four samples in range or none
 #pragma unroll
     for (int c = 0; c < 4; ++c) in[c] = s + (VEC ? 0 : 32 * c) < B;
@@ -1072,6 +1084,12 @@ csr_reduce_kernel(const float* __restrict__ P, long long B, const int* __restric
 #pragma unroll
         for (int u = 0; u < kCsrBatch; ++u)
             if (q0 + u < deg) acc = add4(acc, v[u]);
+    }
+    if constexpr (SPLIT) {
+        run[threadIdx.x >> 5][lane] = acc;
+        __syncthreads();
+        if (part != 0) return;
+        for (int r = 1; r < parts; ++r) acc = add4(acc, run[r * warps + warp][lane]);
     }
     if constexpr (VEC) {
         if (in[0]) *reinterpret_cast<float4*>(out) = acc;
@@ -1301,10 +1319,18 @@ extern "C" int bitlogic_csr_reduce(const float* edge_terms, int64_t B, const int
     const long long gy = (B + per_block - 1) / per_block;
     if (gy > 65535) return BITLOGIC_ERR_SHAPE;
     dim3 grid((unsigned)w_in, (unsigned)gy);
-    if (vec)
-        csr_reduce_kernel<true><<<grid, warps * 32, 0, stream>>>(edge_terms, B, csr_off, csr_edge, w_in, n_edges, dX);
-    else
-        csr_reduce_kernel<false><<<grid, warps * 32, 0, stream>>>(edge_terms, B, csr_off, csr_edge, w_in, n_edges, dX);
+    // more warps per row while the block holds them, they all fit one wave and
+    // keep 16 terms each on average (layer forward and backward: 64000 nodes of
+    // fan-in 6 over 500 rows, 32 samples 409 -> 191 us; 20000 of fan-in 3 over
+    // 600, 500 samples 125 -> 91 us; with eight terms each, 16000 of fan-in 2
+    // over 2000, 200 samples 37.2 -> 38.9 us)
+    int parts = 1;
+    while (2 * parts * warps <= kCsrWarps && 2ll * parts * warps * w_in <= 64ll * sm_count() &&
+           n_edges / (2ll * parts * w_in) >= 16)
+        parts *= 2;
+    auto kern = parts > 1 ? (vec ? csr_reduce_kernel<true, true> : csr_reduce_kernel<false, true>)
+                          : (vec ? csr_reduce_kernel<true, false> : csr_reduce_kernel<false, false>);
+    kern<<<grid, warps * parts * 32, 0, stream>>>(edge_terms, B, csr_off, csr_edge, w_in, n_edges, parts, dX);
     return launch_status();
 }
 

@@ -83,3 +83,32 @@ def test_head_on_any_batch(C, g, B, offset):
     check_fwd(loss, np.array([wloss]), "loss")
     check_grad(dY, wdy, "dY")
     assert bl.bitlogic_device_error() == 0
+
+
+@pytest.mark.parametrize("w_in,deg", [(1, 32), (3, 63), (7, 500), (900, 33)])
+@pytest.mark.parametrize("B,offset", [(1, 0), (4, 0), (130, 0), (256, 0), (300, 1), (515, 0)])
+def test_csr_reduce_of_few_rows(w_in, deg, B, offset):
+    # several warps per row: runs of unequal length, rows without a term
+    rng = np.random.default_rng(w_in + deg + B)
+    n = w_in * deg
+    owner = np.sort(rng.integers(0, w_in, size=n))
+    if w_in > 2:
+        owner[owner == 1] = 0
+    csr_off = np.searchsorted(owner, np.arange(w_in + 1)).astype(np.int32)
+    P = rng.standard_normal((n, B), dtype=np.float32)
+    total, size = np.zeros((w_in, B)), np.zeros((w_in, B))
+    np.add.at(total, owner, P.astype(np.float64))
+    np.add.at(size, owner, np.abs(P).astype(np.float64))
+    perm = rng.permutation(n).astype(np.int32)
+    shuffled = np.empty_like(P)
+    shuffled[perm] = P
+    outs = []
+    for rows, edge in ((P, None), (shuffled, dev(perm))):
+        dX = torch.full((w_in, B), np.nan, device="cuda")
+        bl.bitlogic_csr_reduce(off_boundary(rows, offset), dev(csr_off), edge, dX)
+        outs.append(dX.cpu().numpy())
+    check_exact(outs[1], outs[0], "with an edge map")
+    # fp32 sums of m terms: error below m 2^-24 of the terms' magnitudes
+    m = np.diff(csr_off)[:, None] + 8
+    assert np.all(np.abs(outs[0] - total) <= size * m * 2.0 ** -24)
+    assert bl.bitlogic_device_error() == 0
