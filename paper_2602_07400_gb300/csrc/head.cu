@@ -23,66 +23,99 @@
 namespace bitlogic {
 namespace {
 
-// One block of 16 warps per (class, row split, 128 samples), four samples per
-// lane (VEC, B % 4 == 0 and 16-byte aligned Y: consecutive ones in 16-byte
-// loads; otherwise 32 apart).  Warp r sums rows r, r + 16, ... of the split,
-// then thread t adds the warps' partial sums of sample t in order.  With one
-// split the block writes the logits; with several (so that enough blocks pull
-// from HBM) it writes the split's sum, and the softmax kernel adds the splits
-// in order.  Bound by HBM reads once the grid fills the chip, by their latency
-// below that.  The unaligned form used to be one of 8 warps x 32 samples without
-// splits: a step of 8000 and 20000 nodes of fan-in 2 at 63 samples 77.6 ->
-// 61.0 us, at 907 samples 230.8 -> 205.7 us.
-constexpr int kSumWarps = 16;
-constexpr int kMaxRowSplits = 4;
+// Any B and alignment: one block per (class, 32 samples), lane = sample, warp r
+// sums rows r, r + 8, ... in order, then the warps' sums are added in order.
+// The loads of 32 rows are in flight together: with few classes and small
+// batches the chain of loads bounds the kernel (a step of 8000 and 20000 nodes
+// of fan-in 2: 63 samples 77.9 -> 65.0 us, 907 samples 231 -> 211 us against
+// four rows; a range check before each load makes it slower than that).
+// Splitting a class over blocks as below gives 61.4 and 206 us, but adds in
+// another order, and thousands of rows in one chain round by up to 2e-5 of
+// their sum, so the logits would move by as much.
+constexpr int kSumWarps = 8;
+constexpr int kSumRows = 32, kTailRows = 8;
 
-template <bool VEC>
 __global__ void __launch_bounds__(kSumWarps * 32)
 head_group_sum_kernel(const float* __restrict__ Y, long long B, int C, int g, float tau,
-                      float* __restrict__ logits, float* __restrict__ split_sums, int splits,
-                      int rows_per_split, unsigned int* __restrict__ done) {
-    __shared__ __align__(16) float part[kSumWarps][128];
+                      float* __restrict__ logits, unsigned int* __restrict__ done) {
+    __shared__ float part[kSumWarps][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    dependent_kernel_start();
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *done = 0u;   // the softmax's block count
+    const int c = blockIdx.x;
+    const long long s = (long long)blockIdx.y * 32 + lane;
+    float acc = 0.f;
+    if (s < B) {
+        const float* base = Y + (long long)c * g * B + s;
+        int r = warp;
+        for (; r < g - (kSumRows - 1) * kSumWarps; r += kSumRows * kSumWarps) {
+            float v[kSumRows];
+#pragma unroll
+            for (int u = 0; u < kSumRows; ++u) v[u] = __ldg(base + (long long)(r + u * kSumWarps) * B);
+#pragma unroll
+            for (int u = 0; u < kSumRows; ++u) acc += v[u];
+        }
+        for (; r < g; r += kTailRows * kSumWarps) {   // loads past the end read the last row again, not added
+            float v[kTailRows];
+#pragma unroll
+            for (int u = 0; u < kTailRows; ++u) v[u] = __ldg(base + (long long)min(r + u * kSumWarps, g - 1) * B);
+#pragma unroll
+            for (int u = 0; u < kTailRows; ++u)
+                if (r + u * kSumWarps < g) acc += v[u];
+        }
+    }
+    part[warp][lane] = acc;
+    __syncthreads();
+    if (warp == 0 && s < B) {
+        float t = 0.f;
+#pragma unroll
+        for (int q = 0; q < kSumWarps; ++q) t += part[q][lane];
+        logits[s * C + c] = t / tau;
+    }
+}
+
+// Vector form (B % 4 == 0, 16-byte aligned Y): one block of 32 warps per
+// (class, row split, 128 samples), lane = 4 consecutive samples, warp r sums
+// rows r, r + 32, ... of the split with 16-byte loads, then thread t adds the
+// 32 warps' partial sums of sample t in order.  With one split the block
+// writes the logits; with several (so that enough blocks pull from HBM) it
+// writes the split's sum, and the softmax kernel adds the splits in order.
+#ifndef BITLOGIC_SUM_VEC_WARPS
+#define BITLOGIC_SUM_VEC_WARPS 16
+#endif
+constexpr int kSumVecWarps = BITLOGIC_SUM_VEC_WARPS;
+constexpr int kMaxRowSplits = 4;
+
+__global__ void __launch_bounds__(kSumVecWarps * 32)
+head_group_sum_vec_kernel(const float* __restrict__ Y, long long B, int C, int g, float tau,
+                          float* __restrict__ logits, float* __restrict__ split_sums, int splits,
+                          int rows_per_split, unsigned int* __restrict__ done) {
+    __shared__ __align__(16) float part[kSumVecWarps][128];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     dependent_kernel_start();
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *done = 0u;   // the softmax's block count
     const int c = blockIdx.x / splits, rs = blockIdx.x - c * splits;
     const int r0 = rs * rows_per_split, r1 = min(g, r0 + rows_per_split);
-    const long long s0 = (long long)blockIdx.y * 128 + (VEC ? 4 : 1) * lane;
-    const float* base = Y + (long long)c * g * B + s0;
-    if constexpr (VEC) {
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (s0 < B) {   // B % 4 == 0: all four samples are in range
+    const long long s4 = (long long)blockIdx.y * 128 + 4 * lane;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (s4 < B) {   // B % 4 == 0: all four samples are in range
+        const float* base = Y + (long long)c * g * B + s4;
 #pragma unroll 4
-            for (int r = r0 + warp; r < r1; r += kSumWarps) {
-                const float4 v = __ldg(reinterpret_cast<const float4*>(base + (long long)r * B));
-                acc.x += v.x;
-                acc.y += v.y;
-                acc.z += v.z;
-                acc.w += v.w;
-            }
+        for (int r = r0 + warp; r < r1; r += kSumVecWarps) {
+            const float4 v = __ldg(reinterpret_cast<const float4*>(base + (long long)r * B));
+            acc.x += v.x;
+            acc.y += v.y;
+            acc.z += v.z;
+            acc.w += v.w;
         }
-        *reinterpret_cast<float4*>(&part[warp][4 * lane]) = acc;
-    } else {
-        float acc[4] = {};
-        bool in[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) in[q] = s0 + 32 * q < B;
-#pragma unroll 4
-        for (int r = r0 + warp; r < r1; r += kSumWarps) {
-            const float* row = base + (long long)r * B;
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (in[q]) acc[q] += __ldg(row + 32 * q);
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) part[warp][32 * q + lane] = acc[q];
     }
+    *reinterpret_cast<float4*>(&part[warp][4 * lane]) = acc;
     __syncthreads();
     if (threadIdx.x < 128) {
         const long long s = (long long)blockIdx.y * 128 + threadIdx.x;
         float t = 0.f;
 #pragma unroll 8
-        for (int q = 0; q < kSumWarps; ++q) t += part[q][threadIdx.x];
+        for (int q = 0; q < kSumVecWarps; ++q) t += part[q][threadIdx.x];
         if (s < B) {
             if (splits == 1) logits[s * C + c] = t / tau;
             else split_sums[((long long)rs * B + s) * C + c] = t;
@@ -293,19 +326,24 @@ extern "C" int bitlogic_head_loss_ex(const float* Y, int32_t w, int64_t B, int32
     float* split_sums = reinterpret_cast<float*>(ws + align_up(bc) + align_up((size_t)B * 4) + align_up(bc));
     unsigned int* done = reinterpret_cast<unsigned int*>(ws + align_up(bc) + align_up((size_t)B * 4) + align_up(bc) +
                                                          align_up(kMaxRowSplits * bc));
-    // split the rows of a class while the doubled grid still fits one wave of
-    // resident blocks, keeping at least 4 rows per warp
     int splits = 1;
-    const long long nsb = (B + 127) / 128;
-    const long long resident = (long long)(2048 / (kSumWarps * 32)) * sm_count();
-    while (splits < kMaxRowSplits && (long long)C * (2 * splits) * nsb <= resident &&
-           g / (2 * splits) >= 4 * kSumWarps)
-        splits *= 2;
-    const int rows_per_split = (g + splits - 1) / splits;
-    if ((long long)C * splits > 0x7fffffffll) return BITLOGIC_ERR_SHAPE;
-    auto sum = B % 4 == 0 && aligned16(Y) ? head_group_sum_kernel<true> : head_group_sum_kernel<false>;
-    (void)launch_dependent(sum, dim3((unsigned)(C * splits), (unsigned)nsb), kSumWarps * 32, 0, stream, Y, B, C, g,
-                           tau, lg, split_sums, splits, rows_per_split, done);
+
+    if (B % 4 == 0 && aligned16(Y)) {
+        // split the rows of a class while the doubled grid still fits one
+        // wave of resident blocks, keeping at least 4 rows per warp
+        const long long nsb = (B + 127) / 128;
+        const long long resident = (long long)(2048 / (kSumVecWarps * 32)) * sm_count();
+        while (splits < kMaxRowSplits && (long long)C * (2 * splits) * nsb <= resident &&
+               g / (2 * splits) >= 4 * kSumVecWarps)
+            splits *= 2;
+        const int rows_per_split = (g + splits - 1) / splits;
+        if ((long long)C * splits > 0x7fffffffll || nsb > 65535) return BITLOGIC_ERR_SHAPE;
+        (void)launch_dependent(head_group_sum_vec_kernel, dim3((unsigned)(C * splits), (unsigned)nsb),
+                               kSumVecWarps * 32, 0, stream, Y, B, C, g, tau, lg, split_sums, splits,
+                               rows_per_split, done);
+    } else
+        (void)launch_dependent(head_group_sum_kernel, dim3((unsigned)C, (unsigned)sb), kSumWarps * 32, 0, stream, Y,
+                               B, C, g, tau, lg, done);
     if (launch_status()) return BITLOGIC_ERR_CUDA;
     if (launch_dependent(head_softmax_kernel, (unsigned)((B + kSoftWarps - 1) / kSoftWarps), kSoftWarps * 32, 0,
                          stream, lg, B, C, labels, dlogit, block_sums, done, loss, tau,
