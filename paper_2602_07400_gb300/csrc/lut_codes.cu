@@ -701,28 +701,29 @@ corner_reduce_kernel(const float* __restrict__ corner, const int* __restrict__ o
         e1 = min(e0 + len, e1);
     }
     float2 s = make_float2(0.f, 0.f);
+    bool bad = false;
     for (int q = e0; q < e1; q += kRows) {
+        // no branch before a load: past the end the last position once more,
+        // for a position out of range row 0, neither added
         float2 v[kRows];
+        bool add[kRows];
 #pragma unroll
         for (int r = 0; r < kRows; ++r) {
-            v[r] = make_float2(0.f, 0.f);
-            if (q + r < e1) {
-                const int id = edge ? __ldg(edge + q + r) : q + r;
-                if ((unsigned)id >= (unsigned)n_edges) {
-                    if (lane == 0) flag_index_error();
-                } else {
-                    const float* row = corner + ((long long)id << k);
-                    if constexpr (WIDE) v[r] = __ldcs(reinterpret_cast<const float2*>(row) + lane);
-                    else if (in) v[r].x = __ldcs(row + lane);
-                }
-            }
+            const int at_q = min(q + r, e1 - 1), id = edge ? __ldg(edge + at_q) : at_q;
+            const bool ok = (unsigned)id < (unsigned)n_edges;
+            add[r] = ok && q + r < e1;
+            bad |= !ok;
+            const float* row = corner + ((long long)(ok ? id : 0) << k);
+            if constexpr (WIDE) v[r] = __ldcs(reinterpret_cast<const float2*>(row) + lane);
+            else v[r] = make_float2(__ldcs(row + (lane & (K - 1))), 0.f);
         }
 #pragma unroll
         for (int r = 0; r < kRows; ++r) {
-            s.x += v[r].x;
-            s.y += v[r].y;
+            s.x += add[r] ? v[r].x : 0.f;
+            if constexpr (WIDE) s.y += add[r] ? v[r].y : 0.f;
         }
     }
+    if (bad && lane == 0) flag_index_error();
     if constexpr (SPLIT) {
         run[warp][lane] = s;
         __syncthreads();
