@@ -21,6 +21,8 @@
 // Codes are stored as 4 a (the byte offset into an fp32 table), rows padded
 // with zeros to whole 128-sample blocks.  Readers mask them to the offsets of
 // a table of 2^k1 entries, so no byte value leads outside it.
+#include <type_traits>
+
 #include "common.cuh"
 #include "packed.cuh"
 
@@ -442,13 +444,23 @@ constexpr int coded_bwd_smem() {
     return (Order<k>::kArrays * 64 * 32 + k * 64) * (int)sizeof(float);
 }
 
-template <int k, bool TAIL>
+// Samples past the batch in the last stage have a zero output gradient and
+// code 0 (the rows' padding), so their terms are zeros, unless the node's
+// table or entry 0 of an input table is NaN (a NaN logit): for such a node
+// they take the codes of the batch's last sample instead, whose own terms are
+// NaN wherever theirs are, so that a NaN reaches only the sums of samples that
+// meet it.  FORM: whole stages (no such samples), the last stage partly
+// filled, or short_tail.
+enum { kWhole, kRagged, kShort };
+
+template <int k, int FORM>
 __global__ void __launch_bounds__(32, coded_bwd_blocks<k>())
 coded_backward_kernel(const uint8_t* __restrict__ codes, long long stride, const float* __restrict__ table1, int w_in,
                       int k1, long long B, const int* __restrict__ conn, const float* __restrict__ theta, int w,
                       int node, const float* __restrict__ dY, int group, bool vec, float* __restrict__ dtheta,
                       float* __restrict__ corner, const int* __restrict__ epos) {
     using O = Order<k>;
+    constexpr bool TAIL = FORM == kShort;
     constexpr int C = O::C, K = O::K, H = O::H;
     constexpr int NF = K >= 32 ? K / 32 : 1;
     extern __shared__ __align__(256) float smem[];
@@ -527,6 +539,25 @@ coded_backward_kernel(const uint8_t* __restrict__ codes, long long stride, const
             x[m] = lds(ea[m] + table_off(m));
         }
     };
+    // the codes of the last sample for those past the batch, once cw holds the
+    // last stage's, and their first lookup again
+    auto fill = [&] {
+        const int last = (int)(B - 1 - 128ll * (nst - 1)), nc = TAIL ? tail.nc : 4;
+        const int part = (last & 3) >> (TAIL ? nc - 1 : 2);   // nc 1 or 2 with TAIL
+        const int owner = (last >> 2) + part * (8 * nc), r = last & (nc - 1);   // its lane and byte there
+        const bool past = (TAIL ? tail.at : 4 * lane) + nc > last;
+        const int from = past ? owner : lane;
+        const uint32_t bytes = !past || r == 3 ? 0x3210u : r == 2 ? 0x2210u : r == 1 ? 0x1110u : 0u;
+        uint32_t v[k];   // by slot: the two lane halves hold the slots in different orders
+#pragma unroll
+        for (int i = 0; i < k; ++i) {
+            v[i] = __shfl_sync(0xffffffffu, h ? cw[(i + k - C) % k] : cw[i], from);
+            v[i] = __byte_perm(v[i], 0u, bytes);
+        }
+#pragma unroll
+        for (int m = 0; m < k; ++m) cw[m] = h ? v[(m + C) % k] : v[m];
+        look(0);
+    };
     ahead(blockIdx.x);
     start(blockIdx.x);
     for (int q = lane; q < O::kArrays * 64 * 32; q += 32) smem[q] = 0.f;
@@ -558,58 +589,75 @@ coded_backward_kernel(const uint8_t* __restrict__ codes, long long stride, const
         ahead(j + G);
         cp_async_wait<0>();
         __syncwarp();
+        bool nan = false;   // among the values that samples past the batch would meet
+        if constexpr (FORM != kWhole) {
+            const float first = sTab[64 * (lane < k ? lane : 0)];
+            nan = first != first;
+#pragma unroll
+            for (int i = 0; i < NF; ++i) nan |= sg[i] != sg[i];
+            nan = __any_sync(0xffffffffu, nan);
+        }
 #pragma unroll
         for (int m = 0; m < k; ++m) cw[m] = (cw[m] & cmask) >> (TAIL && nst == 1 ? tail.shift : 0);
         look(0);
+        auto stages = [&](auto nan_met) {
 #pragma unroll 1
-        for (int st = 0; st < nst; ++st) {
-            uint32_t cn[k];
-            float4 gn;
+            for (int st = 0; st < nst; ++st) {
+                if (decltype(nan_met)::value && nan && st + 1 == nst) fill();
+                uint32_t cn[k];
+                float4 gn;
 #pragma unroll
-            for (int m = 0; m < k; ++m) cn[m] = 0u;
-            gn = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (st + 1 < nst) {
+                for (int m = 0; m < k; ++m) cn[m] = 0u;
+                gn = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (st + 1 < nst) {
 #pragma unroll
-                for (int m = 0; m < k; ++m) cn[m] = __ldg(src[m] + 32 * (st + 1) + (TAIL ? word_of(st + 1) : 0));
-                gn = load_g(st + 1);
-            }
-            // one sample: its tree, the inputs of sample `next` of the words in cw
-            // (after moving on to the next stage's words when `step`), its terms
-            // into the columns
-            auto sample = [&](float g, bool step, int next) {
-                float dx[k];
-                node_sample2<k>(cp, x, g, dx, acc);
-                uint32_t at[k];   // this sample's columns
-#pragma unroll
-                for (int m = 0; m < k; ++m) at[m] = 32u * ea[m] + cb[base(m)];
-                if (step) {   // on to the next stage
-#pragma unroll
-                    for (int m = 0; m < k; ++m) cw[m] = (cn[m] & cmask) >> (TAIL && st + 2 == nst ? tail.shift : 0);
+                    for (int m = 0; m < k; ++m) cn[m] = __ldg(src[m] + 32 * (st + 1) + (TAIL ? word_of(st + 1) : 0));
+                    gn = load_g(st + 1);
                 }
-                look(next);
+                // one sample: its tree, the inputs of sample `next` of the words in cw
+                // (after moving on to the next stage's words when `step`), its terms
+                // into the columns
+                auto sample = [&](float g, bool step, int next) {
+                    float dx[k];
+                    node_sample2<k>(cp, x, g, dx, acc);
+                    uint32_t at[k];   // this sample's columns
 #pragma unroll
-                for (int m0 = 0; m0 < k; m0 += C) {   // a step: slots m0 .. m0 + C - 1 of this lane's order
-                    float old[C];
+                    for (int m = 0; m < k; ++m) at[m] = 32u * ea[m] + cb[base(m)];
+                    if (step) {   // on to the next stage
 #pragma unroll
-                    for (int i = 0; i < C; ++i)
-                        if (m0 + i < k) old[i] = lds(at[m0 + i] + column_off(m0 + i));
+                        for (int m = 0; m < k; ++m) cw[m] = (cn[m] & cmask) >> (TAIL && st + 2 == nst ? tail.shift : 0);
+                    }
+                    look(next);
 #pragma unroll
-                    for (int i = 0; i < C; ++i)
-                        if (m0 + i < k) sts(at[m0 + i] + column_off(m0 + i), old[i] + dx[m0 + i]);
-                    __syncwarp();   // the other lane of these columns comes to them in another step
-                }
-            };
-            if (!TAIL || st + 1 < nst) {
-                sample(g4.x, false, 1);
-                sample(g4.y, false, 2);
-                sample(g4.z, false, 3);
-                sample(g4.w, true, 0);
-            } else {
+                    for (int m0 = 0; m0 < k; m0 += C) {   // a step: slots m0 .. m0 + C - 1 of this lane's order
+                        float old[C];
+#pragma unroll
+                        for (int i = 0; i < C; ++i)
+                            if (m0 + i < k) old[i] = lds(at[m0 + i] + column_off(m0 + i));
+#pragma unroll
+                        for (int i = 0; i < C; ++i)
+                            if (m0 + i < k) sts(at[m0 + i] + column_off(m0 + i), old[i] + dx[m0 + i]);
+                        __syncwarp();   // the other lane of these columns comes to them in another step
+                    }
+                };
+                if (!TAIL || st + 1 < nst) {
+                    sample(g4.x, false, 1);
+                    sample(g4.y, false, 2);
+                    sample(g4.z, false, 3);
+                    sample(g4.w, true, 0);
+                } else {
 #pragma unroll 1
-                for (int c = 0; c < tail.nc; ++c) sample(c ? g4.y : g4.x, false, c + 1);   // nc <= 2
+                    for (int c = 0; c < tail.nc; ++c) sample(c ? g4.y : g4.x, false, c + 1);   // nc <= 2
+                }
+                g4 = gn;
             }
-            g4 = gn;
-        }
+        };
+        // the check in the loop, or a loop of its own for such nodes: 8000 nodes
+        // x 907 samples, step 170 us at fan-in 6 without it, 172.6 and 173.6;
+        // 82.2 at fan-in 4, 83.9 and 81.7
+        if constexpr (k >= 6) stages(std::integral_constant<bool, FORM != kWhole>{});
+        else if (FORM != kWhole && nan) stages(std::true_type{});
+        else stages(std::false_type{});
         __syncwarp();
         if (j + G < w) start(j + G);   // the next node's loads fly during the epilogue
 
@@ -779,7 +827,9 @@ int launch_coded_backward(const uint8_t* codes, long long stride, const float* t
     // 1 KB of it per block) hold
     constexpr int fit = (228 * 1024) / (smem + 1024);
     const long long resident = (long long)sm_count() * (fit < coded_bwd_blocks<k>() ? fit : coded_bwd_blocks<k>());
-    auto kern = short_tail(B) ? coded_backward_kernel<k, true> : coded_backward_kernel<k, false>;
+    auto kern = B % 128 == 0    ? coded_backward_kernel<k, kWhole>
+                : short_tail(B) ? coded_backward_kernel<k, kShort>
+                                : coded_backward_kernel<k, kRagged>;
     kern<<<(unsigned)(w < resident ? w : resident), 32, smem, st>>>(
         codes, stride, table, w_in, k1, B, conn, theta, w, node, dY, group, B % 4 == 0 && aligned16(dY), dtheta, corner,
         epos);

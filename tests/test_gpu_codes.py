@@ -205,3 +205,43 @@ def test_corner_reduce_with_few_nodes(k1, w, deg):
     bound = s * (1 - s) * (size * (deg * 8 + 8) * 2.0 ** -24 + 2.0 ** -20 * np.abs(total)) + 1e-30
     assert np.all(np.abs(outs[0] - s * (1 - s) * total) <= bound)
     assert bl.bitlogic_device_error() == 0
+
+
+@pytest.mark.parametrize("k,k1,B", [(6, 6, 5), (6, 6, 64), (6, 5, 100), (6, 1, 131), (6, 6, 256), (6, 6, 1001), (5, 5, 200),
+                                    (5, 3, 333), (5, 6, 260), (6, 6, 1030), (4, 4, 127), (4, 2, 37), (4, 6, 190),
+                                    (4, 5, 385)])
+def test_nan_logits_reach_only_the_samples_that_select_them(k, k1, B):
+    # a table entry that no sample selects changes nothing, whatever it holds:
+    # lanes past the batch must not stand for a sample at entry 0
+    rng = np.random.default_rng(k + B)
+    w1, w, K1 = 20, 24, 1 << k1
+    a = rng.integers(0, K1, size=(w1, B))
+    a[3] = rng.integers(1, K1, size=B)
+    padded = np.zeros((w1, bl.code_bytes(B)), np.uint8)
+    padded[:, :B] = 4 * a
+    conn = synth.connectivity(w, k, w1, seed=1)
+    conn[2, 0], conn[2, 1:] = 3, np.arange(4, 3 + k)
+    theta = synth.table_logits(w, 1 << k, seed=2)
+    table = rng.random((w1, K1)).astype(np.float32)
+    dY = synth.uniform_gradients(w, B, seed=3, scale=1e-2)
+
+    def backward(table, theta):
+        dth, H = torch.empty(w, 1 << k, device="cuda"), torch.empty(w * k, K1, device="cuda")
+        bl.bitlogic_lut_backward_coded(dev(padded), dev(table), B, dev(conn), dev(theta), dth, H, dev(dY))
+        return dth.cpu().numpy(), H.cpu().numpy()
+
+    dth, H = backward(table, theta)
+    assert np.isfinite(dth).all() and np.isfinite(H).all()
+    hole = table.copy()
+    hole[3, 0] = np.nan
+    for got, want, name in zip(backward(hole, theta), (dth, H), ("dtheta", "corner sums")):
+        check_exact(got, want, name + " with an unselected NaN entry")
+    bad = theta.copy()
+    bad[2, 1] = np.nan
+    dth_b, H_b = backward(table, bad)
+    others = np.arange(w) != 2
+    check_exact(dth_b[others], dth[others], "other nodes' dtheta")
+    check_exact(H_b[np.repeat(others, k)], H[np.repeat(others, k)], "other nodes' corner sums")
+    for i in range(k):
+        unread = np.setdiff1d(np.arange(K1), a[conn[2, i]])
+        assert not H_b[2 * k + i, unread].any(), "corners that no sample is on"
