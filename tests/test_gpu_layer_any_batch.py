@@ -112,3 +112,44 @@ def test_csr_reduce_of_few_rows(w_in, deg, B, offset):
     m = np.diff(csr_off)[:, None] + 8
     assert np.all(np.abs(outs[0] - total) <= size * m * 2.0 ** -24)
     assert bl.bitlogic_device_error() == 0
+
+
+@pytest.mark.parametrize("k,w", [(3, 5000), (4, 5200), (6, 3000)])
+@pytest.mark.parametrize("B,offset", [(129, 0), (260, 0), (260, 1), (37, 0)])
+def test_backward_over_several_nodes_per_block(k, w, B, offset):
+    # more nodes than two waves of the persistent blocks: what a block carries
+    # from one node to the next (ring slots, rows, logits, positions), for the
+    # gradient from rows and summed from several upstream terms per node
+    w_in = 300
+    X = synth.uniform_activations(w_in, B, seed=B)
+    conn = synth.connectivity(w, k, w_in, seed=1)
+    theta = synth.table_logits(w, 1 << k, seed=2)
+    Xd = off_boundary(X, offset)
+    off, edge = bl.bitlogic_build_csr(conn, w_in)
+    pos = bl.bitlogic_csr_positions(edge)
+    rng = np.random.default_rng(k + B)
+    # upstream terms: 0 to 4 per node, their rows in any order
+    deg = rng.integers(0, 5, size=w)
+    up_off = np.concatenate(([0], np.cumsum(deg))).astype(np.int32)
+    n = int(up_off[-1])
+    up_edge = rng.permutation(n).astype(np.int32)
+    terms = synth.uniform_gradients(n, B, seed=4, scale=1e-2)
+    summed = np.zeros((w, B))
+    np.add.at(summed, np.repeat(np.arange(w), deg), terms[up_edge].astype(np.float64))
+    dY = synth.uniform_gradients(w // 2, B, seed=3, scale=1e-2)
+    sources = [(dict(dY=off_boundary(dY, offset), dy_group=2), np.repeat(dY, 2, axis=0).astype(np.float64)),
+               (dict(up_terms=off_boundary(terms, offset), up_off=dev(up_off), up_edge=dev(up_edge)), summed)]
+    for source, full in sources:
+        dth = torch.full((w, 1 << k), np.nan, device="cuda")
+        P = torch.full((w * k, B), np.nan, device="cuda")
+        used = torch.full((w, B), np.nan, device="cuda")
+        bl.bitlogic_lut_backward_node(Xd, dev(conn), dev(theta), dth, "soft", edge_terms=P, edge_pos=dev(pos),
+                                      dY_out=used, **source)
+        dX = torch.full((w_in, B), np.nan, device="cuda")
+        bl.bitlogic_csr_reduce(P, dev(off), None, dX)
+        wth, wdx = oracle.lut_backward(X.astype(np.float64), conn, theta, full, want_dx=True)
+        # up to four fp32 terms of at most 0.06: three roundings of at most 2^-24 x 0.24
+        check_fwd(used, full, "gradient used", atol=5e-8)
+        check_grad(dth, wth, "dtheta")
+        check_grad(dX, wdx, "dX")
+    assert bl.bitlogic_device_error() == 0
