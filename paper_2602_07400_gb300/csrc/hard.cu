@@ -799,6 +799,21 @@ long long hard_word_chunk(int w_in, long long W) {
 #endif
 constexpr long long kStagedMinWords = BITLOGIC_HARD_STAGED_MIN;
 
+// The kernels for rows of W words: 16-byte staged (W % 4 == 0, 16-byte aligned
+// rows, 32-bit offsets in 16-byte units), 4-byte staged (any other rows with
+// 32-bit offsets in words, as long as their groups of stages fit grid.y), or
+// one word per lane, which puts word groups on grid.x (head) or takes longer
+// chunks (layer) and so has no such limit.
+enum HardRoute { kOneWord = 0, kStaged4 = 1, kStaged16 = 2 };
+constexpr long long kGridY = 65535;
+HardRoute hard_route(int w_in, long long W, bool aligned, bool head) {
+    const unsigned long long rows = (unsigned long long)w_in;
+    if (W % 4 == 0 && aligned && rows * (unsigned long long)(W / 4) < (1ull << 32)) return kStaged16;
+    const long long per_y = head ? kStageWords : kLayerNS * kStageWords;
+    return W >= kStagedMinWords && rows * (unsigned long long)W < (1ull << 32) && W <= kGridY * per_y ? kStaged4
+                                                                                                  : kOneWord;
+}
+
 // Splits of a class for the staged head when there are few word groups: the
 // grid is then a few waves of blocks.  Least estimated time over all splits
 // that leave a warp at least four nodes, in instructions of a warp: waves x
@@ -842,17 +857,14 @@ int launch_hard(const uint32_t* xp, int w_in, long long N, const int* conn, cons
                 int w, uint32_t* yp, int C, int* counts, int* pred, cudaStream_t st) {
     const long long W = (N + 31) / 32;
     const uint32_t tail_mask = (N % 32) ? ((1u << (N % 32)) - 1u) : 0xffffffffu;
-    // staged kernels: 16-byte rows with 32-bit row offsets in 16-byte units, or
-    // any rows with 32-bit offsets in words
-    const bool vec4 = (W % 4 == 0) && aligned16(xp) && (!yp || aligned16(yp)) &&
-                      (unsigned long long)w_in * (unsigned long long)(W / 4) < (1ull << 32);
-    const bool staged = vec4 || (W >= kStagedMinWords && (unsigned long long)w_in * (unsigned long long)W < (1ull << 32));
+    const HardRoute route = hard_route(w_in, W, aligned16(xp) && (!yp || aligned16(yp)), C > 0);
+    const bool vec4 = route == kStaged16, staged = route != kOneWord;
     if (C == 0) {
         if (staged) {
             // chunks of kLayerNS stages; nodes per warp: enough blocks for
             // about four waves of two per SM
             const long long gy = (W + kLayerNS * kStageWords - 1) / (kLayerNS * kStageWords);
-            if (gy > 65535) return BITLOGIC_ERR_SHAPE;
+            if (gy > kGridY) return BITLOGIC_ERR_SHAPE;
             const long long groups = (w + kHardWarps - 1) / kHardWarps;
             long long npw = groups * gy / (8ll * sm_count());
             npw = npw < 1 ? 1 : (npw > 8 ? 8 : npw);
@@ -893,7 +905,7 @@ int launch_hard(const uint32_t* xp, int w_in, long long N, const int* conn, cons
             splits *= 2;
             per_split = (g + splits - 1) / splits;
         }
-        if ((long long)C * splits > 0x7fffffffll || wg > 65535) return BITLOGIC_ERR_SHAPE;
+        if ((long long)C * splits > 0x7fffffffll || wg > kGridY) return BITLOGIC_ERR_SHAPE;
         const int smem = head_smem_bytes<k>();
         auto kern = vec4 ? hard_head_staged_kernel<k, true> : hard_head_staged_kernel<k, false>;
         if (set_dynamic_smem(kern, smem)) return BITLOGIC_ERR_CUDA;
@@ -924,6 +936,11 @@ int launch_hard(const uint32_t* xp, int w_in, long long N, const int* conn, cons
 using namespace bitlogic;
 
 BITLOGIC_ERROR_READER(hard)
+
+// The route of a hard call, for host checks of the rule (HardRoute).
+extern "C" int bitlogic_internal_hard_route(int32_t w_in, int64_t words, int32_t aligned, int32_t head) {
+    return hard_route(w_in, words, aligned != 0, head != 0);
+}
 
 extern "C" int bitlogic_binarize_tables(const float* theta, int32_t w, int32_t k,
                                         uint64_t* table, cudaStream_t stream) {

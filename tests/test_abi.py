@@ -291,3 +291,21 @@ def test_compute_calls_reject_host_tensors():
         bl.bitlogic_pack_bits(x, [64, 128], torch.zeros(16, 1, dtype=torch.int32))
     with pytest.raises(ValueError, match="CUDA"):
         bl.bitlogic_issue_probe("lop3", 1, torch.zeros(8, dtype=torch.int32))
+
+
+def test_hard_route_of_long_rows():
+    # 4-byte staged rows only while their groups of stages (128 words in the
+    # head, 384 in a layer) fit grid.y, beyond that the one-word kernels; the
+    # 16-byte form keeps aligned rows of whole 16 bytes whatever their length
+    route = bl.load().bitlogic_internal_hard_route
+    route.argtypes = [ctypes.c_int32, ctypes.c_int64, ctypes.c_int32, ctypes.c_int32]
+    for head, per_y in ((1, 128), (0, 384)):
+        top = 65535 * per_y
+        for w_in in (2, 100):
+            for words, want in [(1, 0), (32, 0), (33, 1), (top - 1, 1), (top, 1), (top + 1, 0), (top + 3, 0)]:
+                if w_in * words >= 1 << 32:
+                    want = 0
+                assert route(w_in, words, 1, head) == (2 if words % 4 == 0 else want), (head, w_in, words)
+                assert route(w_in, words, 0, head) == want, (head, w_in, words)
+        assert route(1 << 20, 4097, 1, head) == 0 and route(1 << 20, 4095, 1, head) == 1
+        assert route(1 << 20, 4096, 1, head) == 2 and route(1 << 20, 4 << 12, 1, head) == 0

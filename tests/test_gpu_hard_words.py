@@ -71,3 +71,40 @@ def test_rows_off_a_16_byte_boundary(W, offset):
 def test_large_groups_and_few_classes():
     # more nodes per class than one block's slice: several splits
     _case(161, 9, 6, 200, 3000, 2)
+
+
+def _node_words(x, table):
+    """Output words of one fan-in-2 node on the words x [2, W] (device int32)."""
+    a, b = x[0], x[1]
+    corner = [~a & ~b, a & ~b, ~a & b, a & b]
+    out = torch.zeros_like(a)
+    for i in range(4):
+        if table >> i & 1:
+            out |= corner[i]
+    return out
+
+
+@pytest.mark.parametrize("W,head", [(65535 * 128 + 1, True), (65535 * 384 + 1, False)])
+def test_rows_of_more_stages_than_grid_y_holds(W, head):
+    # no multiple of four words, and longer than the staged kernels' grids take
+    N = 32 * W - 5
+    g = torch.Generator(device="cuda").manual_seed(W)
+    x = torch.randint(-2 ** 31, 2 ** 31, (2, W), generator=g, device="cuda", dtype=torch.int64).to(torch.int32)
+    x[:, -1] &= (1 << 27) - 1
+    conn, tables = np.array([[0, 1], [1, 0], [0, 1]], np.int32), [0b0110, 0b1011, 0b0001]
+    want = torch.stack([_node_words(x[c], t) for c, t in zip(conn.tolist(), tables)])
+    want[:, -1] &= (1 << 27) - 1
+    yp = torch.full((3, W), -1, dtype=torch.int32, device="cuda")
+    kw = {}
+    if head:
+        kw = dict(C=1, counts=torch.full((N, 1), -1, dtype=torch.int32, device="cuda"))
+    bl.bitlogic_hard_forward(x, N, dev(conn), dev(np.array(tables, np.int64)), yp=yp, **kw)
+    assert torch.equal(yp, want)
+    if head:
+        bit = torch.arange(32, device="cuda", dtype=torch.int32)
+        for w0 in range(0, W, 1 << 20):
+            part = want[:, w0:w0 + (1 << 20)]
+            count = sum((row[:, None] >> bit & 1) for row in part).reshape(-1)
+            got = kw["counts"][32 * w0:32 * w0 + count.numel(), 0]
+            assert torch.equal(got, count[:got.numel()])
+    assert bl.bitlogic_device_error() == 0
