@@ -737,8 +737,10 @@ corner_reduce_kernel(const float* __restrict__ corner, const int* __restrict__ o
     const long long o = (long long)j * K + (WIDE ? 2 * lane : lane);
     const bool in = WIDE || lane < K;
     float2 th = make_float2(0.f, 0.f);
-    if constexpr (WIDE) th = __ldg(reinterpret_cast<const float2*>(theta + o));
-    else if (in) th.x = __ldg(theta + o);
+    // logits and gradient by single values: a caller's parameter may start at
+    // any float
+    if (in) th.x = __ldg(theta + o);
+    if constexpr (WIDE) th.y = __ldg(theta + o + 1);
     if (e0 < 0 || e1 < e0 || e1 > n_edges) {
         if (lane == 0) flag_index_error();
         e0 = e1 = 0;
@@ -784,9 +786,8 @@ corner_reduce_kernel(const float* __restrict__ corner, const int* __restrict__ o
         }
     }
     const float t0 = sigmoidf(th.x), t1 = sigmoidf(th.y);
-    const float2 d = make_float2(t0 * (1.0f - t0) * s.x, t1 * (1.0f - t1) * s.y);
-    if constexpr (WIDE) *reinterpret_cast<float2*>(dtheta + o) = d;
-    else if (in) dtheta[o] = d.x;
+    if (in) dtheta[o] = t0 * (1.0f - t0) * s.x;
+    if constexpr (WIDE) dtheta[o + 1] = t1 * (1.0f - t1) * s.y;
 }
 
 // ------------------------------------------------------------- launchers --
@@ -934,9 +935,7 @@ extern "C" int bitlogic_corner_reduce(const float* corner_sums, const int32_t* c
     if (w <= 0 || n_edges < 0) return BITLOGIC_ERR_SHAPE;
     if (k < 1 || k > 6) return BITLOGIC_ERR_FANIN;
     const bool wide = k == 6;
-    if (wide && ((reinterpret_cast<uintptr_t>(corner_sums) | reinterpret_cast<uintptr_t>(theta) |
-                  reinterpret_cast<uintptr_t>(dtheta)) & 7u) != 0)
-        return BITLOGIC_ERR_ALIGN;
+    if (wide && (reinterpret_cast<uintptr_t>(corner_sums) & 7u) != 0) return BITLOGIC_ERR_ALIGN;
     // more warps per node while they all fit one wave and keep four positions
     // each on average: few nodes with many readers are bound by the chain of
     // their rows (training steps of fan-in 6: 1015 and 9110 nodes at 68 samples

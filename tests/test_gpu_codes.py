@@ -245,3 +245,29 @@ def test_nan_logits_reach_only_the_samples_that_select_them(k, k1, B):
     for i in range(k):
         unread = np.setdiff1d(np.arange(K1), a[conn[2, i]])
         assert not H_b[2 * k + i, unread].any(), "corners that no sample is on"
+
+
+@pytest.mark.parametrize("k", [6, 5, 4])
+@pytest.mark.parametrize("B", [256, 37])
+def test_step_on_parameters_off_an_aligned_address(k, B):
+    # logits that are slices of one parameter vector, starting at any float
+    wl = synth.Workload("codes", B, 60, 5, 40.0, (64, 128, 192), (300, 200), k, 5.0)
+    params = synth.network(wl, seed=3)
+    x, labels = synth.blob_batch(B, wl.d, wl.classes, wl.sigma, seed=4)
+    outs = []
+    for offset in (0, 1, 3):
+        net = Network(*params, wl.w_in)
+        for name in ("theta1", "theta2"):
+            t = getattr(net, name)
+            flat = torch.zeros(t.numel() + 4, device="cuda")
+            view = flat[offset:offset + t.numel()].view(t.shape)
+            view.copy_(t)
+            setattr(net, name, view)
+        st = TrainStep(net, B, wl.d, wl.thresholds, wl.classes, wl.tau)
+        st.load(x.cuda(), labels.cuda())
+        st.run()
+        outs.append([t.cpu().numpy() for t in (st.logits, st.dth1, st.dth2)])
+    for got in outs[1:]:
+        for a, b in zip(got, outs[0]):
+            check_exact(a, b, "as with aligned logits")
+    assert bl.bitlogic_device_error() == 0
