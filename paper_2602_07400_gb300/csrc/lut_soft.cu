@@ -1010,31 +1010,20 @@ lut_backward_theta_kernel(const float* __restrict__ X, int w_in, long long B,
 // slots of blocks and warps, and a fixed eight left up to seven of them idle
 // (8000 rows of 16000 nodes, layer backward and forward: fan-in 4, 47 samples
 // 57 -> 36 us, 245 samples 80 -> 62 us; fan-in 2, 64 samples 45 -> 33 us; one
-// sample per lane instead: 245 samples 73 us).  SPLIT: `parts` times as many
-// warps, each group over a run of the row's positions in increasing order,
-// then the runs in order, for few rows with many terms, where the chain of a
-// row's loads bounds the kernel.
+// sample per lane instead: 245 samples 73 us).
 constexpr int kCsrWarps = 8;
 
-template <bool VEC, bool SPLIT>
+template <bool VEC>
 __global__ void __launch_bounds__(kCsrWarps * 32)
 csr_reduce_kernel(const float* __restrict__ P, long long B, const int* __restrict__ off,
-                  const int* __restrict__ edge, int w_in, int nE, int parts, float* __restrict__ dX) {
-    __shared__ float4 run[SPLIT ? kCsrWarps : 1][32];
-    const int lane = threadIdx.x & 31;
-    const int warps = (blockDim.x >> 5) / (SPLIT ? parts : 1);   // over the batch
-    const int part = SPLIT ? (threadIdx.x >> 5) / warps : 0;
-    const int warp = (threadIdx.x >> 5) - part * warps;
+                  const int* __restrict__ edge, int w_in, int nE, float* __restrict__ dX) {
+    const int warps = blockDim.x >> 5;   // over the batch
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int i = blockIdx.x;
     int e0 = __ldg(off + i), e1 = __ldg(off + i + 1);
     if (e0 < 0 || e1 < e0 || e1 > nE) {
         if (threadIdx.x == 0) flag_index_error();
         e0 = e1 = 0;
-    }
-    if constexpr (SPLIT) {
-        const int len = (e1 - e0 + parts - 1) / parts;
-        e0 = min(e0 + part * len, e1);
-        e1 = min(e0 + len, e1);
     }
     const int deg = e1 - e0;
     int my_id = -1;   // ids of the first 32 positions, -1 when out of range
@@ -1085,12 +1074,105 @@ csr_reduce_kernel(const float* __restrict__ P, long long B, const int* __restric
         for (int u = 0; u < kCsrBatch; ++u)
             if (q0 + u < deg) acc = add4(acc, v[u]);
     }
-    if constexpr (SPLIT) {
-        run[threadIdx.x >> 5][lane] = acc;
-        __syncthreads();
-        if (part != 0) return;
-        for (int r = 1; r < parts; ++r) acc = add4(acc, run[r * warps + warp][lane]);
+    if constexpr (VEC) {
+        if (in[0]) *reinterpret_cast<float4*>(out) = acc;
+    } else {
+        if (in[0]) out[0] = acc.x;
+        if (in[1]) out[32] = acc.y;
+        if (in[2]) out[64] = acc.z;
+        if (in[3]) out[96] = acc.w;
     }
+}
+
+// The same sum for few rows with many terms, where the chain of a row's loads
+// bounds the kernel: a ring of kRingRows term rows in shared memory, filled by
+// cp.async in groups of eight.  A lane copies and adds its own four samples,
+// so the ring needs no synchronisation, and the adds keep the order of the
+// positions: a sum split over warps is not the one that a layer forms from
+// the same terms.  Layer forward and backward, against the kernel above:
+// 64000 nodes of fan-in 6 over 500 rows, 32 samples 402 -> 201 us; 30000 of
+// fan-in 4 over 700, 100 samples 118 -> 67 us; 20000 of fan-in 3 over 600, 500
+// samples 128 -> 84 us (64 rows: 195, 66 and 90 us); 30000 of fan-in 6 over
+// 500, 47 samples 217 -> 117 us (copies and zero stores behind a branch
+// instead of cp.async's zero fill: 163 us).
+constexpr int kRingRows = 32, kRingGroup = 8, kRingWarps = 4;
+constexpr int kRingGroups = kRingRows / kRingGroup;
+
+template <bool VEC>
+__global__ void __launch_bounds__(kRingWarps * 32)
+csr_reduce_ring_kernel(const float* __restrict__ P, long long B, const int* __restrict__ off,
+                       const int* __restrict__ edge, int nE, float* __restrict__ dX) {
+    extern __shared__ __align__(16) float csr_ring[];
+    const int warps = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int i = blockIdx.x;
+    int e0 = __ldg(off + i), e1 = __ldg(off + i + 1);
+    if (e0 < 0 || e1 < e0 || e1 > nE) {
+        if (threadIdx.x == 0) flag_index_error();
+        e0 = e1 = 0;
+    }
+    const int deg = e1 - e0, groups = (deg + kRingGroup - 1) / kRingGroup;
+    // lane u: id of position q0 + u, -1 past the end or out of range
+    auto ids_from = [&](int q0) {
+        int id = -1;
+        if (q0 + lane < deg) {
+            id = edge ? __ldg(edge + e0 + q0 + lane) : e0 + q0 + lane;
+            if ((unsigned)id >= (unsigned)nE) {
+                if (warp == 0) flag_index_error();
+                id = -1;
+            }
+        }
+        return id;
+    };
+    const long long s = ((long long)blockIdx.y * warps + warp) * 128 + (VEC ? 4 : 1) * lane;
+    const float* col = P + (s < B ? s : 0);
+    bool in[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) in[c] = s + (VEC ? 0 : 32 * c) < B;
+    float* ring = csr_ring + warp * (kRingRows * 128) + (VEC ? 4 : 1) * lane;
+    int ids = ids_from(0), next = ids_from(32);   // of the 32 positions being issued, and of the 32 after
+    int gi = 0, slot = 0;                         // group to issue, and its place
+    auto issue = [&]() {
+        if (gi < groups) {
+            const int q = (gi * kRingGroup) & 31;
+            if (q == 0 && gi > 0) {
+                ids = next;
+                next = ids_from(gi * kRingGroup + 32);
+            }
+            float* row = ring + slot * (kRingGroup * 128);
+#pragma unroll
+            for (int u = 0; u < kRingGroup; ++u) {
+                const int id = __shfl_sync(0xffffffffu, ids, q + u);
+                const float* src = col + (long long)max(id, 0) * B;
+#pragma unroll
+                for (int c = 0; c < (VEC ? 1 : 4); ++c) {   // zeros without a read for what adds nothing
+                    const bool take = id >= 0 && in[c];
+                    if constexpr (VEC) cp_async16_or_zero(row + u * 128, src, take);
+                    else cp_async4_or_zero(row + u * 128 + 32 * c, src + (in[c] ? 32 * c : 0), take);
+                }
+            }
+        }
+        ++gi;
+        slot = slot + 1 == kRingGroups ? 0 : slot + 1;
+        cp_async_commit();
+    };
+#pragma unroll 1
+    for (int g = 0; g < kRingGroups - 1; ++g) issue();
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    int at = 0;
+#pragma unroll 1
+    for (int g = 0; g < groups; ++g) {
+        issue();
+        cp_async_wait<kRingGroups - 1>();
+        const float* row = ring + at * (kRingGroup * 128);
+#pragma unroll
+        for (int u = 0; u < kRingGroup; ++u) {   // rows past the end are zeros
+            if constexpr (VEC) acc = add4(acc, *reinterpret_cast<const float4*>(row + u * 128));
+            else acc = add4(acc, make_float4(row[u * 128], row[u * 128 + 32], row[u * 128 + 64], row[u * 128 + 96]));
+        }
+        at = at + 1 == kRingGroups ? 0 : at + 1;
+    }
+    cp_async_wait<0>();
+    float* out = dX + (long long)i * B + s;
     if constexpr (VEC) {
         if (in[0]) *reinterpret_cast<float4*>(out) = acc;
     } else {
@@ -1319,18 +1401,20 @@ extern "C" int bitlogic_csr_reduce(const float* edge_terms, int64_t B, const int
     const long long gy = (B + per_block - 1) / per_block;
     if (gy > 65535) return BITLOGIC_ERR_SHAPE;
     dim3 grid((unsigned)w_in, (unsigned)gy);
-    // more warps per row while the block holds them, they all fit one wave and
-    // keep 16 terms each on average (layer forward and backward: 64000 nodes of
-    // fan-in 6 over 500 rows, 32 samples 409 -> 191 us; 20000 of fan-in 3 over
-    // 600, 500 samples 125 -> 91 us; with eight terms each, 16000 of fan-in 2
-    // over 2000, 200 samples 37.2 -> 38.9 us)
-    int parts = 1;
-    while (2 * parts * warps <= kCsrWarps && 2ll * parts * warps * w_in <= 64ll * sm_count() &&
-           n_edges / (2ll * parts * w_in) >= 16)
-        parts *= 2;
-    auto kern = parts > 1 ? (vec ? csr_reduce_kernel<true, true> : csr_reduce_kernel<false, true>)
-                          : (vec ? csr_reduce_kernel<true, false> : csr_reduce_kernel<false, false>);
-    kern<<<grid, warps * parts * 32, 0, stream>>>(edge_terms, B, csr_off, csr_edge, w_in, n_edges, parts, dX);
+    // the ring while all warps fit half a wave and a row has 32 terms or more on
+    // average (8 and 16: 20000 nodes of fan-in 2 over 5000 rows, 75 samples
+    // 38.9 -> 41.0 us; 16000 over 2000, 200 samples 37.2 -> 38.7 us)
+    if (warps <= kRingWarps && 2ll * warps * w_in <= 64ll * sm_count() && n_edges / w_in >= 32) {
+        const int smem = warps * kRingRows * 128 * (int)sizeof(float);
+        auto kern = vec ? csr_reduce_ring_kernel<true> : csr_reduce_ring_kernel<false>;
+        if (smem > 40 * 1024 &&
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
+            return BITLOGIC_ERR_CUDA;
+        kern<<<grid, warps * 32, smem, stream>>>(edge_terms, B, csr_off, csr_edge, n_edges, dX);
+    } else {
+        auto kern = vec ? csr_reduce_kernel<true> : csr_reduce_kernel<false>;
+        kern<<<grid, warps * 32, 0, stream>>>(edge_terms, B, csr_off, csr_edge, w_in, n_edges, dX);
+    }
     return launch_status();
 }
 

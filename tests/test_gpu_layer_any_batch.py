@@ -153,3 +153,28 @@ def test_backward_over_several_nodes_per_block(k, w, B, offset):
         check_grad(dth, wth, "dtheta")
         check_grad(dX, wdx, "dX")
     assert bl.bitlogic_device_error() == 0
+
+
+@pytest.mark.parametrize("w_in,deg", [(1, 40), (7, 500), (60, 70), (900, 33), (3, 20)])
+@pytest.mark.parametrize("B,offset", [(4, 0), (130, 0), (256, 0), (300, 1), (515, 0)])
+def test_upstream_terms_are_the_csr_reduction_bit_for_bit(w_in, deg, B, offset):
+    # the gradient that a layer sums from the next layer's terms is
+    # bitlogic_csr_reduce of them, also where few rows have many terms
+    rng = np.random.default_rng(w_in + deg + B)
+    n = w_in * deg
+    off = np.searchsorted(np.sort(rng.integers(0, w_in, size=n)), np.arange(w_in + 1)).astype(np.int32)
+    terms = rng.standard_normal((n, B), dtype=np.float32)
+    edge = rng.permutation(n).astype(np.int32)
+    Pd = off_boundary(terms, offset)
+    dX = torch.full((w_in, B), np.nan, device="cuda")
+    bl.bitlogic_csr_reduce(Pd, dev(off), dev(edge), dX)
+    X = synth.uniform_activations(8, B, seed=5)
+    for k in (1, 2, 4):
+        conn = synth.connectivity(w_in, k, 8, seed=6)
+        theta = dev(synth.table_logits(w_in, 1 << k, seed=7))
+        for terms_out in (None, torch.empty(w_in * k, B, device="cuda")):
+            used = torch.full((w_in, B), np.nan, device="cuda")
+            bl.bitlogic_lut_backward_node(dev(X), dev(conn), theta, torch.empty_like(theta), "soft", up_terms=Pd,
+                                          up_off=dev(off), up_edge=dev(edge), edge_terms=terms_out, dY_out=used)
+            check_exact(used.cpu().numpy(), dX.cpu().numpy(), "gradient used")
+    assert bl.bitlogic_device_error() == 0
