@@ -95,6 +95,8 @@ _SIGS = {
     "bitlogic_lut_forward_coded": ([_P, _P, _I32, _I32, _I64, _P, _P, _I32, _I32, _I32, _P, _P], ctypes.c_int),
     "bitlogic_lut_backward_coded": ([_P, _P, _I32, _I32, _I64, _P, _P, _I32, _I32, _I32, _P, _I32, _P, _P, _P, _P],
                                     ctypes.c_int),
+    "bitlogic_internal_lut_backward_coded": ([_P, _P, _I32, _I32, _I64, _P, _P, _I32, _I32, _I32, _P, _I32, _P, _P, _P,
+                                              _P, _P], ctypes.c_int),
     "bitlogic_corner_reduce": ([_P, _P, _P, _I32, _P, _I32, _I32, _P, _P], ctypes.c_int),
     "bitlogic_lut_backward_workspace": ([_I32, _I64, _I32, _I32, _I32], _SZ),
     "bitlogic_lut_backward": ([_P, _I32, _I64, _P, _P, _I32, _I32, _P, _P, _P, _P, _P,
@@ -739,9 +741,11 @@ def bitlogic_lut_forward_coded(codes: torch.Tensor, table: torch.Tensor, conn: t
 def bitlogic_lut_backward_coded(codes: torch.Tensor, table: torch.Tensor, B: int, conn: torch.Tensor,
                                 theta: torch.Tensor, dtheta: torch.Tensor, corner_sums: torch.Tensor,
                                 dY: torch.Tensor, dy_group: int = 1, node="soft",
-                                edge_pos: Optional[torch.Tensor] = None, stream=None):
+                                edge_pos: Optional[torch.Tensor] = None, stream=None,
+                                theta_read: Optional[torch.Tensor] = None):
     """Layer backward (fan-in 4..6) on corner codes: dtheta, and per edge the
-    corner sums [w*k, 2^k_in] of its input-gradient terms."""
+    corner sums [w*k, 2^k_in] of its input-gradient terms; theta_read receives
+    the logits that the call read."""
     w, k = conn.shape
     w_in, k_in = _need_codes(codes, table, B)
     _need(conn, "conn", torch.int32, (w, k))
@@ -753,9 +757,11 @@ def bitlogic_lut_backward_coded(codes: torch.Tensor, table: torch.Tensor, B: int
     _need(dY, "dY", torch.float32, (w // dy_group, B))
     if edge_pos is not None:
         _need(edge_pos, "edge_pos", torch.int32, (w * k,))
-    _check("bitlogic_lut_backward_coded", load().bitlogic_lut_backward_coded(
+    if theta_read is not None:
+        _need(theta_read, "theta_read", torch.float32, (w, 1 << k))
+    _check("bitlogic_lut_backward_coded", load().bitlogic_internal_lut_backward_coded(
         _ptr(codes), _ptr(table), w_in, k_in, B, _ptr(conn), _ptr(theta), w, k, _node_code(node), _ptr(dY),
-        int(dy_group), _ptr(dtheta), _ptr(corner_sums), _ptr(edge_pos), _stream(stream)))
+        int(dy_group), _ptr(dtheta), _ptr(corner_sums), _ptr(edge_pos), _ptr(theta_read), _stream(stream)))
 
 
 def bitlogic_corner_reduce(corner_sums: torch.Tensor, csr_off: torch.Tensor, csr_edge: Optional[torch.Tensor],

@@ -458,7 +458,7 @@ __global__ void __launch_bounds__(32, coded_bwd_blocks<k>())
 coded_backward_kernel(const uint8_t* __restrict__ codes, long long stride, const float* __restrict__ table1, int w_in,
                       int k1, long long B, const int* __restrict__ conn, const float* __restrict__ theta, int w,
                       int node, const float* __restrict__ dY, int group, bool vec, float* __restrict__ dtheta,
-                      float* __restrict__ corner, const int* __restrict__ epos) {
+                      float* __restrict__ corner, const int* __restrict__ epos, float* __restrict__ theta_read) {
     using O = Order<k>;
     constexpr bool TAIL = FORM == kShort;
     constexpr int C = O::C, K = O::K, H = O::H;
@@ -586,6 +586,11 @@ coded_backward_kernel(const uint8_t* __restrict__ codes, long long stride, const
         for (int a = 0; a < H; ++a) acc[a] = 0ull;
         __syncwarp();
         for (int q = lane; q < 2 * O::kCopy; q += 32) smem[q] = 0.f;
+        if (FORM != kWhole && theta_read) {
+#pragma unroll
+            for (int i = 0; i < NF; ++i)
+                if (e0 + i < K) theta_read[(long long)j * K + e0 + i] = th[i];
+        }
         ahead(j + G);
         cp_async_wait<0>();
         __syncwarp();
@@ -822,7 +827,7 @@ int launch_coded_forward(const uint8_t* codes, long long stride, const float* ta
 template <int k>
 int launch_coded_backward(const uint8_t* codes, long long stride, const float* table, int w_in, int k1, long long B,
                           const int* conn, const float* theta, int w, int node, const float* dY, int group,
-                          float* dtheta, float* corner, const int* epos, cudaStream_t st) {
+                          float* dtheta, float* corner, const int* epos, float* theta_read, cudaStream_t st) {
     constexpr int smem = coded_bwd_smem<k>();
     // one wave: as many blocks per SM as registers and shared memory (228 KB,
     // 1 KB of it per block) hold
@@ -833,7 +838,7 @@ int launch_coded_backward(const uint8_t* codes, long long stride, const float* t
                                 : coded_backward_kernel<k, kRagged>;
     kern<<<(unsigned)(w < resident ? w : resident), 32, smem, st>>>(
         codes, stride, table, w_in, k1, B, conn, theta, w, node, dY, group, B % 4 == 0 && aligned16(dY), dtheta, corner,
-        epos);
+        epos, theta_read);
     return launch_status();
 }
 
@@ -906,14 +911,22 @@ extern "C" int bitlogic_lut_forward_coded(const uint8_t* codes, const float* tab
     }
 }
 
-extern "C" int bitlogic_lut_backward_coded(const uint8_t* codes, const float* table, int32_t w_in, int32_t k_in,
-                                           int64_t B, const int32_t* conn, const float* theta, int32_t w, int32_t k,
-                                           int32_t node, const float* dY, int32_t dy_group, float* dtheta,
-                                           float* corner_sums, const int32_t* edge_pos, cudaStream_t stream) {
+// bitlogic_lut_backward_coded; theta_read (or NULL) receives the logits that
+// the call read, for a caller that forms more of this backward once theta has
+// moved on.  The kernels of partly filled stages store them as they go.
+extern "C" int bitlogic_internal_lut_backward_coded(const uint8_t* codes, const float* table, int32_t w_in,
+                                                    int32_t k_in, int64_t B, const int32_t* conn, const float* theta,
+                                                    int32_t w, int32_t k, int32_t node, const float* dY,
+                                                    int32_t dy_group, float* dtheta, float* corner_sums,
+                                                    const int32_t* edge_pos, float* theta_read, cudaStream_t stream) {
     int st = check_coded(codes, table, w_in, k_in, B, conn, theta, w, k, node);
     if (st) return st;
     if (!dtheta || !corner_sums || (B > 0 && !dY)) return BITLOGIC_ERR_NULL;
     if (dy_group < 1 || dy_group > w) return BITLOGIC_ERR_SHAPE;
+    if (theta_read && B % 128 == 0 &&
+        cudaMemcpyAsync(theta_read, theta, sizeof(float) * (size_t)w << k, cudaMemcpyDeviceToDevice, stream) !=
+            cudaSuccess)
+        return BITLOGIC_ERR_CUDA;
     if (B == 0) {   // empty batch: the batch sums are zero
         if (cudaMemsetAsync(dtheta, 0, sizeof(float) * (size_t)w << k, stream) != cudaSuccess ||
             cudaMemsetAsync(corner_sums, 0, sizeof(float) * (size_t)w * k << k_in, stream) != cudaSuccess)
@@ -921,11 +934,23 @@ extern "C" int bitlogic_lut_backward_coded(const uint8_t* codes, const float* ta
         return BITLOGIC_OK;
     }
     const long long sd = code_stride(B);
+#define BITLOGIC_CODED_K(K)                                                                                       \
+    return launch_coded_backward<K>(codes, sd, table, w_in, k_in, B, conn, theta, w, node, dY, dy_group, dtheta, \
+                                    corner_sums, edge_pos, theta_read, stream)
     switch (k) {
-        case 4: return launch_coded_backward<4>(codes, sd, table, w_in, k_in, B, conn, theta, w, node, dY, dy_group, dtheta, corner_sums, edge_pos, stream);
-        case 5: return launch_coded_backward<5>(codes, sd, table, w_in, k_in, B, conn, theta, w, node, dY, dy_group, dtheta, corner_sums, edge_pos, stream);
-        default: return launch_coded_backward<6>(codes, sd, table, w_in, k_in, B, conn, theta, w, node, dY, dy_group, dtheta, corner_sums, edge_pos, stream);
+        case 4: BITLOGIC_CODED_K(4);
+        case 5: BITLOGIC_CODED_K(5);
+        default: BITLOGIC_CODED_K(6);
     }
+#undef BITLOGIC_CODED_K
+}
+
+extern "C" int bitlogic_lut_backward_coded(const uint8_t* codes, const float* table, int32_t w_in, int32_t k_in,
+                                           int64_t B, const int32_t* conn, const float* theta, int32_t w, int32_t k,
+                                           int32_t node, const float* dY, int32_t dy_group, float* dtheta,
+                                           float* corner_sums, const int32_t* edge_pos, cudaStream_t stream) {
+    return bitlogic_internal_lut_backward_coded(codes, table, w_in, k_in, B, conn, theta, w, k, node, dY, dy_group,
+                                                dtheta, corner_sums, edge_pos, nullptr, stream);
 }
 
 extern "C" int bitlogic_corner_reduce(const float* corner_sums, const int32_t* csr_off, const int32_t* csr_edge,

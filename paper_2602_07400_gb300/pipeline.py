@@ -214,8 +214,9 @@ class TrainStep:
     inputs from those, and its backward reduces each edge's terms to the
     2^k1 corner sums that layer 1's table gradient adds up
     (bitlogic_lut_backward_coded, bitlogic_corner_reduce), so no per-edge rows
-    are stored.  ``y1`` is then written out on demand.  Set
-    ``keep_dy1`` to also write dY1 (e.g. to check it).  ``node`` picks the
+    are stored.  ``y1`` is then written out on demand, and on a batch that is
+    no multiple of four ``dy1`` too.  Set ``keep_dy1`` to also write dY1 in
+    every step (e.g. to check it).  ``node`` picks the
     LightLUT form of both layers: "soft", or "st" (hard table samples in the
     forward, straight-through gradient to the logits)."""
 
@@ -278,8 +279,12 @@ class TrainStep:
             self.corners2 = torch.empty(net.w2 * net.k2, 1 << net.k1, **f32)
         if not self.codes1 or keep_dy1:
             self._y1 = torch.empty(net.w1, B, **f32)
+        # dY1 under codes1: written by the step when kept, and on a ragged batch,
+        # where the step's default used to form it, on demand from the logits
+        # that the last backward read
         if self.codes1 and keep_dy1:
             self._dth2_terms = torch.empty_like(net.theta2)
+        self._theta2_read = torch.empty_like(net.theta2) if self.codes1 and ragged_codes and not keep_dy1 else None
         # the encoder's output: wire bit rows (bits1), byte rows (bytes1) or
         # fp32 rows
         if self.bits1:
@@ -289,9 +294,9 @@ class TrainStep:
         # per-edge terms stored in CSR order (each input's terms contiguous,
         # read without the edge map) instead of edge order
         self.csr_order = bool(csr_order)
-        self.dy1 = torch.empty(net.w1, B, **f32) if (keep_dy1 or not (self.fuse_dy1 or self.through)) else None
+        self._dy1 = torch.empty(net.w1, B, **f32) if (keep_dy1 or not (self.fuse_dy1 or self.through)) else None
         # under codes1 nothing but dY1 itself needs the per-edge terms
-        need_terms = not self.through and not (self.codes1 and self.dy1 is None)
+        need_terms = not self.through and not (self.codes1 and self._dy1 is None)
         self.dth1 = torch.empty_like(net.theta1)
         self.dth2 = torch.empty_like(net.theta2)
         self.dbits = torch.empty(net.w_in, B, **f32) if want_dx1 else None
@@ -311,6 +316,27 @@ class TrainStep:
         out = torch.empty(self.net.w1, self.B, dtype=torch.float32, device=self.codes.device)
         bitlogic_codes_decode(self.codes, self.table1, out)
         return out
+
+    @property
+    def dy1(self) -> Optional[torch.Tensor]:
+        """Layer 1's output gradient [w1, B] of the last backward: the buffer
+        that the step writes, or under ``codes1`` on a batch that is no
+        multiple of four formed into a new tensor (``keep_dy1``: a buffer
+        there too).  None where the route does not form it."""
+        if self._theta2_read is None:
+            return self._dy1
+        n = self.net
+        terms = torch.empty(n.w2 * n.k2, self.B, dtype=torch.float32, device=self.codes.device)
+        out = torch.empty(n.w1, self.B, dtype=torch.float32, device=self.codes.device)
+        self._write_dy1(self.y1, self._theta2_read, torch.empty_like(n.theta2), terms, out)
+        return out
+
+    def _write_dy1(self, y1, theta2, dth2, terms, out, stream=None):
+        """dY1 from layer 2's per-edge terms, as the other routes form it."""
+        n = self.net
+        bitlogic_lut_backward_node(y1, n.conn2, theta2, dth2, self.node, dY=self.dyg, dy_group=n.w2 // self.C,
+                                   edge_terms=terms, edge_pos=n.pos2, stream=stream)
+        bitlogic_csr_reduce(terms, n.off2, None, out, stream)
 
     def load(self, x: torch.Tensor, labels: torch.Tensor, non_blocking: bool = False):
         self.x.copy_(x, non_blocking=non_blocking)
@@ -351,15 +377,13 @@ class TrainStep:
         g = n.w2 // self.C
         if self.codes1:
             bitlogic_lut_backward_coded(self.codes, self.table1, self.B, n.conn2, n.theta2, self.dth2, self.corners2,
-                                        self.dyg, g, nd, edge_pos=n.pos2, stream=stream)
+                                        self.dyg, g, nd, edge_pos=n.pos2, stream=stream, theta_read=self._theta2_read)
             mark("backward2")
             bitlogic_corner_reduce(self.corners2, n.off2, None, n.theta1, self.dth1, stream)
             mark("backward1")
-            if self.dy1 is not None:   # dY1 is kept: from the terms, as the other routes form it
+            if self._dy1 is not None:   # dY1 is kept
                 bitlogic_codes_decode(self.codes, self.table1, self._y1, stream)
-                bitlogic_lut_backward_node(self._y1, n.conn2, n.theta2, self._dth2_terms, nd, dY=self.dyg, dy_group=g,
-                                           edge_terms=self.edges2, edge_pos=n.pos2, stream=stream)
-                bitlogic_csr_reduce(self.edges2, n.off2, None, self.dy1, stream)
+                self._write_dy1(self._y1, n.theta2, self._dth2_terms, self.edges2, self._dy1, stream)
                 mark("dy1")
             return
         if self.through:
@@ -370,7 +394,7 @@ class TrainStep:
             mark("backward2")
             bitlogic_lut_backward_through(self.bits, n.conn1, n.theta1, self.dth1,
                                           self.y1, n.conn2, n.theta2, self.dyg, g, n.off2, n.edge2, node=nd,
-                                          dY_out=self.dy1, stream=stream)
+                                          dY_out=self._dy1, stream=stream)
             mark("backward1")
             return
         # the bit-row layer-1 backward reads the terms through the CSR map in
@@ -384,25 +408,25 @@ class TrainStep:
         edge2 = None if co else n.edge2
         if ordered:
             bitlogic_lut_backward_bitrows(self.bits, self.B, n.conn1, n.theta1, self.dth1, nd, up_terms=self.edges2,
-                                          up_off=n.off2o, up_edge=None if co else n.edge2o, dY_out=self.dy1,
+                                          up_off=n.off2o, up_edge=None if co else n.edge2o, dY_out=self._dy1,
                                           order=n.order1, stream=stream)
         elif self.fuse_dy1 and self.bytes1:
             bitlogic_lut_backward_u8(self.bits, n.conn1, n.theta1, self.dth1, nd, up_terms=self.edges2,
-                                     up_off=n.off2, up_edge=edge2, dY_out=self.dy1, stream=stream)
+                                     up_off=n.off2, up_edge=edge2, dY_out=self._dy1, stream=stream)
         elif self.fuse_dy1:
             bitlogic_lut_backward_node(self.bits, n.conn1, n.theta1, self.dth1, nd, up_terms=self.edges2,
                                        up_off=n.off2, up_edge=edge2, edge_terms=self.edges1,
-                                       edge_pos=pos1, dY_out=self.dy1, stream=stream)
+                                       edge_pos=pos1, dY_out=self._dy1, stream=stream)
         else:
-            bitlogic_csr_reduce(self.edges2, n.off2, edge2, self.dy1, stream)
+            bitlogic_csr_reduce(self.edges2, n.off2, edge2, self._dy1, stream)
             mark("csr2")
             if self.bits1:
-                bitlogic_lut_backward_bitrows(self.bits, self.B, n.conn1, n.theta1, self.dth1, nd, dY=self.dy1,
+                bitlogic_lut_backward_bitrows(self.bits, self.B, n.conn1, n.theta1, self.dth1, nd, dY=self._dy1,
                                               stream=stream)
             elif self.bytes1:
-                bitlogic_lut_backward_u8(self.bits, n.conn1, n.theta1, self.dth1, nd, dY=self.dy1, stream=stream)
+                bitlogic_lut_backward_u8(self.bits, n.conn1, n.theta1, self.dth1, nd, dY=self._dy1, stream=stream)
             else:
-                bitlogic_lut_backward_node(self.bits, n.conn1, n.theta1, self.dth1, nd, dY=self.dy1,
+                bitlogic_lut_backward_node(self.bits, n.conn1, n.theta1, self.dth1, nd, dY=self._dy1,
                                            edge_terms=self.edges1, edge_pos=pos1, stream=stream)
         mark("backward1")
         if self.dbits is not None:
@@ -456,7 +480,7 @@ class TrainStep:
     @property
     def kernels_per_run(self) -> int:
         if self.codes1:
-            return 7 + (3 if self.dy1 is not None else 0)
+            return 7 + (3 if self._dy1 is not None else 0)
         return 7 + (0 if (self.fuse_dy1 or self.through) else 1) + (1 if self.dbits is not None else 0)
 
 

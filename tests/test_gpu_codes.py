@@ -147,7 +147,8 @@ def test_training_step_on_codes(B, k, node):
     steps = []
     for keep in (False, True):
         st = TrainStep(net, B, wl.d, wl.thresholds, wl.classes, wl.tau, node=node, keep_dy1=keep)
-        assert st.codes1 and st.bits1 and st.fuse_dy1 and (st.dy1 is not None) == keep
+        # a ragged batch offers dY1 with or without keep_dy1
+        assert st.codes1 and st.bits1 and st.fuse_dy1 and (st.dy1 is not None) == (keep or B % 4 != 0)
         st.load(x.cuda(), labels.cuda())
         st.run()
         steps.append(st)
@@ -270,4 +271,38 @@ def test_step_on_parameters_off_an_aligned_address(k, B):
     for got in outs[1:]:
         for a, b in zip(got, outs[0]):
             check_exact(a, b, "as with aligned logits")
+    assert bl.bitlogic_device_error() == 0
+
+
+@pytest.mark.parametrize("B,k,node", [(127, 6, "soft"), (37, 4, "st"), (257, 5, "soft")])
+def test_ragged_step_offers_the_gradient_of_layer_1(B, k, node):
+    # without keep_dy1, eager and replayed, also once the logits have moved on
+    wl = synth.Workload("codes", B, 60, 5, 40.0, (64, 128, 192), (300, 200), k, 5.0)
+    params = synth.network(wl, seed=3)
+    x, labels = synth.blob_batch(B, wl.d, wl.classes, wl.sigma, seed=4)
+    conn1, th1, conn2, th2 = params
+    r = oracle.train_step(x.numpy(), labels.numpy(), wl.thresholds, conn1, th1, conn2, th2, wl.classes, wl.tau,
+                          want_dx1=False, node=node)
+    for captured in (False, True):
+        st = TrainStep(Network(*params, wl.w_in), B, wl.d, wl.thresholds, wl.classes, wl.tau, node=node)
+        assert st.dy1.shape == (300, B)
+        st.load(x.cuda(), labels.cuda())
+        if captured:
+            st.capture().replay()
+        else:
+            st.run()
+        before = st.dy1
+        check_grad(before, r["dy1"], "dy1")
+        st.update(lr=0.5)
+        st.x.zero_()
+        check_exact(st.dy1.cpu().numpy(), before.cpu().numpy(), "dy1 after the update")
+        side = torch.cuda.Stream()
+        side.wait_stream(torch.cuda.current_stream())
+        st.load(x.cuda(), labels.cuda())
+        torch.cuda.synchronize()
+        st.run(stream=side)
+        side.synchronize()
+        want = oracle.train_step(x.numpy(), labels.numpy(), wl.thresholds, conn1, st.net.theta1.cpu().numpy(), conn2,
+                                 st.net.theta2.cpu().numpy(), wl.classes, wl.tau, want_dx1=False, node=node)
+        check_grad(st.dy1, want["dy1"], "dy1 of a step on another stream")
     assert bl.bitlogic_device_error() == 0
