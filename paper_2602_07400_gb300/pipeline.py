@@ -239,9 +239,11 @@ class TrainStep:
             raise ValueError("the through route needs layer-2 fan-in <= 3, B % 4 == 0 and no layer-1 input gradient")
         self.through = bool(through)
         # a batch that is no multiple of four takes binary wires for layer 1
-        # only on corner codes, whose kernels accept any B
-        ragged_codes = (B % 4 != 0 and not want_dx1 and csr_order and net.k2 >= 4 and fuse_dy1 is None
-                        and bytes1 is None and bits1 is None and codes1 is not False)
+        # only on corner codes, whose kernels accept any B: when codes are asked
+        # for, or the whole route is left to the step
+        route = (fuse_dy1, bytes1, bits1)
+        ragged_codes = (B % 4 != 0 and not want_dx1 and csr_order and net.k2 >= 4
+                        and (False not in route if codes1 else codes1 is None and route == (None, None, None)))
         if bytes1 is None:
             bytes1 = (B % 4 == 0 or ragged_codes) and not want_dx1
         terms_asked = fuse_dy1 is not None

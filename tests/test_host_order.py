@@ -4,10 +4,11 @@ sequence, as `pipeline.Network` prepares them, and the bit-row byte
 accounting of the benchmark for a batch that is not a whole number of
 1024-sample blocks."""
 import numpy as np
+import pytest
 
 import paper_2602_07400_gb300 as bl
 from paper_2602_07400_gb300 import synth
-from paper_2602_07400_gb300.pipeline import Network
+from paper_2602_07400_gb300.pipeline import Network, TrainStep
 
 
 def test_network_orders_layer1_by_consumer_count_with_a_matching_csr_map():
@@ -45,3 +46,25 @@ def test_bit_row_accounting_pads_the_batch_to_whole_blocks():
     assert work["forward1"][0] - xw1 == bench.call_work(wl, B, fuse_dy1=True, bytes1=True)["forward1"][0] - wl.w_in * B
     assert bl.bitrow_words(B) == 32 and bl.bitrow_words(1024) == 32 and bl.bitrow_words(1025) == 64
     assert bl.bitrow_words(0) == 0
+
+
+@pytest.mark.parametrize("B", [37, 130])
+def test_ragged_batch_takes_codes_that_are_asked_for(B):
+    # corner codes named together with the wires and route they imply, which
+    # without them need B % 4 == 0
+    wl = synth.Workload("t", B, 20, 4, 1.0, [64, 128, 192], (300, 200), 4, 10.0)
+    net = Network(*synth.network(wl, seed=4), wl.w_in, device="cpu")
+
+    def step(**kw):
+        return TrainStep(net, B, wl.d, wl.thresholds, wl.classes, wl.tau, device="cpu", **kw)
+
+    for kw in (dict(), dict(codes1=True), dict(codes1=True, bytes1=True), dict(codes1=True, bits1=True),
+               dict(codes1=True, bytes1=True, bits1=True, fuse_dy1=True)):
+        st = step(**kw)
+        assert st.codes1 and st.bits1 and st.bytes1 and st.fuse_dy1
+    for kw in (dict(bytes1=True), dict(bits1=True), dict(codes1=True, bits1=False), dict(codes1=True, bytes1=False),
+               dict(codes1=True, fuse_dy1=False), dict(codes1=True, want_dx1=True), dict(codes1=True, csr_order=False),
+               dict(codes1=False, bytes1=True)):
+        with pytest.raises(ValueError):
+            step(**kw)
+    assert not step(fuse_dy1=True).codes1 and not step(codes1=False).codes1
