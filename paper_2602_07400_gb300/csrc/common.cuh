@@ -71,6 +71,13 @@ inline int make_thresholds(const uint8_t* thr_host, int32_t b, Thresholds* out) 
 // IEEE-rounded division (no fast-math).
 __device__ __forceinline__ float sigmoidf(float z) { return 1.0f / (1.0f + expf(-z)); }
 
+// Table entry of a node form (bitlogic_node_t): the sigmoid sg of the logit
+// th for the soft LightLUT node, the hard sample [th > 0] for the
+// straight-through node (whose theta gradient still takes the slope of sg).
+__device__ __forceinline__ float table_value(float th, float sg, int node) {
+    return node == BITLOGIC_NODE_ST ? (th > 0.f ? 1.f : 0.f) : sg;
+}
+
 // Asynchronous global -> shared copies (cp.async), 16 bytes (bypassing L1) or
 // 4, grouped per pipeline stage.
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {

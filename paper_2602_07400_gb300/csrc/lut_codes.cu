@@ -40,10 +40,6 @@ namespace {
 #endif
 constexpr int kCodesWarps = 8;
 
-__device__ __forceinline__ float node_value(float th, float sg, int node) {
-    return node == BITLOGIC_NODE_ST ? (th > 0.f ? 1.f : 0.f) : sg;
-}
-
 // ------------------------------------------------- layer 1: codes, tables --
 
 // A warp per node and range of 1024-sample blocks; lanes and wire words as in
@@ -74,7 +70,7 @@ codes_forward_kernel(const uint32_t* __restrict__ X, int w_in, long long words, 
         for (int a = 0; a < K; a += 32) {
             if (a + lane < K) {
                 const float th = __ldg(theta + (long long)j * K + a + lane);
-                table[(long long)j * K + a + lane] = node_value(th, sigmoidf(th), node);
+                table[(long long)j * K + a + lane] = table_value(th, sigmoidf(th), node);
             }
         }
     }
@@ -248,7 +244,7 @@ coded_forward_kernel(const uint8_t* __restrict__ codes, long long stride, const 
     for (int j = blockIdx.x; j < w; j += G) {
 #pragma unroll
         for (int i = 0; i < NF; ++i)
-            if (e0 + i < K) sT[e0 + i] = node_value(th[i], sigmoidf(th[i]), node);
+            if (e0 + i < K) sT[e0 + i] = table_value(th[i], sigmoidf(th[i]), node);
         __syncwarp();
         // lane m: subtable m into its subset differences, stored with the
         // table's halves interleaved
@@ -575,7 +571,7 @@ coded_backward_kernel(const uint8_t* __restrict__ codes, long long stride, const
 #pragma unroll
                 for (int ah = 0; ah < 2; ++ah) {
                     const int v = O::to_tree(ah, a);
-                    smem[ah * O::kCopy + 2 * (v & (H - 1)) + (v >> (k - 1))] = node_value(th[i], sg[i], node);
+                    smem[ah * O::kCopy + 2 * (v & (H - 1)) + (v >> (k - 1))] = table_value(th[i], sg[i], node);
                 }
             }
         }

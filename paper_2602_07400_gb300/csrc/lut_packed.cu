@@ -159,7 +159,7 @@ lut_backward_packed_kernel(const float* __restrict__ X, int w_in, long long B, c
             sg[i] = sigmoidf(thn[i]);
             const int a = e0 + i;   // the table's halves interleaved, as packed_quads reads them
             if ((lane & ((1 << SH) - 1)) == 0)
-                sT[2 * (a & (H - 1)) + (a >> (k - 1))] = node == BITLOGIC_NODE_ST ? (thn[i] > 0.f ? 1.f : 0.f) : sg[i];
+                sT[2 * (a & (H - 1)) + (a >> (k - 1))] = table_value(thn[i], sg[i], node);
         }
         float* pst[k];
 #pragma unroll

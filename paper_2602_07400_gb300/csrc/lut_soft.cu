@@ -35,7 +35,7 @@ namespace {
 #define BITLOGIC_BWD_MIN_BLOCKS_SMALL 24  // dtheta-only kernel: blocks per SM (k <= 3, fewer registers)
 #endif
 #ifndef BITLOGIC_NODE_MIN_BLOCKS
-#define BITLOGIC_NODE_MIN_BLOCKS 12  // backward with input gradient: blocks per SM
+#define BITLOGIC_NODE_MIN_BLOCKS 12  // lut_backward_node_kernel: blocks per SM
 #endif
 #ifndef BITLOGIC_FWD_WARPS
 #define BITLOGIC_FWD_WARPS 1
@@ -213,13 +213,6 @@ __device__ __forceinline__ void load_rows(const int* __restrict__ conn, int j, i
     if (bad && lane == 0) flag_index_error();
 }
 
-// Table entry of a node form (bitlogic_node_t): the sigmoid sg of the logit
-// th for the soft LightLUT node, the hard sample [th > 0] for the
-// straight-through node (whose theta gradient still takes the slope of sg).
-__device__ __forceinline__ float table_value(float th, float sg, int node) {
-    return node == BITLOGIC_NODE_ST ? (th > 0.f ? 1.f : 0.f) : sg;
-}
-
 // Per-warp node set-up: connectivity rows (range-checked), table entries of
 // the node form, level-0 constants broadcast to every lane through shared
 // memory.  Lane l (l < 2^(k-1)) keeps the sigmoids of entries 2l and 2l+1
@@ -264,8 +257,8 @@ static_assert(kStages >= 2 && kStages <= 8, "the rings hold 2 to 8 stages");
 
 // ------------------------------------------------------------- forward --
 
-// Scalar forward (any B, any alignment): one warp per (node, batch slice),
-// one sample per lane.
+// Scalar forward (any B and alignment, fan-in below BITLOGIC_FWD_STAGED_MIN_K):
+// one warp per (node, batch slice), one sample per lane.
 template <int k>
 __global__ void __launch_bounds__(kFwdWarps * 32)
 lut_forward_kernel(const float* __restrict__ X, int w_in, long long B,
@@ -296,8 +289,8 @@ lut_forward_kernel(const float* __restrict__ X, int w_in, long long B,
 // Staged forward: one warp per (node, batch slice).  Each lane copies, reads
 // back and evaluates its own 4 samples of a stage, so the ring needs no warp
 // synchronisation: with VEC (B % 4 == 0, chunk % 4 == 0, 16-byte aligned X and
-// Y) 4 consecutive ones in 16-byte pieces, otherwise samples lane + 32 c, 4
-// bytes each.  From fan-in 4 on the table's halves under the top input are
+// Y) 4 consecutive ones in 16-byte pieces, otherwise (fan-in
+// BITLOGIC_FWD_STAGED_MIN_K and more) samples lane + 32 c, 4 bytes each.  From fan-in 4 on the table's halves under the top input are
 // evaluated together on packed pairs (fwd_tree2), the same expressions in
 // half the instructions: 96 registers instead of 125 at fan-in 6, and 16000
 // nodes x 1000 samples, forward and backward, 324 -> 316 us.
@@ -1207,12 +1200,13 @@ int launch_forward(const float* X, int w_in, long long B, const int* conn, const
     const long long ny = (B + chunk - 1) / chunk;
     if (ny > 65535) return BITLOGIC_ERR_SHAPE;
     dim3 grid((unsigned)((w + kFwdWarps - 1) / kFwdWarps), (unsigned)ny);
-    if (vec)
+    if (vec) {
         lut_forward_staged_kernel<k, true><<<grid, kFwdWarps * 32, 0, st>>>(X, w_in, B, conn, theta, w, node, Y, chunk);
-    else if (k >= BITLOGIC_FWD_STAGED_MIN_K)
+    } else if constexpr (k >= BITLOGIC_FWD_STAGED_MIN_K) {
         lut_forward_staged_kernel<k, false><<<grid, kFwdWarps * 32, 0, st>>>(X, w_in, B, conn, theta, w, node, Y, chunk);
-    else
+    } else {
         lut_forward_kernel<k><<<grid, kFwdWarps * 32, 0, st>>>(X, w_in, B, conn, theta, w, node, Y, chunk);
+    }
     return launch_status();
 }
 
