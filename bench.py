@@ -512,7 +512,8 @@ def roofline_of(call, work, per_call_ms, sms, clocks, workload, hbm, sm_max, pea
     issue-rate lane-operations, whichever takes longer at peak), achieved
     rate, peak, fraction (also at the median SM clock sampled during the
     timed region) and the ncu DRAM traffic per launch."""
-    byts, ops, moved = work[call]
+    alg, ops, moved = work[call]
+    byts = min(alg, moved)   # a more compact form (corner codes) moves fewer
     t_s = per_call_ms[call] * 1e-3
     alu_peak = issue_peak(sms, sm_max)
     t_hbm, t_alu = byts / (hbm * 1e9), ops / alu_peak
@@ -528,9 +529,9 @@ def roofline_of(call, work, per_call_ms, sms, clocks, workload, hbm, sm_max, pea
     roof["frac"] = roof["achieved"] / roof["peak"]
     traffic, traffic_note = kernel_traffic(workload, call, (kernels or KERNEL_OF_CALL)[call])
     roof.update({"traffic": traffic, "traffic_source": traffic_note,
-                 "traffic_over_algorithmic": (traffic / byts) if traffic else None,
+                 "traffic_over_algorithmic": (traffic / alg) if traffic else None,
                  "kernel": (kernels or KERNEL_OF_CALL)[call], "call": call,
-                 "ms_per_launch": per_call_ms[call], "algorithmic_bytes": byts, "bytes_moved": moved,
+                 "ms_per_launch": per_call_ms[call], "algorithmic_bytes": alg, "bytes_moved": moved,
                  "algorithmic_ops": ops,
                  "peak_source": f"{peak_kind} HBM copy ({hbm:.1f} GB/s); {sms} SMs (read from the device) x "
                                 f"{FP32_LANES_PER_SM} lanes x {sm_max:.0f} MHz (alu: one issue per lane and clock)"})
@@ -541,8 +542,11 @@ def calls_table(work, per_call_ms, hbm, workload=None, kernels=None):
     out = {}
     for n, t in per_call_ms.items():
         b_, o_, m_ = work[n]
+        # the fraction of the measured copy rate by the bytes that the call must
+        # move: the algorithmic ones, or what a more compact form (corner codes)
+        # moves in their place
         e = {"ms": round(t, 5), "alg_GB/s": round(b_ / (t * 1e-3) / 1e9, 1),
-             "frac_hbm": round(b_ / (t * 1e-3) / 1e9 / hbm, 3),
+             "frac_hbm": round(min(b_, m_) / (t * 1e-3) / 1e9 / hbm, 3),
              "Tops/s": round(o_ / (t * 1e-3) / 1e12, 2) if o_ else None}
         if m_ != b_:
             e["moved_GB/s"] = round(m_ / (t * 1e-3) / 1e9, 1)

@@ -183,6 +183,23 @@ def test_byte_wire_layer1_work_and_kernel_names():
     assert bench.route_of_step(st)["layer1_wires"].startswith("bits")
 
 
+def test_corner_code_calls_are_rated_by_the_bytes_they_move():
+    # codes and corner sums take the place of fp32 rows and per-edge terms: a
+    # call's share of the copy rate counts what it moves
+    import bench
+    from paper_2602_07400_gb300 import synth
+    wl = synth.WORKLOADS["cifar100"]
+    work = bench.call_work(wl, 2048, fuse_dy1=True, bytes1=True, bits1=True, codes1=True)
+    per_call = {"forward1": 0.091, "backward1": 0.055, "forward2": 0.896, "backward2": 2.78}
+    rows = bench.calls_table(work, per_call, 6767.1)
+    for n, t in per_call.items():
+        assert work[n][2] < work[n][0]
+        want = min(work[n][0], work[n][2]) / (t * 1e-3) / 1e9 / 6767.1
+        assert abs(rows[n]["frac_hbm"] - want) < 1e-3 and rows[n]["frac_hbm"] < 1.05
+    roof = bench.roofline_of("backward1", work, per_call, 152, {}, "none", 6767.1, 2070.0, "measured")
+    assert roof["bound"] == "hbm" and roof["frac"] < 1.05
+
+
 def test_hard_roofline_uses_the_measured_mix_rate():
     # the hard layer's peak is the measured issue rate of its instruction mix
     # (per SM and clock) at the sampled clock; the issue-rate fraction stays
