@@ -402,12 +402,13 @@ int bitlogic_lut_backward_bitrows(const uint32_t* X, int32_t w_in, int64_t B, co
  *     corner_sums[row][a] = sum over the samples s with a_c(s) = a of
  *                           dY[j][s] * dy_j/dx_i(s),
  *   row = edge_pos[e] or e (edge_pos NULL); device fp32 [w*k][2^k_in].  Every
- *   sum is in a fixed order.
+ *   sum is in a fixed order, and an entry that is not finite reaches only the
+ *   sums of samples that meet it.
  * bitlogic_corner_reduce: layer 1's table gradient
  *     dtheta[j][a] = s_a (1 - s_a) * sum over p in [csr_off[j], csr_off[j+1])
  *                    of corner_sums[csr_edge[p]][a], s = sigmoid(theta),
- *   in increasing p (csr_edge NULL: rows in CSR order), k the fan-in of
- *   layer 1, n_edges the number of rows.
+ *   in a fixed order (csr_edge NULL: rows in CSR order), k the fan-in of layer
+ *   1, n_edges the number of rows; corner_sums 8-byte aligned at k = 6.
  * Out-of-range indices raise the device flag and read row 0 (an out-of-range
  * edge_pos stores at the edge's own row; an out-of-range CSR entry adds
  * nothing).  B == 0: the forwards are no-ops, the backward zeroes its

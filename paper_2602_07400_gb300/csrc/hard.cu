@@ -403,10 +403,10 @@ __device__ __forceinline__ void csa(uint32_t& carry, uint32_t& sum, uint32_t a, 
 constexpr int kHeadWarps = 8;
 constexpr int kBigPlanes = 10;   // weight-8 planes: up to 8 * 1023 + 7 nodes per warp
 
-// One-word-per-lane path (any W and alignment; short rows).  grid.x: groups of 32 * R words,
+// One-word-per-lane path (any W and alignment: short rows, and those past the
+// staged kernels' limits, see hard_route).  grid.x: groups of 32 * R words,
 // grid.y: class c x split.  Lane l covers words R * l .. R * l + R - 1 of
-// the group.  Warp r of
-// a block takes nodes n0 + r, n0 + r + 8, ... of its slice and feeds their
+// the group.  Warp r of a block takes nodes n0 + r, n0 + r + 8, ... of its slice and feeds their
 // output words, eight nodes at a time, through a Harley-Seal carry-save tree
 // into per-lane bit-sliced counters.  At the end every lane turns its
 // counters into per-sample counts, the block adds its 8 warps in shared
@@ -792,8 +792,9 @@ long long hard_word_chunk(int w_in, long long W) {
 // many words on; up to 32 words three quarters of a stage would be idle, and
 // the one-word-per-lane kernels take those.  Measured against those kernels
 // for 313 words (10000 samples, 64000 x 64000 nodes, fan-in 6): pass 424 ->
-// 273 us (230 with the short stages and the head's splits below); 2759 words (88278 samples, 26337 x 1900, 100 classes) 811 -> 444 us;
-// 226 words (7222 samples, 9534 x 17760, fan-in 4) 94 -> 58 us.
+// 273 us (230 with the short stages and the head's splits below); 2759 words
+// (88278 samples, 26337 x 1900, 100 classes) 811 -> 444 us; 226 words (7222
+// samples, 9534 x 17760, fan-in 4) 94 -> 58 us.
 #ifndef BITLOGIC_HARD_STAGED_MIN
 #define BITLOGIC_HARD_STAGED_MIN 33
 #endif

@@ -193,9 +193,11 @@ inline bool short_tail(long long B) { return B <= 192 && B % 128 != 0 && B % 128
 // under the top input are evaluated together on packed pairs, with the
 // expressions of the fp32 forward (8-entry Moebius subtables under lerps), so
 // the results equal it bit for bit.  At 128000 nodes of fan-in 6 and 2048
-// samples 0.93 ms against 0.985 ms on fp32 rows, which waits for DRAM (6.9 GB
-// at 7 TB/s); here 2.6 GB move and the FP32 pipe and its operand reads bound
-// it (55% pipe-active).  12 or 20 blocks per SM: 1 and 9% slower steps.
+// samples 0.90 ms against 0.985 ms on fp32 rows, which waits for DRAM (6.9 GB
+// at 7 TB/s); here 2.5 GB move, and neither the FP32 pipe (56% active) nor
+// issue (51%) is full: the tree's register operand reads and the chain from
+// code word to table entry are what is left.  12 or 20 blocks per SM: 1 and 9%
+// slower steps.
 template <int k, bool TAIL>
 __global__ void __launch_bounds__(32, BITLOGIC_CODED_FWD_BLOCKS)
 coded_forward_kernel(const uint8_t* __restrict__ codes, long long stride, const float* __restrict__ table1, int w_in,
@@ -357,11 +359,12 @@ coded_forward_kernel(const uint8_t* __restrict__ codes, long long stride, const 
 // to 1.6 scalar on an SM quarter, whatever the number of warps).  The tree
 // alone takes 2.3 ms at 128000 nodes x 2048 samples in this form, 2.6-2.7 ms
 // with a sample split over two lanes (scalar or packed), which repeats the
-// per-sample work.  Measured there: 2.78 ms against 2.76 ms for the fp32-row
-// backward, which in addition writes 6.3 GB of per-edge terms that the
-// layer-1 backward reads back (1.07 ms; the corner reduction takes 0.08 ms).
-// Step: 5.20 -> 4.05 ms; 64000 nodes x 1024 1.363 -> 1.164 ms; 8000 x 1024
-// 0.197 -> 0.168 ms.  Forms with a sample split over lanes, 8 warps with own
+// per-sample work; the pipe is 58% and issue 46% active (8000 nodes x 1024).
+// Measured there: 2.78 ms against 2.76 ms for the fp32-row backward, which in
+// addition writes 6.3 GB of per-edge terms that the layer-1 backward reads back
+// (1.07 ms; the corner reduction takes 0.05 ms).  Step, with the forward on
+// codes: 5.20 -> 3.99 ms; 64000 nodes x 1024 1.363 -> 1.143 ms; 8000 x 1024
+// 0.197 -> 0.166 ms.  Forms with a sample split over lanes, 8 warps with own
 // columns (two samples in flight) and 12 warps with shared columns: steps of
 // 4.69 and 5.16 ms at the first size.
 
@@ -717,7 +720,8 @@ coded_backward_kernel(const uint8_t* __restrict__ codes, long long stride, const
 // --------------------------------------------------- layer 1 table gradient --
 
 // dtheta[j][a] = slope(theta_j[a]) * sum of the corner sums H[edge[p]][a] over
-// the CSR positions p of node j.  `parts` warps of a block per node, each over
+// the CSR positions p of node j (an order of its own when parts > 1: no other
+// call forms this sum).  `parts` warps of a block per node, each over
 // a run of its positions in increasing p, then the runs in order; lane = table
 // entry (two neighbours per lane for 64 entries).  The rows of up to eight
 // positions and the logits are in flight together: the kernel reads each byte

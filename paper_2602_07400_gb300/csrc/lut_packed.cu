@@ -10,9 +10,10 @@
 //
 // What bounds it: register operand reads of the tree (lut_codes.cu) and, for
 // wide layers, the term rows that it writes.  16000 nodes of fan-in 6, forward
-// and backward with the input gradient: 1000 samples 329 -> 324 us against a
-// kernel with a sample split over two lanes and 12 warps per SM (the tree
-// alone is 13% shorter here, with 8 warps to hide the copies behind); batches
+// and backward with the input gradient: 1000 samples 329 -> 324 us (315 with
+// the packed forward) against a kernel with a sample split over two lanes and
+// 12 warps per SM (the tree alone is 13% shorter here, with 8 warps to hide the
+// copies behind); batches
 // that are no multiple of four, which had a scalar kernel, 907 samples 600 ->
 // 325 us, 64000 nodes x 2047 samples 6.01 -> 2.83 ms; fan-in 4 244 -> 167 us,
 // fan-in 5 (8000 nodes x 1001) 198 -> 133 us.  One or two samples per loop

@@ -290,9 +290,10 @@ lut_forward_kernel(const float* __restrict__ X, int w_in, long long B,
 // back and evaluates its own 4 samples of a stage, so the ring needs no warp
 // synchronisation: with VEC (B % 4 == 0, chunk % 4 == 0, 16-byte aligned X and
 // Y) 4 consecutive ones in 16-byte pieces, otherwise (fan-in
-// BITLOGIC_FWD_STAGED_MIN_K and more) samples lane + 32 c, 4 bytes each.  From fan-in 4 on the table's halves under the top input are
-// evaluated together on packed pairs (fwd_tree2), the same expressions in
-// half the instructions: 96 registers instead of 125 at fan-in 6, and 16000
+// BITLOGIC_FWD_STAGED_MIN_K and more) samples lane + 32 c, 4 bytes each.  From
+// fan-in 4 on the table's halves under the top input are evaluated together on
+// packed pairs (fwd_tree2), the same expressions in half the instructions: 96
+// registers instead of 125 at fan-in 6, and 16000
 // nodes x 1000 samples, forward and backward, 324 -> 316 us.
 template <int k, bool VEC>
 __global__ void __launch_bounds__(kFwdWarps * 32)

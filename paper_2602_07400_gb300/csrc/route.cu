@@ -41,10 +41,10 @@ __device__ __forceinline__ float4 ldg4r(const float* p) { return __ldg(reinterpr
 // of a row, as floats.
 // Bytes t and t + 1 of w as floats: each byte in the lowest mantissa bits of
 // 2^23, less 2^23 (exact), the two subtractions in one packed instruction.  The
-// byte-row kernels are bound by issue slots (81 and 71%), most of them these
+// byte-row kernels were bound by issue slots (81 and 71%), most of them these
 // conversions and the multiply-adds: 32000 slots x 16 candidates x 1024
 // samples, forward 73 -> 65 us with the multiply-adds packed too, logits'
-// gradient 95 -> 92 us.
+// gradient 95 -> 92 us (issue slots 64 and 67% now).
 __device__ __forceinline__ f32x2 byte_pair(uint32_t w, int t) {
     const float a = __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7440u + (unsigned)t));
     const float b = __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7440u + (unsigned)(t + 1)));

@@ -69,9 +69,10 @@ def test_layer2_on_codes(k, k1, w1, w, B, node):
         check_exact(Y.cpu().numpy().astype(np.float64), want, "y (binary inputs)")
     else:
         check_fwd(Y, want, "y")
-    # the fp32-row forward evaluates the same expressions
+    # the fp32-row forward evaluates the same expressions (at fan-in 4 on ragged
+    # rows it is the lerp tree of the scalar kernel, which rounds differently)
     Yr = torch.empty_like(Y)
-    if B % 4 == 0:
+    if B % 4 == 0 or k >= 5:
         bl.bitlogic_lut_forward_node(Y1, dev(conn), dev(theta), Yr, node)
         check_exact(Y.cpu().numpy(), Yr.cpu().numpy(), "y vs fp32 rows")
     group = 2
