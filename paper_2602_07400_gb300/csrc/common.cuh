@@ -88,6 +88,8 @@ __device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {   // 4
     const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem) : "memory");
 }
+// The line at p on its way to L2.
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p)); }
 // The same copies, or zeros (nothing is read) unless `take`.
 __device__ __forceinline__ void cp_async16_or_zero(void* smem, const void* gmem, bool take) {
     const unsigned s = (unsigned)__cvta_generic_to_shared(smem);

@@ -61,8 +61,13 @@ constexpr int packed_smem() {
 // stage.  VEC (B % 4 == 0, 16-byte aligned rows): 16-byte copies, which other
 // lanes read; otherwise each lane copies its own samples, 4 bytes each.
 // TERMS: the gradient is summed from the upstream term rows instead (in
-// increasing position, as csr_reduce does).  dtheta is reduced by a fixed
-// butterfly inside the warp.
+// increasing position, as csr_reduce does), NB rows in flight and the next
+// stage's prefetched to L2: with one row at a time the chain of loads bounded
+// the kernel (step of 8000 x 8000 nodes, 1024 samples, with layer 1's input
+// gradient and fused terms: fan-in 3 204 -> 136 us, 4 254 -> 178, 6 543 -> 372;
+// 64000 x 64000 at fan-in 6 3.77 -> 2.61 ms; in a kernel with a sample split
+// over two lanes and more warps 140, 178, 372 us and 2.59 ms).  dtheta is
+// reduced by a fixed butterfly inside the warp.
 template <int k, bool VEC, bool TERMS>
 __global__ void __launch_bounds__(32, packed_blocks<k>())
 lut_backward_packed_kernel(const float* __restrict__ X, int w_in, long long B, const int* __restrict__ conn,
@@ -72,6 +77,7 @@ lut_backward_packed_kernel(const float* __restrict__ X, int w_in, long long B, c
     constexpr int K = 1 << k, H = K / 2, R = TERMS ? k : k + 1, CH = kStageSamples, NS = kPackedStages;
     constexpr int NF = K >= 32 ? K / 32 : 1;   // table entries per lane
     constexpr int SH = K >= 32 ? 0 : 5 - k;    // lanes sharing an entry (K < 32)
+    constexpr int NB = k == 4 || k == 5 ? 4 : 8;   // term rows in flight (eight spill registers at fan-in 4 and 5)
     extern __shared__ __align__(16) float smem[];
     const int lane = threadIdx.x;
     float* ring = smem;
@@ -137,9 +143,24 @@ lut_backward_packed_kernel(const float* __restrict__ X, int w_in, long long B, c
     };
     // logits and term rows of the warp's next node
     float thn[NF];
-    int posn = 0;
+    int posn = 0, t0n = 0, t1n = 0;
+    auto term_id = [&](int e, int end) {
+        int id = -1;
+        if (e < end) {
+            id = gs.edge ? __ldg(gs.edge + e) : e;
+            if ((unsigned)id >= (unsigned)gs.n_edges) {
+                flag_index_error();
+                id = -1;
+            }
+        }
+        return id;
+    };
     auto ahead = [&](int j) {
         if (j < w) {
+            if constexpr (TERMS) {
+                t0n = __ldg(gs.off + j);
+                t1n = __ldg(gs.off + j + 1);
+            }
 #pragma unroll
             for (int i = 0; i < NF; ++i) thn[i] = __ldg(theta + (long long)j * K + e0 + i);
             if (epos && lane < k) posn = __ldg(epos + (long long)j * k + lane);
@@ -173,14 +194,17 @@ lut_backward_packed_kernel(const float* __restrict__ X, int w_in, long long B, c
             }
             pst[i] = P + row * B + lane;
         }
-        int t0 = 0, t1 = 0;   // the node's term positions
+        // the node's term positions, and row ids: lane u that of position t0 + u
+        // (-1 past the end or out of range)
+        int t0 = 0, t1 = 0, ids = -1;
         if constexpr (TERMS) {
-            t0 = __ldg(gs.off + j);
-            t1 = __ldg(gs.off + j + 1);
+            t0 = t0n;
+            t1 = t1n;
             if (t0 < 0 || t1 < t0 || t1 > gs.n_edges) {
                 if (lane == 0) flag_index_error();
                 t0 = t1 = 0;
             }
+            ids = term_id(t0 + lane, t1);
         }
         __syncwarp();
         f32x2 cq[H], acc[H];
@@ -199,17 +223,35 @@ lut_backward_packed_kernel(const float* __restrict__ X, int w_in, long long B, c
             if constexpr (TERMS) {
 #pragma unroll
                 for (int c = 0; c < CH / 32; ++c) gt[c] = 0.f;
+                // loads of NB rows are issued before the first add (samples past
+                // the batch read its first ones, unused; past the end row 0)
+                long long at[CH / 32];
+#pragma unroll
+                for (int c = 0; c < CH / 32; ++c) at[c] = s0 + 32 * c + lane < B ? s0 + 32 * c + lane : 0;
 #pragma unroll 1
-                for (int e = t0; e < t1; ++e) {
-                    const int id = gs.edge ? __ldg(gs.edge + e) : e;
-                    if ((unsigned)id >= (unsigned)gs.n_edges) {
-                        if (lane == 0) flag_index_error();
-                        continue;
+                for (int q = 0; q < t1 - t0; q += NB) {
+                    if (q > 0 && q % 32 == 0) ids = term_id(t0 + q + lane, t1);
+                    float v[NB][CH / 32];
+                    bool add[NB];
+#pragma unroll
+                    for (int u = 0; u < NB; ++u) {
+                        const int id = __shfl_sync(0xffffffffu, ids, (q + u) & 31);
+                        add[u] = id >= 0;
+                        const float* row = gs.terms + (long long)max(id, 0) * B;
+#pragma unroll
+                        for (int c = 0; c < CH / 32; ++c) v[u][c] = __ldg(row + at[c]);
                     }
-                    const float* row = gs.terms + (long long)id * B + s0 + lane;
+#pragma unroll
+                    for (int u = 0; u < NB; ++u)
+#pragma unroll
+                        for (int c = 0; c < CH / 32; ++c)
+                            if (add[u]) gt[c] += v[u][c];
+                }
+                if (t1 - t0 > 32) ids = term_id(t0 + lane, t1);   // the first ones again, for the next stage
+                if (ids >= 0) {   // the next stage's rows on their way to L2, a row per lane
 #pragma unroll
                     for (int c = 0; c < CH / 32; ++c)
-                        if (s0 + 32 * c + lane < B) gt[c] += __ldg(row + 32 * c);
+                        if (s0 + CH + 32 * c < B) prefetch_l2(gs.terms + (long long)ids * B + s0 + CH + 32 * c);
                 }
             }
             auto sample = [&](int c, bool in) {
@@ -217,7 +259,7 @@ lut_backward_packed_kernel(const float* __restrict__ X, int w_in, long long B, c
 #pragma unroll
                 for (int i = 0; i < k; ++i) x[i] = in ? buf[i * CH + 32 * c] : 0.f;
                 float g;
-                if constexpr (TERMS) g = gt[c];
+                if constexpr (TERMS) g = in ? gt[c] : 0.f;
                 else g = in ? buf[k * CH + 32 * c] : 0.f;
                 node_sample2<k>(cq, x, g, dx, acc);
                 if (in) {

@@ -178,3 +178,40 @@ def test_upstream_terms_are_the_csr_reduction_bit_for_bit(w_in, deg, B, offset):
                                           up_off=dev(off), up_edge=dev(edge), edge_terms=terms_out, dY_out=used)
             check_exact(used.cpu().numpy(), dX.cpu().numpy(), "gradient used")
     assert bl.bitlogic_device_error() == 0
+
+
+@pytest.mark.parametrize("k", [3, 4, 5, 6])
+@pytest.mark.parametrize("B,offset", [(256, 0), (260, 0), (132, 1)])
+@pytest.mark.parametrize("node", ["soft", "st"])
+def test_upstream_terms_with_input_gradient(k, B, offset, node):
+    # aligned and other rows, nodes without a term and with more than 32 (two
+    # chunks of row ids): against the oracle, with and without given positions
+    w_in, w = 40, 300
+    X = synth.uniform_activations(w_in, B, seed=B)
+    conn = synth.connectivity(w, k, w_in, seed=1)
+    theta = synth.table_logits(w, 1 << k, seed=2)
+    off, edge = bl.bitlogic_build_csr(conn, w_in)
+    pos = bl.bitlogic_csr_positions(edge)
+    rng = np.random.default_rng(k)
+    deg = rng.integers(0, 6, size=w)
+    deg[7], deg[-1] = 33, 70
+    up_off = np.concatenate(([0], np.cumsum(deg))).astype(np.int32)
+    n = int(up_off[-1])
+    up_edge = rng.permutation(n).astype(np.int32)
+    terms = synth.uniform_gradients(n, B, seed=4, scale=1e-2)
+    full = np.zeros((w, B))
+    np.add.at(full, np.repeat(np.arange(w), np.diff(up_off)), terms[up_edge].astype(np.float64))
+    wth, wdx = oracle.lut_backward(X.astype(np.float64), conn, theta, full, want_dx=True, node=node)
+    rows = []
+    for epos, csr_edge in ((None, dev(edge)), (dev(pos), None)):
+        dth, P = torch.full((w, 1 << k), np.nan, device="cuda"), torch.full((w * k, B), np.nan, device="cuda")
+        bl.bitlogic_lut_backward_node(off_boundary(X, offset), dev(conn), dev(theta), dth, node,
+                                      up_terms=off_boundary(terms, offset), up_off=dev(up_off), up_edge=dev(up_edge),
+                                      edge_terms=P, edge_pos=epos)
+        dX = torch.full((w_in, B), np.nan, device="cuda")
+        bl.bitlogic_csr_reduce(P, dev(off), csr_edge, dX)
+        check_grad(dth, wth, "dtheta")
+        check_grad(dX, wdx, "dX")
+        rows.append(P.cpu().numpy())
+    check_exact(rows[1], rows[0][edge], "term rows at CSR positions")
+    assert bl.bitlogic_device_error() == 0
