@@ -571,9 +571,10 @@ constexpr size_t node_smem_bytes() {
            (size_t)kNodesPerBlock * (1 << k) * sizeof(float);
 }
 
-// Staged backward for fan-in 2 with the input gradient, and for every fan-in
-// from 2 on without it when the gradient comes from upstream terms (fan-in 3
-// and more with the input gradient: lut_packed.cu).  A block holds
+// Staged backward of 16-byte rows: for fan-in 2 with the input gradient, for
+// fan-in 3 and 4 with it over large inputs (otherwise and from fan-in 5 on:
+// lut_packed.cu), and for every fan-in from 2 on without it when the gradient
+// comes from upstream terms.  A block holds
 // kNodesPerBlock nodes with kWarpsPerNode
 // warps each (by default one warp per node and per block, over the whole
 // batch); each warp of a node takes a contiguous range of its 128-sample
@@ -1212,23 +1213,30 @@ int launch_forward(const float* X, int w_in, long long B, const int* conn, const
 }
 
 template <int k, bool WANT_DX, bool TERMS>
+int launch_backward_staged(const float* X, int w_in, long long B, const int* conn, const float* theta,
+                           int w, int node, const GradSource& gs, float* dtheta, float* P, const int* epos,
+                           float* dY_out, cudaStream_t st) {
+    constexpr size_t smem = node_smem_bytes<k, TERMS>();
+    // term rows at caller-given positions: a separate instantiation, so the
+    // common form compiles without the position lookups
+    auto kern = (WANT_DX && epos) ? lut_backward_node_kernel<k, WANT_DX, TERMS, WANT_DX>
+                                  : lut_backward_node_kernel<k, WANT_DX, TERMS, false>;
+    if (smem > 48 * 1024 &&
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        return BITLOGIC_ERR_CUDA;
+    kern<<<(unsigned)((w + kNodesPerBlock - 1) / kNodesPerBlock), kBwdWarps * 32, smem, st>>>(
+        X, w_in, B, conn, theta, w, node, gs, dtheta, P, epos, dY_out);
+    return launch_status();
+}
+
+template <int k, bool WANT_DX, bool TERMS>
 int launch_backward_impl(const float* X, int w_in, long long B, const int* conn, const float* theta,
                          int w, int node, const GradSource& gs, float* dtheta, float* P, const int* epos,
                          float* dY_out, bool staged, cudaStream_t st) {
     if constexpr (k >= 2) {
-        if (staged) {
-            constexpr size_t smem = node_smem_bytes<k, TERMS>();
-            // term rows at caller-given positions: a separate instantiation,
-            // so the common form compiles without the position lookups
-            auto kern = (WANT_DX && epos) ? lut_backward_node_kernel<k, WANT_DX, TERMS, WANT_DX>
-                                          : lut_backward_node_kernel<k, WANT_DX, TERMS, false>;
-            if (smem > 48 * 1024 &&
-                cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-                return BITLOGIC_ERR_CUDA;
-            kern<<<(unsigned)((w + kNodesPerBlock - 1) / kNodesPerBlock), kBwdWarps * 32, smem, st>>>(
-                X, w_in, B, conn, theta, w, node, gs, dtheta, P, epos, dY_out);
-            return launch_status();
-        }
+        if (staged)
+            return launch_backward_staged<k, WANT_DX, TERMS>(X, w_in, B, conn, theta, w, node, gs, dtheta, P, epos,
+                                                             dY_out, st);
     }
     dim3 grid((unsigned)((w + kFwdWarps - 1) / kFwdWarps));
     lut_backward_kernel<k, WANT_DX, TERMS><<<grid, kFwdWarps * 32, 0, st>>>(X, w_in, B, conn, theta, w, node,
@@ -1259,7 +1267,25 @@ int launch_backward(const float* X, int w_in, long long B, const int* conn, cons
             X, w_in, B, conn, theta, w, gs.dY, gs.group, dtheta, dY_out);
         return launch_status();
     }
-    // with the input gradient: fan-in 3 and more on packed pairs
+    // with the input gradient: fan-in 3 and more on packed pairs; but fan-in 3
+    // and 4 on 16-byte rows stay with the staged kernel where the input is too
+    // large for half of L2 and the batch long (per-edge terms from dY rows,
+    // staged against packed: 32000 nodes of fan-in 4, 1024 samples over 64000
+    // rows 166, 198 us, over 8000 rows 139, 134; 12000, 2048 samples over 8000
+    // rows 111, 129, over 1000 100, 91; 64000, 384 samples over 64000 rows 136,
+    // 126; fan-in 3: 12000, 1024 samples over 64000 rows 52, 57, 32000 of 512
+    // samples over 64000 65, 68, of 256 samples 41, 36).  A layer with a row per
+    // slot (w_in = w k, as a routed one) reads each row once, in order, and stays
+    // with the packed kernel (routed step of 8000 x 8000 nodes, 4 candidates, 512
+    // samples 204, 194 us).  The rule is the same for both sources of the
+    // gradient, which give the same bits.
+    if constexpr (k == 3 || k == 4) {
+        if (P && staged && B >= 512 && (long long)w_in * B >= 16000000 && (long long)w * k != w_in)
+            return terms ? launch_backward_staged<k, true, true>(X, w_in, B, conn, theta, w, node, gs, dtheta, P, epos,
+                                                                 dY_out, st)
+                         : launch_backward_staged<k, true, false>(X, w_in, B, conn, theta, w, node, gs, dtheta, P, epos,
+                                                                  dY_out, st);
+    }
     if constexpr (k >= 3) {
         if (P) return launch_backward_packed(k, X, w_in, B, conn, theta, w, node, gs, dtheta, P, epos, dY_out, st);
     } else if (P) {

@@ -215,3 +215,31 @@ def test_upstream_terms_with_input_gradient(k, B, offset, node):
         rows.append(P.cpu().numpy())
     check_exact(rows[1], rows[0][edge], "term rows at CSR positions")
     assert bl.bitlogic_device_error() == 0
+
+
+@pytest.mark.parametrize("k", [3, 4])
+@pytest.mark.parametrize("B", [512, 516])
+@pytest.mark.parametrize("over", [False, True])
+def test_large_inputs_take_the_staged_kernel(k, B, over):
+    # both sides of the line, for both sources of the gradient
+    w_in, w = -(-16000000 // B) - (0 if over else 1), 90
+    X = synth.uniform_activations(w_in, B, seed=B)
+    conn = synth.connectivity(w, k, w_in, seed=1)
+    theta = synth.table_logits(w, 1 << k, seed=2)
+    dY = synth.uniform_gradients(w, B, seed=3, scale=1e-2)
+    Xd, rows = dev(X), np.unique(conn)
+    small = np.searchsorted(rows, conn).astype(np.int32)   # the same layer on the rows that it reads
+    wth, wdx = oracle.lut_backward(X[rows].astype(np.float64), small, theta, dY.astype(np.float64), want_dx=True)
+    off, edge = bl.bitlogic_build_csr(small, len(rows))
+    outs = []
+    for source in (dict(dY=dev(dY)), dict(up_terms=dev(dY), up_off=dev(np.arange(w + 1, dtype=np.int32)))):
+        dth, P = torch.full((w, 1 << k), np.nan, device="cuda"), torch.full((w * k, B), np.nan, device="cuda")
+        bl.bitlogic_lut_backward_node(Xd, dev(conn), dev(theta), dth, "soft", edge_terms=P, **source)
+        dX = torch.full((len(rows), B), np.nan, device="cuda")
+        bl.bitlogic_csr_reduce(P, dev(off), dev(edge), dX)
+        check_grad(dth, wth, "dtheta")
+        check_grad(dX, wdx, "dX")
+        outs.append((dth.cpu().numpy(), P.cpu().numpy()))
+    for a, b in zip(*outs):
+        check_exact(a, b, "gradient from rows and from terms")
+    assert bl.bitlogic_device_error() == 0
