@@ -788,31 +788,42 @@ long long hard_word_chunk(int w_in, long long W) {
     return c < W ? c : W;
 }
 
-// Rows that the 16-byte form cannot take go to the staged kernels from this
-// many words on; up to 32 words three quarters of a stage would be idle, and
-// the one-word-per-lane kernels take those.  Measured against those kernels
-// for 313 words (10000 samples, 64000 x 64000 nodes, fan-in 6): pass 424 ->
-// 273 us (230 with the short stages and the head's splits below); 2759 words
-// (88278 samples, 26337 x 1900, 100 classes) 811 -> 444 us; 226 words (7222
-// samples, 9534 x 17760, fan-in 4) 94 -> 58 us.
-#ifndef BITLOGIC_HARD_STAGED_MIN
-#define BITLOGIC_HARD_STAGED_MIN 33
-#endif
-constexpr long long kStagedMinWords = BITLOGIC_HARD_STAGED_MIN;
-
 // The kernels for rows of W words: 16-byte staged (W % 4 == 0, 16-byte aligned
-// rows, 32-bit offsets in 16-byte units), 4-byte staged (any other rows with
-// 32-bit offsets in words, as long as their groups of stages fit grid.y), or
-// one word per lane, which puts word groups on grid.x (head) or takes longer
-// chunks (layer) and so has no such limit.
+// rows, 32-bit offsets in 16-byte units); 4-byte staged (any other rows with
+// 32-bit offsets in words, as long as their groups of stages fit grid.y); or one
+// word per lane, which puts word groups on grid.x (head) or takes longer chunks
+// (layer) and so has no such limit.
+//
+// Head on other rows: 4-byte staged from 33 words on; up to 32 words three
+// quarters of a stage would be idle.  Against the one-word kernel, 0.3 to 0.9 of
+// its time over fan-in 2, 4 and 6, 1 to 100 classes, 500 to 64000 nodes and 33
+// to 625 words (7222 samples, 17760 nodes of fan-in 4: pass 94 -> 58 us).
+//
+// Layer on other rows: the one-word kernel has no copies to issue, and only from
+// fan-in 5 on is the tree long enough to gain from the ring (64000 nodes, 313
+// words: fan-in 2 23.6 us one-word, 29.4 staged; fan-in 6 0.90 of its time;
+// 32000 nodes of fan-in 4, 469 words 28.8, 41.7 us; 21504 input rows of 2501
+// words, fan-in 6 0.56 of its time, fan-in 4 0.9).  It also leaves SMs idle when
+// few nodes run over long rows (500 nodes of fan-in 4, 1251 words: 0.42 of its
+// time staged; 2000: 0.8; fan-in 2, 1600 input rows of 10001 words, 1000 nodes:
+// 0.48).  The lines were drawn from 1000 sizes; over them the rule takes 0.88 of
+// the one-word kernel's time and at worst 1.07 of it.
 enum HardRoute { kOneWord = 0, kStaged4 = 1, kStaged16 = 2 };
 constexpr long long kGridY = 65535;
-HardRoute hard_route(int w_in, long long W, bool aligned, bool head) {
+HardRoute hard_route(int k, int w_in, int w, long long W, bool aligned, bool head, int sms) {
     const unsigned long long rows = (unsigned long long)w_in;
     if (W % 4 == 0 && aligned && rows * (unsigned long long)(W / 4) < (1ull << 32)) return kStaged16;
     const long long per_y = head ? kStageWords : kLayerNS * kStageWords;
-    return W >= kStagedMinWords && rows * (unsigned long long)W < (1ull << 32) && W <= kGridY * per_y ? kStaged4
-                                                                                                  : kOneWord;
+    if (W < 33 || rows * (unsigned long long)W >= (1ull << 32) || W > kGridY * per_y) return kOneWord;
+    if (head) return kStaged4;
+    const long long chunk = hard_word_chunk(w_in, W), chunks = (W + chunk - 1) / chunk;
+    const long long warps = w * chunks;   // of the one-word kernel
+    bool staged = warps < 8ll * sms && W >= (k >= 4 ? 200 : 300);
+    if (k >= 5) staged = staged || W >= 300 || (k == 6 && w >= 32000);
+    else if (k == 4) staged = staged || (w <= 16ll * sms && W >= 200 && (chunks == 1 || chunk >= 1000)) ||
+                              (chunks > 1 && (long long)w * W >= 8000000);
+    else staged = staged || (chunks > 1 && chunk >= 4000 && warps <= (k == 1 ? 40ll : 20ll) * sms);
+    return staged ? kStaged4 : kOneWord;
 }
 
 // Splits of a class for the staged head when there are few word groups: the
@@ -858,7 +869,7 @@ int launch_hard(const uint32_t* xp, int w_in, long long N, const int* conn, cons
                 int w, uint32_t* yp, int C, int* counts, int* pred, cudaStream_t st) {
     const long long W = (N + 31) / 32;
     const uint32_t tail_mask = (N % 32) ? ((1u << (N % 32)) - 1u) : 0xffffffffu;
-    const HardRoute route = hard_route(w_in, W, aligned16(xp) && (!yp || aligned16(yp)), C > 0);
+    const HardRoute route = hard_route(k, w_in, w, W, aligned16(xp) && (!yp || aligned16(yp)), C > 0, sm_count());
     const bool vec4 = route == kStaged16, staged = route != kOneWord;
     if (C == 0) {
         if (staged) {
@@ -939,8 +950,9 @@ using namespace bitlogic;
 BITLOGIC_ERROR_READER(hard)
 
 // The route of a hard call, for host checks of the rule (HardRoute).
-extern "C" int bitlogic_internal_hard_route(int32_t w_in, int64_t words, int32_t aligned, int32_t head) {
-    return hard_route(w_in, words, aligned != 0, head != 0);
+extern "C" int bitlogic_internal_hard_route(int32_t k, int32_t w_in, int32_t w, int64_t words, int32_t aligned,
+                                            int32_t head, int32_t sms) {
+    return hard_route(k, w_in, w, words, aligned != 0, head != 0, sms);
 }
 
 extern "C" int bitlogic_binarize_tables(const float* theta, int32_t w, int32_t k,

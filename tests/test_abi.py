@@ -293,19 +293,39 @@ def test_compute_calls_reject_host_tensors():
         bl.bitlogic_issue_probe("lop3", 1, torch.zeros(8, dtype=torch.int32))
 
 
+def _hard_route(k, w_in, w, words, aligned, head):
+    fn = bl.load().bitlogic_internal_hard_route
+    fn.argtypes = [ctypes.c_int32, ctypes.c_int32, ctypes.c_int32, ctypes.c_int64] + [ctypes.c_int32] * 3
+    return fn(k, w_in, w, words, aligned, head, 152)
+
+
 def test_hard_route_of_long_rows():
     # 4-byte staged rows only while their groups of stages (128 words in the
     # head, 384 in a layer) fit grid.y, beyond that the one-word kernels; the
     # 16-byte form keeps aligned rows of whole 16 bytes whatever their length
-    route = bl.load().bitlogic_internal_hard_route
-    route.argtypes = [ctypes.c_int32, ctypes.c_int64, ctypes.c_int32, ctypes.c_int32]
     for head, per_y in ((1, 128), (0, 384)):
         top = 65535 * per_y
         for w_in in (2, 100):
-            for words, want in [(1, 0), (32, 0), (33, 1), (top - 1, 1), (top, 1), (top + 1, 0), (top + 3, 0)]:
+            for words, want in [(1, 0), (32, 0), (top - 1, 1), (top, 1), (top + 1, 0), (top + 3, 0)]:
                 if w_in * words >= 1 << 32:
                     want = 0
-                assert route(w_in, words, 1, head) == (2 if words % 4 == 0 else want), (head, w_in, words)
-                assert route(w_in, words, 0, head) == want, (head, w_in, words)
-        assert route(1 << 20, 4097, 1, head) == 0 and route(1 << 20, 4095, 1, head) == 1
-        assert route(1 << 20, 4096, 1, head) == 2 and route(1 << 20, 4 << 12, 1, head) == 0
+                assert _hard_route(6, w_in, 64000, words, 1, head) == (2 if words % 4 == 0 else want)
+                assert _hard_route(6, w_in, 64000, words, 0, head) == want, (head, w_in, words)
+        assert _hard_route(6, 1 << 20, 64000, 4097, 1, head) == 0 and _hard_route(6, 1 << 20, 64000, 4095, 1, head) == 1
+        assert _hard_route(6, 1 << 20, 64000, 4096, 1, head) == 2 and _hard_route(6, 1 << 20, 64000, 1 << 14, 1, head) == 0
+
+
+def test_hard_route_of_a_layer_on_other_rows():
+    # measured lines: the one-word kernel up to fan-in 4 unless its warps leave
+    # SMs idle or the input outgrows L2, the staged one for long rows from
+    # fan-in 5 on; aligned rows and the head do not depend on them
+    for k, w_in, w, words, want in [
+            (2, 3000, 64000, 313, 0), (2, 3000, 4000, 1251, 0), (1, 3000, 500, 313, 1), (3, 3000, 1000, 299, 0),
+            (4, 3000, 1000, 219, 1), (4, 3000, 4000, 469, 0), (4, 3000, 2000, 1251, 1), (4, 3000, 4000, 1251, 0),
+            (4, 21504, 16000, 625, 1), (4, 21504, 4000, 625, 0), (5, 3000, 8000, 219, 0), (5, 3000, 8000, 313, 1),
+            (6, 3000, 8000, 157, 0), (6, 3000, 32000, 33, 1), (6, 3000, 31999, 33, 0), (6, 21504, 64000, 313, 1),
+            (6, 3000, 500, 219, 1), (6, 3000, 500, 157, 0), (4, 21504, 2000, 1251, 0), (2, 3000, 700, 10001, 1),
+            (3, 6144, 1000, 2501, 0), (1, 3000, 2000, 10001, 1), (2, 3000, 2000, 10001, 0)]:
+        assert _hard_route(k, w_in, w, words, 1, 0) == want, (k, w_in, w, words)
+        assert _hard_route(k, w_in, w, words + 1 - words % 4 + 4, 0, 1) == 1      # head, any other row
+        assert _hard_route(k, w_in, w, words // 4 * 4, 1, 0) == 2
