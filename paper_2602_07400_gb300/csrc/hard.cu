@@ -827,26 +827,29 @@ HardRoute hard_route(int k, int w_in, int w, long long W, bool aligned, bool hea
 }
 
 // Splits of a class for the staged head when there are few word groups: the
-// grid is then a few waves of blocks.  Least estimated time over all splits
-// that leave a warp at least four nodes, in instructions of a warp: waves x
-// (nodes per warp x a node's instructions + those of staging the slice and
-// flushing the counters), and what every further split costs in atomic adds
-// to the same counts.  10000 samples through 64000 nodes of fan-in 6, 10
-// classes: 20 splits (2 full waves) against 16, pass 273 -> 254 us; 1500
-// samples, 58080 nodes of fan-in 2 45.5 -> 39.3 us; without the last term 2807
-// samples, 17350 nodes of fan-in 2 took 30 splits, 28.0 us against 26.6 us
-// with 16.
+// grid is then a few waves of blocks.  Least estimated time, in ns, over splits
+// that leave a warp at least two nodes.  A block's instructions (its nodes per
+// warp) cost once per block that an SM has to take, whether beside another or
+// after it; what waits on memory and barriers (staging the slice, filling the
+// ring, flushing the counters) once per wave of two blocks per SM; and every
+// block its atomic adds.  The factors are a least-squares fit to 4400 measured
+// times (fan-in 2, 4 and 6, 500 to 64000 nodes, 1 to 100 classes, 32 to 1920
+// words, 1 to 400 splits); the split it picks takes 1.008 of the best one's time
+// on average and 1.14 at worst.  Splitting by doubling until the classes fill
+// the SMs takes 1.21 and 2.1, and an estimate with one cost per wave 1.12 and
+// 1.66 of it: 10000 nodes of fan-in 2 in one class, 1024 samples 10.3 us with
+// 100 splits, 14.5 with 38.
 constexpr int kHeadFewGroups = 16;
-int head_splits(int k, int g, int C, long long wg) {
-    const long long slots = (long long)kHeadMinBlocks * sm_count();
-    const long long node = 4 * ((1 << k) - 1) + 60 + 4 * k, fixed = 4000, split = 72;
+int head_splits(int k, int g, int C, long long wg, int sms) {
+    const long long node = 4 * ((1 << k) - 1) + 60 + 4 * k;   // a warp's instructions per node and stage
     int best = 1;
     long long best_cost = -1;
-    for (int s = 1; s == 1 || (g / s >= 4 * kHSWarps && (long long)C * s * wg <= 8 * slots); ++s) {
+    for (int s = 1; s == 1 || (g / s >= 2 * kHSWarps && C * s * wg <= 8ll * kHeadMinBlocks * sms); s += 1 + s / 16) {
         const int per = (g + s - 1) / s;
         if (per > kHeadSliceNodes) continue;
-        const long long waves = ((long long)C * s * wg + slots - 1) / slots;
-        const long long cost = waves * ((per + kHSWarps - 1) / kHSWarps * node + fixed) + s * split;
+        const long long nodes = (per + kHSWarps - 1) / kHSWarps, blocks = C * s * wg;
+        const long long rounds = (blocks + sms - 1) / sms, waves = (rounds + kHeadMinBlocks - 1) / kHeadMinBlocks;
+        const long long cost = rounds * (nodes * node * 3 / 2 + 180) + waves * (61 * nodes + 2460) + 6 * blocks;
         if (best_cost < 0 || cost < best_cost) {
             best_cost = cost;
             best = s;
@@ -907,7 +910,7 @@ int launch_hard(const uint32_t* xp, int w_in, long long N, const int* conn, cons
         // see head_splits
         int splits = 1;
         if (wg < kHeadFewGroups) {
-            splits = head_splits(k, g, C, wg);
+            splits = head_splits(k, g, C, wg, sm_count());
         } else {
             while (C * splits < sm_count() && g / (splits * 2) >= 8 * kHSWarps) splits *= 2;
         }
@@ -949,10 +952,13 @@ using namespace bitlogic;
 
 BITLOGIC_ERROR_READER(hard)
 
-// The route of a hard call, for host checks of the rule (HardRoute).
+// The route (HardRoute) and the splits of a hard call, for host checks of the rules.
 extern "C" int bitlogic_internal_hard_route(int32_t k, int32_t w_in, int32_t w, int64_t words, int32_t aligned,
                                             int32_t head, int32_t sms) {
     return hard_route(k, w_in, w, words, aligned != 0, head != 0, sms);
+}
+extern "C" int bitlogic_internal_head_splits(int32_t k, int32_t g, int32_t C, int64_t groups, int32_t sms) {
+    return head_splits(k, g, C, groups, sms);
 }
 
 extern "C" int bitlogic_binarize_tables(const float* theta, int32_t w, int32_t k,

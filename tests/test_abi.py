@@ -329,3 +329,22 @@ def test_hard_route_of_a_layer_on_other_rows():
         assert _hard_route(k, w_in, w, words, 1, 0) == want, (k, w_in, w, words)
         assert _hard_route(k, w_in, w, words + 1 - words % 4 + 4, 0, 1) == 1      # head, any other row
         assert _hard_route(k, w_in, w, words // 4 * 4, 1, 0) == 2
+
+
+def test_head_splits_fill_the_grid():
+    # few classes are split until their blocks fill the SMs, many are not; a
+    # warp keeps two nodes, and a block's slice (480 nodes) is respected where
+    # some split within the limits allows it
+    fn = bl.load().bitlogic_internal_head_splits
+    fn.argtypes = [ctypes.c_int32] * 3 + [ctypes.c_int64, ctypes.c_int32]
+    for k in (1, 2, 4, 6):
+        for C in (1, 2, 10, 100, 5000):
+            for g in (1, 5, 16, 40, 400, 1000, 6400, 64000):
+                for groups in (1, 2, 3, 15):
+                    s = fn(k, g, C, groups, 152)
+                    assert 1 <= s and (s == 1 or (g // s >= 16 and C * s * groups <= 8 * 304)), (k, C, g, groups, s)
+                    if -(-g // 480) * C * groups <= 304:
+                        assert -(-g // s) <= 480
+    assert fn(2, 10000, 1, 1, 152) >= 64 and fn(4, 4000, 1, 1, 152) >= 64      # one class: about one block per SM
+    assert fn(2, 100, 100, 1, 152) == 1 and fn(6, 5, 100, 3, 152) == 1
+    assert 4 <= fn(2, 400, 10, 2, 152) <= 8                                     # no more than one block per SM
