@@ -28,13 +28,17 @@ namespace {
 // The loads of 32 rows are in flight together: with few classes and small
 // batches the chain of loads bounds the kernel (a step of 8000 and 20000 nodes
 // of fan-in 2: 63 samples 77.9 -> 65.0 us, 907 samples 231 -> 211 us against
-// four rows; a range check before each load makes it slower than that).
+// four rows; a range check before each load makes it slower than that).  DEEP
+// is for groups of 64 rows and more: below, the registers of the long batch cost
+// more blocks per SM than it gives (100 classes of 10 nodes, 907 samples 8.9 ->
+// 10.0 us).
 // Splitting a class over blocks as below gives 61.4 and 206 us, but adds in
 // another order, and thousands of rows in one chain round by up to 2e-5 of
 // their sum, so the logits would move by as much.
 constexpr int kSumWarps = 8;
 constexpr int kSumRows = 32, kTailRows = 8;
 
+template <bool DEEP>
 __global__ void __launch_bounds__(kSumWarps * 32)
 head_group_sum_kernel(const float* __restrict__ Y, long long B, int C, int g, float tau,
                       float* __restrict__ logits, unsigned int* __restrict__ done) {
@@ -48,21 +52,24 @@ head_group_sum_kernel(const float* __restrict__ Y, long long B, int C, int g, fl
     if (s < B) {
         const float* base = Y + (long long)c * g * B + s;
         int r = warp;
-        for (; r < g - (kSumRows - 1) * kSumWarps; r += kSumRows * kSumWarps) {
-            float v[kSumRows];
+        if constexpr (DEEP) {
+            for (; r < g - (kSumRows - 1) * kSumWarps; r += kSumRows * kSumWarps) {
+                float v[kSumRows];
 #pragma unroll
-            for (int u = 0; u < kSumRows; ++u) v[u] = __ldg(base + (long long)(r + u * kSumWarps) * B);
+                for (int u = 0; u < kSumRows; ++u) v[u] = __ldg(base + (long long)(r + u * kSumWarps) * B);
 #pragma unroll
-            for (int u = 0; u < kSumRows; ++u) acc += v[u];
+                for (int u = 0; u < kSumRows; ++u) acc += v[u];
+            }
+            for (; r < g - (kTailRows - 1) * kSumWarps; r += kTailRows * kSumWarps) {
+                float v[kTailRows];
+#pragma unroll
+                for (int u = 0; u < kTailRows; ++u) v[u] = __ldg(base + (long long)(r + u * kSumWarps) * B);
+#pragma unroll
+                for (int u = 0; u < kTailRows; ++u) acc += v[u];
+            }
         }
-        for (; r < g; r += kTailRows * kSumWarps) {   // loads past the end read the last row again, not added
-            float v[kTailRows];
-#pragma unroll
-            for (int u = 0; u < kTailRows; ++u) v[u] = __ldg(base + (long long)min(r + u * kSumWarps, g - 1) * B);
-#pragma unroll
-            for (int u = 0; u < kTailRows; ++u)
-                if (r + u * kSumWarps < g) acc += v[u];
-        }
+#pragma unroll 4
+        for (; r < g; r += kSumWarps) acc += __ldg(base + (long long)r * B);
     }
     part[warp][lane] = acc;
     __syncthreads();
@@ -341,9 +348,10 @@ extern "C" int bitlogic_head_loss_ex(const float* Y, int32_t w, int64_t B, int32
         (void)launch_dependent(head_group_sum_vec_kernel, dim3((unsigned)(C * splits), (unsigned)nsb),
                                kSumVecWarps * 32, 0, stream, Y, B, C, g, tau, lg, split_sums, splits,
                                rows_per_split, done);
-    } else
-        (void)launch_dependent(head_group_sum_kernel, dim3((unsigned)C, (unsigned)sb), kSumWarps * 32, 0, stream, Y,
-                               B, C, g, tau, lg, done);
+    } else {
+        (void)launch_dependent(g >= 64 ? head_group_sum_kernel<true> : head_group_sum_kernel<false>,
+                               dim3((unsigned)C, (unsigned)sb), kSumWarps * 32, 0, stream, Y, B, C, g, tau, lg, done);
+    }
     if (launch_status()) return BITLOGIC_ERR_CUDA;
     if (launch_dependent(head_softmax_kernel, (unsigned)((B + kSoftWarps - 1) / kSoftWarps), kSoftWarps * 32, 0,
                          stream, lg, B, C, labels, dlogit, block_sums, done, loss, tau,

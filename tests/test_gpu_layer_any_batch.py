@@ -243,3 +243,17 @@ def test_large_inputs_take_the_staged_kernel(k, B, over):
     for a, b in zip(*outs):
         check_exact(a, b, "gradient from rows and from terms")
     assert bl.bitlogic_device_error() == 0
+
+
+@pytest.mark.parametrize("C,g,B", [(100, 10, 907), (10, 63, 130), (10, 64, 31), (7, 1, 5), (10, 120, 67)])
+def test_head_of_short_groups(C, g, B):
+    # both sides of the group size from which long batches of rows are read
+    Y = np.random.default_rng(C + B).random((C * g, B)).astype(np.float32)
+    labels = np.random.default_rng(B).integers(0, C, size=B).astype(np.int32)
+    loss, logits = torch.zeros(1, device="cuda"), torch.full((B, C), np.nan, device="cuda")
+    ws = torch.empty(bl.bitlogic_head_loss_workspace(B, C), dtype=torch.uint8, device="cuda")
+    bl.bitlogic_head_loss(dev(Y), dev(labels), C, 20.0, loss, ws, logits=logits)
+    wl, wloss, _ = oracle.head_loss(Y.astype(np.float64), labels, C, 20.0)
+    check_fwd(logits, wl, "logits")
+    check_fwd(loss, np.array([wloss]), "loss")
+    assert bl.bitlogic_device_error() == 0
