@@ -304,12 +304,13 @@ route_dr_kernel(const T* __restrict__ X, int w_in, long long B, const int* __res
 // slots (75%).
 constexpr int kRdxWarps = 8;
 
-template <bool VEC>
+template <int NG>   // groups of four samples per lane, 0: one sample
 __global__ void __launch_bounds__(kRdxWarps * 32)
 route_dx_kernel(const float* __restrict__ G, long long B, const float* __restrict__ prob, int Kc,
                 const int* __restrict__ off, const int* __restrict__ edge, int w_in, int nE,
                 float* __restrict__ dX) {
-    constexpr int SPW = VEC ? 256 : 32;
+    constexpr bool VEC = NG > 0;
+    constexpr int SPW = VEC ? 128 * NG : 32;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int i = blockIdx.x * kRdxWarps + warp;
     if (i >= w_in) return;
@@ -341,7 +342,7 @@ route_dx_kernel(const float* __restrict__ G, long long B, const float* __restric
         return __any_sync(0xffffffffu, bad);
     };
     if constexpr (VEC) {
-        const bool in0 = s < B, in1 = s + 128 < B;
+        const bool in0 = s < B, in1 = NG > 1 && s + 128 < B;
         float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
         const float* base = G + (in0 ? s : 0);
         const int second = in1 ? 128 : 0;   // lanes out of range read, and drop, the first samples
@@ -355,7 +356,7 @@ route_dx_kernel(const float* __restrict__ G, long long B, const float* __restric
             const bool bad = take(c0);
             const int n = min(32, deg - c0);
             int q = 0;
-            constexpr int kBatch = 4;
+            constexpr int kBatch = 8 / NG;
             if (!bad) {
                 for (; q + kBatch <= n; q += kBatch) {
                     float4 v0[kBatch], v1[kBatch];
@@ -365,12 +366,12 @@ route_dx_kernel(const float* __restrict__ G, long long B, const float* __restric
                         const float* row = base + (long long)__shfl_sync(0xffffffffu, my_slot, q + u) * B;
                         wt[u] = __shfl_sync(0xffffffffu, my_w, q + u);
                         v0[u] = ldg4r(row);
-                        v1[u] = ldg4r(row + second);
+                        if constexpr (NG > 1) v1[u] = ldg4r(row + second);
                     }
 #pragma unroll
                     for (int u = 0; u < kBatch; ++u) {
                         add(a0, wt[u], v0[u]);
-                        add(a1, wt[u], v1[u]);
+                        if constexpr (NG > 1) add(a1, wt[u], v1[u]);
                     }
                 }
             }
@@ -379,9 +380,9 @@ route_dx_kernel(const float* __restrict__ G, long long B, const float* __restric
                 const float w = __shfl_sync(0xffffffffu, my_w, q);
                 if (slot >= 0) {
                     const float* row = base + (long long)slot * B;
-                    const float4 v0 = ldg4r(row), v1 = ldg4r(row + second);
+                    const float4 v0 = ldg4r(row);
+                    if constexpr (NG > 1) add(a1, w, ldg4r(row + second));
                     add(a0, w, v0);
-                    add(a1, w, v1);
                 }
             }
         }
@@ -561,10 +562,11 @@ extern "C" int bitlogic_route_backward(const float* X, int32_t w_in, int64_t B, 
     const long long gy = (B + per_block - 1) / per_block;
     if (gy > 65535) return BITLOGIC_ERR_SHAPE;
     dim3 grid((unsigned)((w_in + kRdxWarps - 1) / kRdxWarps), (unsigned)gy);
-    if (vx)
-        route_dx_kernel<true><<<grid, kRdxWarps * 32, 0, stream>>>(G, B, prob, Kc, csr_off, csr_edge, w_in, nE, dX);
-    else
-        route_dx_kernel<false><<<grid, kRdxWarps * 32, 0, stream>>>(G, B, prob, Kc, csr_off, csr_edge, w_in, nE, dX);
+    // a batch of at most 128 samples fills one group of four per lane: with two,
+    // half of the loads were repeats (32000 slots of 16 candidates, 64 samples,
+    // with the logits' gradient 53.4 us)
+    auto kern = !vx ? route_dx_kernel<0> : B <= 128 ? route_dx_kernel<1> : route_dx_kernel<2>;
+    kern<<<grid, kRdxWarps * 32, 0, stream>>>(G, B, prob, Kc, csr_off, csr_edge, w_in, nE, dX);
     return launch_status();
 }
 

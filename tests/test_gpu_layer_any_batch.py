@@ -257,3 +257,23 @@ def test_head_of_short_groups(C, g, B):
     check_fwd(logits, wl, "logits")
     check_fwd(loss, np.array([wloss]), "loss")
     assert bl.bitlogic_device_error() == 0
+
+
+@pytest.mark.parametrize("B", [4, 60, 124, 128, 132, 256, 260])
+def test_routing_input_gradient_around_its_slices(B):
+    # one group of samples per lane up to 128, two beyond; rows with no, few and
+    # more than 32 readers
+    w_in, slots, Kc = 30, 90, 8
+    X, G = synth.uniform_activations(w_in, B, seed=1), synth.uniform_gradients(slots, B, seed=2, scale=1e-2)
+    cand = synth.candidate_pools(slots, Kc, w_in - 1, seed=3)
+    cand[:50, 0] = 5
+    r = synth.table_logits(slots, Kc, seed=4)
+    off, edge = bl.bitlogic_build_csr(cand, w_in)
+    p, dr = torch.empty(slots, Kc, device="cuda"), torch.empty(slots, Kc, device="cuda")
+    bl.bitlogic_route_forward(dev(X), dev(cand), dev(r), torch.empty(slots, B, device="cuda"), p)
+    dX = torch.full((w_in, B), np.nan, device="cuda")
+    bl.bitlogic_route_backward(dev(X), dev(cand), dev(r), dev(G), dr, p, dev(off), dev(edge), dX)
+    wdr, wdX = oracle.route_backward(X.astype(np.float64), cand, r, G.astype(np.float64))
+    check_grad(dX, wdX, "dX")
+    check_grad(dr, wdr, "dr")
+    assert bl.bitlogic_device_error() == 0
