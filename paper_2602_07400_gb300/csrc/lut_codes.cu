@@ -657,9 +657,10 @@ coded_backward_kernel(const uint8_t* __restrict__ codes, long long stride, const
             }
         };
         // the check in the loop, or a loop of its own for such nodes: 8000 nodes
-        // x 907 samples, step 170 us at fan-in 6 without it, 172.6 and 173.6;
-        // 82.2 at fan-in 4, 83.9 and 81.7
-        if constexpr (k >= 6) stages(std::integral_constant<bool, FORM != kWhole>{});
+        // x 907 samples, step 169.7 us at fan-in 6 without it, 171.9 and 173.7;
+        // 82.2 at fan-in 4, 82.3 and 82.1; 88340 nodes of fan-in 4 x 44 samples
+        // 187.9, 194.7 and 197.9
+        if constexpr (k >= 6 || TAIL) stages(std::integral_constant<bool, FORM != kWhole>{});
         else if (FORM != kWhole && nan) stages(std::true_type{});
         else stages(std::false_type{});
         __syncwarp();
