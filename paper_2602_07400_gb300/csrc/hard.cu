@@ -799,15 +799,15 @@ long long hard_word_chunk(int w_in, long long W) {
 // its time over fan-in 2, 4 and 6, 1 to 100 classes, 500 to 64000 nodes and 33
 // to 625 words (7222 samples, 17760 nodes of fan-in 4: pass 94 -> 58 us).
 //
-// Layer on other rows: the one-word kernel has no copies to issue, and only from
-// fan-in 5 on is the tree long enough to gain from the ring (64000 nodes, 313
-// words: fan-in 2 23.6 us one-word, 29.4 staged; fan-in 6 0.90 of its time;
-// 32000 nodes of fan-in 4, 469 words 28.8, 41.7 us; 21504 input rows of 2501
-// words, fan-in 6 0.56 of its time, fan-in 4 0.9).  It also leaves SMs idle when
-// few nodes run over long rows (500 nodes of fan-in 4, 1251 words: 0.42 of its
-// time staged; 2000: 0.8; fan-in 2, 1600 input rows of 10001 words, 1000 nodes:
-// 0.48).  The lines were drawn from 1000 sizes; over them the rule takes 0.88 of
-// the one-word kernel's time and at worst 1.07 of it.
+// Layer on other rows, timed behind the pack that feeds it (1000 sizes; repeated
+// alone, with its input in L2, the one-word kernel looks better): that kernel
+// has no copies to issue, and up to fan-in 4 the tree is too short to gain from
+// the ring unless its warps, one per node, leave the SMs idle over long rows
+// (3920 input rows of 1285 words: 500 nodes of fan-in 2 0.33 of its time staged,
+// of fan-in 4 0.22, 2000 of fan-in 4 0.48, 20000 of fan-in 2 1.35, of fan-in 4
+// 1.29) or the input outgrows L2.  At fan-in 5 and 6 it loses from about 200
+// words on (6000 nodes: 0.55 and 0.70 of its time; 157 words 0.92 and 0.78).
+// Over all sizes the rule takes 0.83 of its time.
 enum HardRoute { kOneWord = 0, kStaged4 = 1, kStaged16 = 2 };
 constexpr long long kGridY = 65535;
 HardRoute hard_route(int k, int w_in, int w, long long W, bool aligned, bool head, int sms) {
@@ -816,13 +816,11 @@ HardRoute hard_route(int k, int w_in, int w, long long W, bool aligned, bool hea
     const long long per_y = head ? kStageWords : kLayerNS * kStageWords;
     if (W < 33 || rows * (unsigned long long)W >= (1ull << 32) || W > kGridY * per_y) return kOneWord;
     if (head) return kStaged4;
-    const long long chunk = hard_word_chunk(w_in, W), chunks = (W + chunk - 1) / chunk;
-    const long long warps = w * chunks;   // of the one-word kernel
-    bool staged = warps < 8ll * sms && W >= (k >= 4 ? 200 : 300);
-    if (k >= 5) staged = staged || W >= 300 || (k == 6 && w >= 32000);
-    else if (k == 4) staged = staged || (w <= 16ll * sms && W >= 200 && (chunks == 1 || chunk >= 1000)) ||
-                              (chunks > 1 && (long long)w * W >= 8000000);
-    else staged = staged || (chunks > 1 && chunk >= 4000 && warps <= (k == 1 ? 40ll : 20ll) * sms);
+    bool staged;
+    if (k == 6) staged = W >= 150 || w >= 200 * sms;
+    else if (k == 5) staged = W >= 200 || (W >= 100 && w <= 50 * sms);
+    else if (k == 4) staged = (W >= 150 && w <= 20 * sms) || (W >= 600 && hard_word_chunk(w_in, W) < W);
+    else staged = W >= 600 && (w <= 5 * sms || (w_in <= 10000 && w <= (k == 3 ? 8 : 16) * sms));
     return staged ? kStaged4 : kOneWord;
 }
 
