@@ -363,52 +363,52 @@ def call_work(wl, B, fuse_dy1=False, through=False, bytes1=False, bits1=False, c
 # later change of the code reports null.
 TRAFFIC = {
     ("mnist", "forward1"): {
-        "bytes": 2550000 + 0, "source": "lut_codes.cu",
-        "sha256": "cf651a1b8e410a504b6b5737032513981184648aeaf11d067ed55dea35f3123d",
+        "bytes": 2551296 + 0, "source": "lut_codes.cu",
+        "sha256": "1662368f23bfc9fdeeb109f0c978d407ab5d1c4bb3d8e09c78a326f8b2c83aff",
         "note": "ncu capture of this workload (one-pass DRAM metrics)"},
     ("mnist", "forward2"): {
-        "bytes": 12490000 + 0, "source": "lut_codes.cu",
-        "sha256": "cf651a1b8e410a504b6b5737032513981184648aeaf11d067ed55dea35f3123d",
+        "bytes": 12486912 + 0, "source": "lut_codes.cu",
+        "sha256": "1662368f23bfc9fdeeb109f0c978d407ab5d1c4bb3d8e09c78a326f8b2c83aff",
         "note": "ncu capture of this workload (one-pass DRAM metrics)"},
     ("mnist", "backward2"): {
-        "bytes": 12740000 + 0, "source": "lut_codes.cu",
-        "sha256": "cf651a1b8e410a504b6b5737032513981184648aeaf11d067ed55dea35f3123d",
+        "bytes": 12767488 + 0, "source": "lut_codes.cu",
+        "sha256": "1662368f23bfc9fdeeb109f0c978d407ab5d1c4bb3d8e09c78a326f8b2c83aff",
         "note": "ncu capture of this workload (one-pass DRAM metrics)"},
     ("mnist", "backward1"): {
-        "bytes": 14380000 + 0, "source": "lut_codes.cu",
-        "sha256": "cf651a1b8e410a504b6b5737032513981184648aeaf11d067ed55dea35f3123d",
+        "bytes": 14376192 + 0, "source": "lut_codes.cu",
+        "sha256": "1662368f23bfc9fdeeb109f0c978d407ab5d1c4bb3d8e09c78a326f8b2c83aff",
         "note": "ncu capture of this workload (one-pass DRAM metrics)"},
     ("cifar10", "forward1"): {
-        "bytes": 20702464 + 19027968, "source": "lut_codes.cu",
-        "sha256": "cf651a1b8e410a504b6b5737032513981184648aeaf11d067ed55dea35f3123d",
+        "bytes": 20715008 + 18802688, "source": "lut_codes.cu",
+        "sha256": "1662368f23bfc9fdeeb109f0c978d407ab5d1c4bb3d8e09c78a326f8b2c83aff",
         "note": "ncu capture of this workload (one-pass DRAM metrics)"},
     ("cifar10", "forward2"): {
-        "bytes": 253983744 + 221038336, "source": "lut_codes.cu",
-        "sha256": "cf651a1b8e410a504b6b5737032513981184648aeaf11d067ed55dea35f3123d",
+        "bytes": 254218240 + 221047808, "source": "lut_codes.cu",
+        "sha256": "1662368f23bfc9fdeeb109f0c978d407ab5d1c4bb3d8e09c78a326f8b2c83aff",
         "note": "ncu capture of this workload (one-pass DRAM metrics)"},
     ("cifar10", "backward2"): {
-        "bytes": 201024000 + 90138112, "source": "lut_codes.cu",
-        "sha256": "cf651a1b8e410a504b6b5737032513981184648aeaf11d067ed55dea35f3123d",
+        "bytes": 201398528 + 90073344, "source": "lut_codes.cu",
+        "sha256": "1662368f23bfc9fdeeb109f0c978d407ab5d1c4bb3d8e09c78a326f8b2c83aff",
         "note": "ncu capture of this workload (one-pass DRAM metrics)"},
     ("cifar10", "backward1"): {
-        "bytes": 114957312 + 1295360, "source": "lut_codes.cu",
-        "sha256": "cf651a1b8e410a504b6b5737032513981184648aeaf11d067ed55dea35f3123d",
+        "bytes": 114959616 + 857600, "source": "lut_codes.cu",
+        "sha256": "1662368f23bfc9fdeeb109f0c978d407ab5d1c4bb3d8e09c78a326f8b2c83aff",
         "note": "ncu capture of this workload (one-pass DRAM metrics)"},
     ("cifar100", "forward1"): {
-        "bytes": 58401792 + 232305152, "source": "lut_codes.cu",
-        "sha256": "cf651a1b8e410a504b6b5737032513981184648aeaf11d067ed55dea35f3123d",
+        "bytes": 58430208 + 235223296, "source": "lut_codes.cu",
+        "sha256": "1662368f23bfc9fdeeb109f0c978d407ab5d1c4bb3d8e09c78a326f8b2c83aff",
         "note": "ncu capture of this workload (one-pass DRAM metrics)"},
     ("cifar100", "forward2"): {
-        "bytes": 1495481088 + 1011905792, "source": "lut_codes.cu",
-        "sha256": "cf651a1b8e410a504b6b5737032513981184648aeaf11d067ed55dea35f3123d",
+        "bytes": 1495578112 + 1011875072, "source": "lut_codes.cu",
+        "sha256": "1662368f23bfc9fdeeb109f0c978d407ab5d1c4bb3d8e09c78a326f8b2c83aff",
         "note": "ncu capture of this workload (one-pass DRAM metrics)"},
     ("cifar100", "backward2"): {
-        "bytes": 1362891008 + 217948160, "source": "lut_codes.cu",
-        "sha256": "cf651a1b8e410a504b6b5737032513981184648aeaf11d067ed55dea35f3123d",
+        "bytes": 1363090688 + 217728256, "source": "lut_codes.cu",
+        "sha256": "1662368f23bfc9fdeeb109f0c978d407ab5d1c4bb3d8e09c78a326f8b2c83aff",
         "note": "ncu capture of this workload (one-pass DRAM metrics)"},
     ("cifar100", "backward1"): {
-        "bytes": 229904640 + 3043584, "source": "lut_codes.cu",
-        "sha256": "cf651a1b8e410a504b6b5737032513981184648aeaf11d067ed55dea35f3123d",
+        "bytes": 229904384 + 3008256, "source": "lut_codes.cu",
+        "sha256": "1662368f23bfc9fdeeb109f0c978d407ab5d1c4bb3d8e09c78a326f8b2c83aff",
         "note": "ncu capture of this workload (one-pass DRAM metrics)"},
     ("cifar10", "encode"): {
         "bytes": 3160576 + 0, "source": "encode.cu",
@@ -419,8 +419,8 @@ TRAFFIC = {
         "sha256": "e6c29181c8e57f1b0f92ecd6dfdad87e8d79378c78599c3d42e80904a0b689a6",
         "note": "ncu capture of this workload (one-pass DRAM metrics)"},
     ("hard_cifar10", "hard1"): {
-        "bytes": 16 * (1215472128 + 2054902784), "source": "hard.cu",
-        "sha256": "efb0142e8ba2a7811eb3a949d4eb60111d25046ffe9d8b7fec5ab83393f997a8",
+        "bytes": 16 * (1207746048 + 2055009280), "source": "hard.cu",
+        "sha256": "f2f288cccb35a50c3ca43bc6f9686eebd8ec3a5137a900d9068bfa266c434da9",
         "note": "ncu capture at 2^18 samples, scaled x16 to 2^22 by the words processed"},
 }
 
